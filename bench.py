@@ -55,7 +55,9 @@ N_FRAMES, W_FULLHD, H_FULLHD = 64, 1920, 1080
 BYTES_PER_PX = 2 + 16 + 1       # uint16 depth in, float4 normal + uint8 mask out
 KERNEL_SOURCES = ("paper_2209_08241_gb300/csrc/nrm_forward.cu", "paper_2209_08241_gb300/csrc/nrm_forward_param.cu",
                   "paper_2209_08241_gb300/csrc/nrm_forward_kernels.cuh", "paper_2209_08241_gb300/csrc/nrm_device.cuh",
-                  "paper_2209_08241_gb300/csrc/nrm_forward_vec.cuh")
+                  "paper_2209_08241_gb300/csrc/nrm_forward_vec.cuh",
+                  "paper_2209_08241_gb300/csrc/nrm_forward_strip.cuh",
+                  "paper_2209_08241_gb300/csrc/nrm_forward_strip.cu")
 
 # DRAM bytes per launch of the batched kernel from ncu (dram__bytes_read.sum +
 # dram__bytes_write.sum) on the 64 x 1080p uint16 workload, valid only while
@@ -402,8 +404,9 @@ def bench_ours(args, dist: Dist):
     traffic = NCU_TRAFFIC.get(khash)
     roofline = {"bound": "hbm", "achieved": round(achieved, 1), "peak": peak, "unit": "GB/s",
                 "frac": round(achieved / peak, 4), "traffic": traffic,
-                "peak_source": f"{peak_kind} hbm_gbs", "kernel": ("fwd_persistent_param_kernel" if N_FRAMES <= 100 else "fwd_persistent_kernel")
-                + f"<{tile['tile_x']},{tile['tile_y']},{tile['threads']},f32x4>",
+                "peak_source": f"{peak_kind} hbm_gbs",
+                "kernel": "fwd_strip_param_kernel<f32x4>" if tuple(tile.values()) == (128, 16, 256, 3, 0)
+                else f"fwd_persistent_param_kernel<{tile['tile_x']},{tile['tile_y']},{tile['threads']},f32x4>",
                 "kernel_ms_mean": round(kernel_ms, 4), "algorithmic_bytes_per_launch": alg_bytes,
                 "kernel_source_hash": khash}
 

@@ -361,7 +361,10 @@ NRM_API int nrm_sync_status(nrm_handle* h);
  * (128,8,128), (128,16,128), (128,32,512), (128,64,512), (64,16,128),
  * (64,32,256), (64,64,256). threads counts the compute threads; the persistent
  * kernel adds one producer warp. stages in {2, 3, 4} (persistent kernel only);
- * ctas_per_sm 0 = as many as fit. */
+ * ctas_per_sm 0 = as many as fit. With the default geometry (128, 16, 256, 3, 0)
+ * batched calls without point buffers use, for alpha <= 4 and frames whose
+ * width is a multiple of 4 and whose buffers are aligned (as a dense allocation
+ * is), kernels with tile shapes of their own; results are the same bits. */
 typedef struct {
   int tile_x, tile_y, threads, stages, ctas_per_sm;
 } nrm_tile_config;

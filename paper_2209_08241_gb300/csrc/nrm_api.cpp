@@ -218,6 +218,9 @@ int validate_intrinsics(const nrm_intrinsics& K) {
 }
 
 constexpr int kSlots = 3;
+// A handle's geometry unless another is asked for. Batched calls of a handle
+// with this geometry take the strip kernels wherever those apply.
+constexpr nrm_tile_config kDefaultConfig = {128, 16, 256, 3, 0};
 constexpr unsigned long long kDefaultTimeoutNs = 2000000000ull;  // 2 s
 
 struct Slot {
@@ -263,7 +266,7 @@ struct nrm_handle {
   int H = 0, W = 0;
   nrm_intrinsics K = {1, 1, 0, 0};
   nrm_params p;
-  nrm_tile_config cfg = {128, 16, 256, 3, 0};
+  nrm_tile_config cfg = kDefaultConfig;
   const FwdKernelSet* ks = nullptr;
   // Persistent grids [u16]: u16 = 1 for batches of uint16 frames only, whose
   // smaller staging buffers let more CTAs share an SM.
@@ -716,7 +719,7 @@ int nrm_create(const nrm_intrinsics* K, int H, int W, const nrm_params* p, nrm_h
       return cuda_fail(e, "cudaEventCreate");
     }
   }
-  nrm_tile_config c = {128, 16, 256, 3, 0};
+  const nrm_tile_config c = kDefaultConfig;
   rc = configure(h, c);
   if (rc) {
     std::string msg = g_last_error;
@@ -873,6 +876,121 @@ int nrm_estimate_points(nrm_handle* h, const void* depth, void* normals, uint8_t
   return estimate_single(h, depth, normals, valid, points, cuda_stream);
 }
 
+// The frames of a batched forward call, in two parts: those that the strip
+// kernel takes, then the rest, each with its own work list.
+namespace {
+
+struct BatchPart {
+  int first = 0, n = 0;  // descriptors [first, first + n)
+  int tiles = 0;
+  int stat_tiles = 0;    // tiles in the handle's geometry (nrm_stats)
+  int tile_y = 0;
+  bool u16 = true;       // uint16 frames only
+};
+
+// True if the handle's batched calls may take the strip kernels.
+bool strip_handle(const nrm_handle* h) {
+  const nrm_tile_config &c = h->cfg, &d = kDefaultConfig;
+  return c.tile_x == d.tile_x && c.tile_y == d.tile_y && c.threads == d.threads && c.stages == d.stages &&
+         c.ctas_per_sm == d.ctas_per_sm && h->p.alpha <= nrm::kStripMaxAlpha;
+}
+
+// True if the strip kernels can take frame f: whole vectors of four pixels to
+// the right edge, outputs on the alignment of the vector stores, and depth rows
+// that TMA can address (make_desc then decides by encoding the map).
+bool strip_frame(const nrm_handle* h, const nrm_frame& f) {
+  if (!strip_handle(h) || f.points) return false;
+  const uintptr_t na = h->p.out_dtype == NRM_OUT_OCT16 ? 16 : 32;
+  const int eb = f.in_dtype == NRM_IN_U16_MM ? 2 : 4;
+  if (f.in_dtype == NRM_IN_U16_MM) {
+    // The strip kernel leaves out the test q >= FLT_MIN for uint16: with every
+    // depth >= 1 unit, n . ray >= 4 c and so q >= 16 c^2 / |ray|^2.
+    const double a = h->p.alpha, s = h->p.depth_scale;
+    const double c = a * a / (4.0 * f.K.fx * f.K.fy) * s * s;
+    const double u = (std::fabs(f.K.cx) + f.W) / f.K.fx, v = (std::fabs(f.K.cy) + f.H) / f.K.fy;
+    if (!(16.0 * c * c / (1.0 + u * u + v * v) >= 4.0 * 1.17549435e-38)) return false;
+  }
+  return f.W % 4 == 0 && f.out_pitch % 4 == 0 && (uintptr_t)f.normals % na == 0 && (uintptr_t)f.valid % 4 == 0 &&
+         (uintptr_t)f.depth % 16 == 0 && (f.depth_pitch * eb) % 16 == 0;
+}
+
+// Descriptors of the n frames into fd: the strip kernel's from the front, the
+// others from the back. Empty frames are left out.
+void split_batch(const nrm_handle* h, const nrm_frame* frames, int n, FrameDesc* fd, BatchPart (&part)[2]) {
+  const int a = h->p.alpha;
+  part[0].tile_y = nrm::strip_tile_y(h->p.out_dtype);
+  part[1].tile_y = h->cfg.tile_y;
+  int front = 0, back = n;
+  for (int i = 0; i < n; ++i) {
+    const nrm_frame& f = frames[i];
+    if ((long long)f.H * f.W == 0) continue;
+    const int eb = f.in_dtype == NRM_IN_U16_MM ? 2 : 4;
+    bool strip = strip_frame(h, f);
+    if (strip) {
+      make_desc(&fd[front], f.depth, f.normals, f.valid, f.H, f.W, f.depth_pitch, f.out_pitch, f.K, f.in_dtype, h->p,
+                nrm::kStripX, part[0].tile_y, nrm::kStripX + 2 * nrm::pad_x(a, eb), part[0].tile_y + 2 * a);
+      strip = fd[front].use_tma != 0;
+    }
+    FrameDesc* d = strip ? &fd[front++] : &fd[--back];
+    if (!strip)
+      make_desc(d, f.depth, f.normals, f.valid, f.H, f.W, f.depth_pitch, f.out_pitch, f.K, f.in_dtype, h->p,
+                h->cfg.tile_x, h->cfg.tile_y, h->cfg.tile_x + 2 * nrm::pad_x(a, eb), h->cfg.tile_y + 2 * a);
+    BatchPart& p = part[strip ? 0 : 1];
+    p.u16 = p.u16 && f.in_dtype == NRM_IN_U16_MM;
+    p.tiles += d->tiles_x * ((f.H + p.tile_y - 1) / p.tile_y);
+    p.stat_tiles += ((f.W + h->cfg.tile_x - 1) / h->cfg.tile_x) * ((f.H + h->cfg.tile_y - 1) / h->cfg.tile_y);
+    ++p.n;
+  }
+  part[0].first = 0;
+  part[1].first = back;
+}
+
+// One part's header and tile offsets (tile_begin: n + 1 entries).
+void fill_work_list(const BatchPart& p, FrameDesc* fd, nrm::BatchHeader* hdr, int* tile_begin) {
+  std::memset(hdr, 0, sizeof(*hdr));
+  hdr->n_frames = p.n;
+  hdr->total_tiles = p.tiles;
+  int acc = 0;
+  for (int i = 0; i < p.n; ++i) {
+    FrameDesc& d = fd[p.first + i];
+    d.tile_begin = acc;
+    tile_begin[i] = acc;
+    acc += d.tiles_x * ((d.H + p.tile_y - 1) / p.tile_y);
+  }
+  tile_begin[p.n] = acc;
+}
+
+// Launches one part: its descriptors as the kernel parameter (param_block) or
+// in the device block that args points to.
+int launch_part(nrm_handle* h, bool strip, const nrm::BatchArgs& args, const BatchPart& p, void* param_block,
+                cudaStream_t st) {
+  nrm::Globals g = make_globals(h);
+  if (strip) {
+    NRM_CUDA(nrm::launch_forward_strip(args, g, h->p.out_dtype, p.tiles, p.u16, st, param_block),
+             "launch strip kernel");
+    return NRM_OK;
+  }
+  const int TX = h->cfg.tile_x, TY = h->cfg.tile_y;
+  nrm::BatchArgs a = args;
+  a.stages = h->cfg.stages;
+  a.stage_bytes = nrm::stage_bytes_for(TX, TY, h->p.alpha, p.u16 ? 2 : 0);
+  const unsigned smem = nrm::persistent_smem_bytes(TX, TY, h->p.alpha, h->cfg.stages, p.u16 ? 2 : 0);
+  const dim3 block(nrm::persistent_threads(h->cfg.threads));
+  if (param_block) {
+    void* pargs[3] = {param_block, &a, &g};
+    NRM_CUDA(cudaLaunchKernel(h->param_persistent, dim3(h->persistent_grid_param[p.u16]), block, pargs, smem, st),
+             "launch fwd_persistent_param_kernel");
+  } else {
+    void* kargs[2] = {&a, &g};
+    NRM_CUDA(cudaLaunchKernel(h->ks->persistent[h->p.out_dtype], dim3(h->persistent_grid[p.u16]), block, kargs, smem,
+                              st),
+             "launch fwd_persistent_kernel");
+  }
+  return NRM_OK;
+}
+
+}  // namespace
+
 // nrm_estimate_batched with the descriptor block as one kernel parameter
 // (frame records and tensor maps in parameter space): no descriptor upload and
 // no tensor-map fences. Used for batches of at most kParamMaxFrames frames
@@ -882,42 +1000,15 @@ int nrm_estimate_points(nrm_handle* h, const void* depth, void* normals, uint8_t
 static int estimate_batched_param(nrm_handle* h, const nrm_frame* frames, int n, cudaStream_t st, bool capture) {
   if (n > nrm::kParamMaxFrames)
     return fail(NRM_ERR_UNSUPPORTED, "at most %d frames per call during stream capture", nrm::kParamMaxFrames);
-  const int TX = h->cfg.tile_x, TY = h->cfg.tile_y;
+  for (int i = 0; i < n; ++i)
+    if (frames[i].points && (long long)frames[i].H * frames[i].W > 0)
+      return fail(NRM_ERR_UNSUPPORTED, "frame %d: point clouds are not written during stream capture", i);
   std::vector<FrameDesc>& fd = h->scratch_desc;
   std::vector<int>& tb = h->scratch_tb;
   if (fd.size() < (size_t)n) fd.resize((size_t)n);
-  if (tb.size() < (size_t)n + 1) tb.resize((size_t)n + 1);
-  bool u16 = true;
-  int acc = 0;
-  for (int i = 0; i < n; ++i) {
-    const nrm_frame& f = frames[i];
-    if (f.points && (long long)f.H * f.W > 0)
-      return fail(NRM_ERR_UNSUPPORTED, "frame %d: point clouds are not written during stream capture", i);
-    u16 = u16 && (f.in_dtype == NRM_IN_U16_MM || (long long)f.H * f.W == 0);
-    const int eb = f.in_dtype == NRM_IN_U16_MM ? 2 : 4;
-    make_desc(&fd[i], f.depth, f.normals, f.valid, f.H, f.W, f.depth_pitch, f.out_pitch, f.K, f.in_dtype, h->p,
-              TX, TY, TX + 2 * nrm::pad_x(h->p.alpha, eb), TY + 2 * h->p.alpha);
-    fd[i].tile_begin = acc;
-    tb[i] = acc;
-    acc += fd[i].tiles_x * ((f.H + TY - 1) / TY);
-  }
-  tb[n] = acc;
-  nrm::BatchHeader hdr;
-  std::memset(&hdr, 0, sizeof(hdr));
-  hdr.n_frames = n;
-  hdr.total_tiles = acc;
-  // The parameter block, 128-byte aligned like the records in it.
-  std::vector<unsigned char>& raw = h->scratch_param;
-  if (raw.size() < nrm::param_batch_bytes() + 128) raw.resize(nrm::param_batch_bytes() + 128);
-  void* pb = raw.data() + (128 - reinterpret_cast<uintptr_t>(raw.data()) % 128) % 128;
-  nrm::pack_param_batch(pb, hdr, tb.data(), fd.data(), n);
-  nrm::BatchArgs ring;
-  std::memset(&ring, 0, sizeof(ring));
-  ring.stages = h->cfg.stages;
-  ring.stage_bytes = nrm::stage_bytes_for(TX, TY, h->p.alpha, u16 ? 2 : 0);
-  nrm::Globals g = make_globals(h);
-  void* args[3] = {pb, &ring, &g};
-  const unsigned smem = nrm::persistent_smem_bytes(TX, TY, h->p.alpha, h->cfg.stages, u16 ? 2 : 0);
+  if (tb.size() < (size_t)n + 2) tb.resize((size_t)n + 2);
+  BatchPart part[2];  // strip kernel, tiled kernel
+  split_batch(h, frames, n, fd.data(), part);
   Slot* s = nullptr;
   if (!capture) {
     // A ring slot supplies the completion (and, with timing on, the kernel
@@ -927,16 +1018,59 @@ static int estimate_batched_param(nrm_handle* h, const nrm_frame* frames, int n,
     NRM_CHECK(retire_slot(h, *s));
     if (h->timing) NRM_CUDA(cudaEventRecord(s->ev_start, st), "cudaEventRecord");
   }
-  NRM_CUDA(cudaLaunchKernel(h->param_persistent, dim3(h->persistent_grid_param[u16]),
-                            dim3(nrm::persistent_threads(h->cfg.threads)), args, smem, st),
-           "launch fwd_persistent_param_kernel");
+  // The parameter block, 128-byte aligned like the records in it.
+  std::vector<unsigned char>& raw = h->scratch_param;
+  if (raw.size() < nrm::param_batch_bytes() + 128) raw.resize(nrm::param_batch_bytes() + 128);
+  void* pb = raw.data() + (128 - reinterpret_cast<uintptr_t>(raw.data()) % 128) % 128;
+  for (int k = 0; k < 2; ++k) {
+    if (part[k].tiles == 0) continue;
+    nrm::BatchHeader hdr;
+    fill_work_list(part[k], fd.data(), &hdr, tb.data());
+    nrm::pack_param_batch(pb, hdr, tb.data(), fd.data() + part[k].first, part[k].n);
+    nrm::BatchArgs ring;
+    std::memset(&ring, 0, sizeof(ring));
+    NRM_CHECK(launch_part(h, k == 0, ring, part[k], pb, st));
+  }
   if (s) {
     if (h->timing) NRM_CUDA(cudaEventRecord(s->ev_end, st), "cudaEventRecord");
     NRM_CUDA(cudaEventRecord(s->done, st), "cudaEventRecord");
     s->in_flight = true;
     s->timed_launch = h->timing;
-    s->tiles = acc;
+    s->tiles = part[0].stat_tiles + part[1].stat_tiles;
   }
+  return NRM_OK;
+}
+
+// A batch of more than kParamMaxFrames frames of which the strip kernel may take
+// some: one upload of the descriptors into slot s (retired, with capacity n),
+// then a launch per part.
+static int estimate_batched_ring(nrm_handle* h, const nrm_frame* frames, int n, Slot& s, cudaStream_t st) {
+  char* base = static_cast<char*>(s.host);
+  FrameDesc* fd = reinterpret_cast<FrameDesc*>(base + nrm::frames_offset(s.capacity));
+  BatchPart part[2];
+  split_batch(h, frames, n, fd, part);
+  const size_t off[2] = {0, nrm::second_header_offset(part[0].n)};
+  for (int k = 0; k < 2; ++k)
+    fill_work_list(part[k], fd, reinterpret_cast<nrm::BatchHeader*>(base + off[k]),
+                   reinterpret_cast<int*>(base + off[k] + nrm::kTileBeginOffset));
+  const size_t used = nrm::frames_offset(s.capacity) + sizeof(FrameDesc) * (size_t)n;
+  NRM_CUDA(cudaMemcpyAsync(s.dev, s.host, used, cudaMemcpyHostToDevice, st), "cudaMemcpyAsync");
+  if (h->timing) NRM_CUDA(cudaEventRecord(s.ev_start, st), "cudaEventRecord");
+  char* dbase = static_cast<char*>(s.dev);
+  for (int k = 0; k < 2; ++k) {
+    if (part[k].tiles == 0) continue;
+    nrm::BatchArgs args;
+    std::memset(&args, 0, sizeof(args));
+    args.hdr = reinterpret_cast<const nrm::BatchHeader*>(dbase + off[k]);
+    args.tile_begin = reinterpret_cast<const int*>(dbase + off[k] + nrm::kTileBeginOffset);
+    args.frames = reinterpret_cast<const FrameDesc*>(dbase + nrm::frames_offset(s.capacity)) + part[k].first;
+    NRM_CHECK(launch_part(h, k == 0, args, part[k], nullptr, st));
+  }
+  if (h->timing) NRM_CUDA(cudaEventRecord(s.ev_end, st), "cudaEventRecord");
+  NRM_CUDA(cudaEventRecord(s.done, st), "cudaEventRecord");
+  s.in_flight = true;
+  s.timed_launch = h->timing;
+  s.tiles = part[0].stat_tiles + part[1].stat_tiles;
   return NRM_OK;
 }
 
@@ -970,6 +1104,8 @@ int nrm_estimate_batched(nrm_handle* h, const nrm_frame* frames, int n, void* cu
   if (rc) return rc;
   rc = ensure_slot_capacity(h, s, n);
   if (rc) return rc;
+  if (!any_points && strip_handle(h))
+    return estimate_batched_ring(h, frames, n, s, st0);
   // Fill the pinned staging block.
   char* base = static_cast<char*>(s.host);
   nrm::BatchHeader* hdr = reinterpret_cast<nrm::BatchHeader*>(base);
@@ -1727,7 +1863,7 @@ int nrm_autotune(nrm_handle* h, const nrm_frame* frames, int n, void* cuda_strea
   // Candidates: every compiled tile shape x pipeline depth x CTAs per SM from
   // 2 up to the occupancy limit (fewer concurrent CTAs can write to HBM
   // faster, so the limit is not always best).
-  std::vector<nrm_tile_config> cands;
+  std::vector<nrm_tile_config> cands = {kDefaultConfig};  // the strip kernels, where they apply
   for (int i = 0; i < nrm::fwd_kernel_count(); ++i) {
     const FwdKernelSet* k = nrm::fwd_kernel(i);
     for (int stages = 2; stages <= 4; ++stages) {

@@ -1,0 +1,411 @@
+// The strip kernels: batched forward pass (arXiv 2209.08241, Section 3.1
+// Eq. 4-6 and the Section 3.2 mask) for frames whose rows TMA can load and
+// whose outputs take whole-vector stores, for pixel distance ALPHA = 1..4.
+//
+// One CTA is strip_warps compute warps and a producer warp. The producer walks
+// the CTA's tiles (128 x strip_tile_y pixels) of the batch's work list and, per
+// tile, issues one TMA box of raw depth into an S-stage ring and writes the
+// tile's record, its column table and its row table next to it. A compute warp
+// takes a band of strip_rows rows, four consecutive columns per lane, and walks
+// down the band in steps of ALPHA rows, so that a row's four depths are
+// converted to float once and serve as lower, centre and upper neighbour in
+// turn from registers; only the left and right neighbours are read a second
+// time. No decoded copy of the tile is kept in shared memory and no barrier
+// joins the warps of a CTA: a warp waits for its stage's TMA copy and frees the
+// stage when it is done with it. Thread instructions per pixel (uint16 input,
+// alpha 2): half4 33 (the tiled kernel's vector loop: 51), octahedral 40 (50).
+//
+// Invalid depths are found per pixel from the smallest of the five depths
+// (three-operand minimum, NaN propagating) instead of coding each of them as
+// NaN: uint16 0 and float32 values <= 0 fail "> 0"; float32 infinities become
+// NaN when they are loaded (0 x inf + inf) and then fail the minimum as NaNs do. For
+// valid pixels every operation is that of emit_pair (nrm_device.cuh), in its
+// order, so both give the same bits. (uint16 frames come here only if q >= FLT_MIN
+// holds for every valid pixel, so that test is left out for them.)
+#pragma once
+
+#include "nrm_forward_kernels.cuh"
+
+namespace nrm {
+
+using namespace dev;
+
+// Per-stage record of the producer.
+struct alignas(16) StripInfo {
+  float a, b, c;  // Eq. 4-6 constants with the sign folded in
+  int u16;
+  unsigned char* normals;  // of the tile's first pixel
+  uint8_t* valid;
+  long long out_pitch;
+  int cols, rows;  // pixels of the tile inside the frame
+#ifdef NRM_DEBUG_CHECKS
+  const void *normals0, *valid0;  // the frame's outputs and their extents
+  long long nlen, mlen;
+#endif
+};
+constexpr unsigned kStripInfoBytes = 128;
+static_assert(sizeof(StripInfo) <= kStripInfoBytes, "StripInfo must fit its slot");
+
+// Shared memory of a stage: raw depth box, record, column table (two float4
+// per lane), row table.
+NRM_HD constexpr unsigned strip_table_bytes(int out_dtype) {
+  return (kStripInfoBytes + (kStripX / 2 + strip_tile_y(out_dtype)) * 16u + 127) / 128 * 128;
+}
+NRM_HD inline unsigned strip_stage_bytes(int out_dtype, int alpha, int eb) {
+  return stage_bytes_for(kStripX, strip_tile_y(out_dtype), alpha, eb) + strip_table_bytes(out_dtype);
+}
+NRM_HD inline unsigned strip_smem_bytes(int out_dtype, int alpha, int eb, int stages) {
+  return (strip_stage_bytes(out_dtype, alpha, eb) + 16) * stages;
+}
+
+__device__ __forceinline__ float min3_nan(float a, float b, float c) {
+  float d;
+  asm("min.NaN.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+  return d;
+}
+
+// 32-byte streaming store (the address is a multiple of 32): every store writes
+// whole 32-byte sectors although a lane's four float4 normals are 64 bytes apart
+// from the next lane's.
+__device__ __forceinline__ void store32(void* p, uint32_t a, uint32_t b, uint32_t c, uint32_t d, uint32_t e,
+                                        uint32_t f, uint32_t g, uint32_t h) {
+  asm volatile("st.global.cs.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(a), "r"(b), "r"(c),
+               "r"(d), "r"(e), "r"(f), "r"(g), "r"(h)
+               : "memory");
+}
+
+// Two raw depths as floats. uint16: 0x4B00uuuu is the float 2^23 + u, and
+// subtracting 2^23 is exact (0 stays 0). float32: 0 x d + d is d for finite d
+// and NaN for infinities.
+__device__ __forceinline__ float2 depth_pair(uint32_t w) {
+  const float2 k = f2(-8388608.0f, -8388608.0f);
+  return __fadd2_rn(f2(__uint_as_float(__byte_perm(w, 0x4B000000u, 0x7410)),
+                       __uint_as_float(__byte_perm(w, 0x4B000000u, 0x7432))), k);
+}
+__device__ __forceinline__ float2 depth_pair(float2 d) { return __ffma2_rn(d, f2(0.0f, 0.0f), d); }
+
+// The lane's four depths of a staged row.
+__device__ __forceinline__ void load_run(const uint16_t* p, float2& a, float2& b) {
+  const uint2 w = NRM_LDS(uint2, reinterpret_cast<const uint2*>(p));
+  a = depth_pair(w.x);
+  b = depth_pair(w.y);
+}
+__device__ __forceinline__ void load_run(const float* p, float2& a, float2& b) {
+  const float4 w = NRM_LDS(float4, reinterpret_cast<const float4*>(p));
+  a = depth_pair(f2(w.x, w.y));
+  b = depth_pair(f2(w.z, w.w));
+}
+__device__ __forceinline__ float2 load_two(const uint16_t* p) {
+  return depth_pair(NRM_LDS(uint32_t, reinterpret_cast<const uint32_t*>(p)));
+}
+__device__ __forceinline__ float2 load_two(const float* p) {
+  return depth_pair(NRM_LDS(float2, reinterpret_cast<const float2*>(p)));
+}
+
+// One pixel pair: the closed form, the statistic and the mask decision, in the
+// operation order of QuadStencil and emit_pair.
+template <bool SECANT, bool U16>
+__device__ __forceinline__ void strip_pair(float2 d1, float2 d2, float2 d3, float2 d4, float2 d5, float2 A, float2 B,
+                                           float2 C, float2 T, float tau2, float2 nu1, float2 ku, float2 nv1,
+                                           float2 kv, float2& nx, float2& ny, float2& nz, float2& q, bool& ka,
+                                           bool& kb) {
+  const float kFltMin = 1.17549435e-38f;
+  const float2 M1 = f2(-1.0f, -1.0f);
+  const float2 S24 = __fadd2_rn(d2, d4), D24 = __ffma2_rn(M1, d4, d2);
+  const float2 S35 = __fadd2_rn(d3, d5), D35 = __ffma2_rn(M1, d5, d3);
+  nx = __fmul2_rn(__fmul2_rn(A, S35), D24);
+  ny = __fmul2_rn(__fmul2_rn(B, S24), D35);
+  const float2 P = __fmul2_rn(__fmul2_rn(C, S24), S35);
+  nz = __ffma2_rn(nu1, nx, __ffma2_rn(nv1, ny, P));
+  q = __ffma2_rn(nx, nx, __ffma2_rn(ny, ny, __fmul2_rn(nz, nz)));
+  ka = min3_nan(min3_nan(d1.x, d2.x, d3.x), d4.x, d5.x) > 0.0f;
+  kb = min3_nan(min3_nan(d1.y, d2.y, d3.y), d4.y, d5.y) > 0.0f;
+  if (!U16) {
+    ka = ka & (q.x >= kFltMin);
+    kb = kb & (q.y >= kFltMin);
+  }
+  if (SECANT) {
+    const float2 lhs = __fmul2_rn(q, __fadd2_rn(ku, kv));
+    const float2 rhs = __fmul2_rn(T, __fmul2_rn(P, P));
+    ka = ka & (lhs.x <= rhs.x);
+    kb = kb & (lhs.y <= rhs.y);
+  } else {
+    ka = ka & (q.x <= tau2);
+    kb = kb & (q.y <= tau2);
+  }
+}
+
+// The octahedral codes of a pixel pair (oct16_code, operation for operation,
+// with the additions, the scale and the rounding steps paired).
+__device__ __forceinline__ void strip_codes(float2 nx, float2 ny, float2 nz, uint32_t& ca, uint32_t& cb) {
+  const float2 r = f2(rcp_ftz(fabsf(nx.x) + fabsf(ny.x) + fabsf(nz.x)), rcp_ftz(fabsf(nx.y) + fabsf(ny.y) + fabsf(nz.y)));
+  const float2 s = __fmul2_rn(f2(32767.0f, 32767.0f), r);
+  const float2 m = f2(fmaxf(-nz.x, 0.0f), fmaxf(-nz.y, 0.0f));
+  const float2 tx = __fadd2_rn(nx, f2(copysignf(m.x, nx.x), copysignf(m.y, nx.y)));
+  const float2 ty = __fadd2_rn(ny, f2(copysignf(m.x, ny.x), copysignf(m.y, ny.y)));
+  const float2 k = f2(12582912.0f, 12582912.0f);  // 1.5 * 2^23
+  const float2 x = __ffma2_rn(tx, s, k), y = __ffma2_rn(ty, s, k);
+  ca = __byte_perm(__float_as_uint(x.x), __float_as_uint(y.x), 0x5410);
+  cb = __byte_perm(__float_as_uint(x.y), __float_as_uint(y.y), 0x5410);
+}
+
+// One band: strip_rows(OUT) rows of 128 columns from the staged box S (its first
+// row is ALPHA above the band's, its column PAD the tile's first).
+template <int OUT, bool SECANT, int ALPHA, typename InT>
+__device__ __forceinline__ void strip_band(const InT* __restrict__ S, const float4* __restrict__ ctab,
+                                           const float4* __restrict__ rtab, const StripInfo& f, int band, float tau2) {
+  constexpr int EB = (int)sizeof(InT);
+  constexpr int PAD = EB == 2 ? 8 : 4;        // pad_x(ALPHA, EB) for ALPHA <= 4
+  constexpr int SP = kStripX + 2 * PAD;       // staged row pitch
+  constexpr int BPP = OUT == NRM_OUT_F32X4 ? 16 : OUT == NRM_OUT_F16X4 ? 8 : 4;
+  constexpr int ROWS = strip_rows(OUT);
+  constexpr int STEPS = (ROWS + ALPHA - 1) / ALPHA;
+  const int lane = threadIdx.x & 31;
+  const float4 c0 = NRM_LDS(float4, ctab + 2 * lane), c1 = NRM_LDS(float4, ctab + 2 * lane + 1);
+  const float2 nu1[2] = {f2(c0.x, c0.y), f2(c1.x, c1.y)};
+  const float2 ku[2] = {f2(c0.z, c0.w), f2(c1.z, c1.w)};
+  const float2 A = f2(f.a, f.a), B = f2(f.b, f.b), C = f2(f.c, f.c), T = f2(tau2, tau2);
+  const int row0 = band * ROWS;
+  const int rows = min(ROWS, f.rows - row0);
+  const bool on = 4 * lane < f.cols;
+  const InT* base = S + row0 * SP + PAD + 4 * lane;
+#pragma unroll 1
+  for (int c = 0; c < ALPHA; ++c) {
+    if (c >= rows) break;
+    const InT* p = base + c * SP;  // staged row of the pixels ALPHA above row c
+    float2 u0, u1, m0, m1;
+    load_run(p, u0, u1);
+    load_run(p + ALPHA * SP, m0, m1);
+    unsigned char* np = f.normals + ((long long)(row0 + c) * f.out_pitch + 4 * lane) * BPP;
+    uint8_t* mp = f.valid + (long long)(row0 + c) * f.out_pitch + 4 * lane;
+#pragma unroll
+    for (int k = 0; k < STEPS; ++k) {
+      const int r = c + k * ALPHA;
+      if (r >= rows) break;
+      float2 b0, b1;
+      load_run(p + (k + 2) * ALPHA * SP, b0, b1);
+      const InT* pc = p + (k + 1) * ALPHA * SP;
+      float2 l0, l1, r0, r1;  // left and right neighbours of the two pairs
+      if (ALPHA == 1) {
+        const float2 l = load_two(pc - 2), e = load_two(pc + 4);
+        l0 = f2(l.y, m0.x);
+        r0 = l1 = f2(m0.y, m1.x);
+        r1 = f2(m1.y, e.x);
+      } else if (ALPHA == 2) {
+        l0 = load_two(pc - 2);
+        l1 = m0;
+        r0 = m1;
+        r1 = load_two(pc + 4);
+      } else {
+        float2 la, lb, ra, rb;  // columns -4..-1 and 4..7
+        load_run(pc - 4, la, lb);
+        load_run(pc + 4, ra, rb);
+        l0 = ALPHA == 4 ? la : f2(la.y, lb.x);
+        l1 = ALPHA == 4 ? lb : f2(lb.y, m0.x);
+        r0 = ALPHA == 4 ? ra : f2(m1.y, ra.x);
+        r1 = ALPHA == 4 ? rb : f2(ra.y, rb.x);
+      }
+      const float4 rr = NRM_LDS(float4, rtab + row0 + r);
+      const float2 nv1 = f2(rr.x, rr.y), kv = f2(rr.z, rr.w);
+      float2 nx[2], ny[2], nz[2], q[2];
+      bool k0, k1, k2, k3;
+      strip_pair<SECANT, EB == 2>(m0, r0, b0, l0, u0, A, B, C, T, tau2, nu1[0], ku[0], nv1, kv, nx[0], ny[0], nz[0],
+                                  q[0], k0, k1);
+      strip_pair<SECANT, EB == 2>(m1, r1, b1, l1, u1, A, B, C, T, tau2, nu1[1], ku[1], nv1, kv, nx[1], ny[1], nz[1],
+                                  q[1], k2, k3);
+      const uint32_t mbits = (k0 ? 1u : 0u) | (k1 ? 0x100u : 0u) | (k2 ? 0x10000u : 0u) | (k3 ? 0x1000000u : 0u);
+      uint32_t w[4 * BPP / 4];
+      if constexpr (OUT == NRM_OUT_OCT16) {
+        strip_codes(nx[0], ny[0], nz[0], w[0], w[1]);
+        strip_codes(nx[1], ny[1], nz[1], w[2], w[3]);
+        w[0] = k0 ? w[0] : 0u;
+        w[1] = k1 ? w[1] : 0u;
+        w[2] = k2 ? w[2] : 0u;
+        w[3] = k3 ? w[3] : 0u;
+      } else {
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+          const bool ka = j ? k2 : k0, kb = j ? k3 : k1;
+          const float2 inv = f2(rsqrt_ftz(q[j].x), rsqrt_ftz(q[j].y));
+          const float2 ox = __fmul2_rn(nx[j], inv), oy = __fmul2_rn(ny[j], inv), oz = __fmul2_rn(nz[j], inv);
+          if constexpr (OUT == NRM_OUT_F16X4) {
+            w[4 * j] = ka ? h2_bits(__floats2half2_rn(ox.x, oy.x)) : 0u;
+            w[4 * j + 1] = ka ? h2_bits(__floats2half2_rn(oz.x, 0.0f)) : 0u;
+            w[4 * j + 2] = kb ? h2_bits(__floats2half2_rn(ox.y, oy.y)) : 0u;
+            w[4 * j + 3] = kb ? h2_bits(__floats2half2_rn(oz.y, 0.0f)) : 0u;
+          } else {
+            w[8 * j] = __float_as_uint(ka ? ox.x : 0.0f);
+            w[8 * j + 1] = __float_as_uint(ka ? oy.x : 0.0f);
+            w[8 * j + 2] = __float_as_uint(ka ? oz.x : 0.0f);
+            w[8 * j + 3] = 0u;
+            w[8 * j + 4] = __float_as_uint(kb ? ox.y : 0.0f);
+            w[8 * j + 5] = __float_as_uint(kb ? oy.y : 0.0f);
+            w[8 * j + 6] = __float_as_uint(kb ? oz.y : 0.0f);
+            w[8 * j + 7] = 0u;
+          }
+        }
+      }
+#ifdef NRM_DEBUG_CHECKS
+      if (on && !(dbg_gmem_ok(np, 4 * BPP, f.normals0, f.nlen, "strip normals", __LINE__) &&
+                  dbg_gmem_ok(mp, 4, f.valid0, f.mlen, "strip mask", __LINE__)))
+        break;
+#endif
+      if (on) {
+        if constexpr (OUT == NRM_OUT_F32X4) {
+          store32(np, w[0], w[1], w[2], w[3], w[4], w[5], w[6], w[7]);
+          store32(np + 32, w[8], w[9], w[10], w[11], w[12], w[13], w[14], w[15]);
+        } else if constexpr (OUT == NRM_OUT_F16X4) {
+          store32(np, w[0], w[1], w[2], w[3], w[4], w[5], w[6], w[7]);
+        } else {
+          __stcs(reinterpret_cast<uint4*>(np), make_uint4(w[0], w[1], w[2], w[3]));
+        }
+        __stcs(reinterpret_cast<unsigned int*>(mp), mbits);
+      }
+      np += ALPHA * f.out_pitch * BPP;
+      mp += ALPHA * f.out_pitch;
+      u0 = m0;
+      u1 = m1;
+      m0 = b0;
+      m1 = b1;
+    }
+  }
+}
+
+template <int OUT, bool SECANT, int ALPHA, bool RING>
+__device__ __forceinline__ void strip_pipeline(const BatchArgs& args, const Globals& g) {
+  extern __shared__ __align__(128) unsigned char smem[];
+  constexpr int BPP = OUT == NRM_OUT_F32X4 ? 16 : OUT == NRM_OUT_F16X4 ? 8 : 4;
+  const int S = args.stages;
+  const unsigned SB = args.stage_bytes;
+  constexpr int WARPS = strip_warps(OUT), TY = strip_tile_y(OUT);
+  constexpr unsigned TB = strip_table_bytes(OUT);
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + (size_t)S * SB);
+  uint64_t* empty = full + S;
+  const int total = args.hdr->total_tiles;
+  const int nf = args.hdr->n_frames;
+  const int G = (int)gridDim.x;
+  const int my = (int)blockIdx.x < total ? (total - 1 - (int)blockIdx.x) / G + 1 : 0;
+  if (my == 0) return;
+  NRM_DEBUG_ENTRY(g.status);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < S; ++s) {
+      mbar_init(smem_u32(&full[s]), 2);
+      mbar_init(smem_u32(&empty[s]), WARPS);
+    }
+    fence_barrier_init();
+  }
+  __syncthreads();
+
+  if (warp == WARPS) {
+    // ------------------------------------------------------------ producer
+    int cur = 0, fenced = -1, s = 0;
+    uint32_t parity = 1;
+    for (int j = 0; j < my; ++j) {
+      if (j >= S && !mbar_wait_warp(smem_u32(&empty[s]), parity, g.timeout_ns)) {
+        if (lane == 0) {
+          record_error(g.status, NRM_ERR_TIMEOUT);
+          for (int k = j - S; k < j; ++k)
+            mbar_wait_bounded(smem_u32(&full[k % S]), (uint32_t)((k / S) & 1), g.timeout_ns);
+        }
+        return;
+      }
+      const int t = (int)blockIdx.x + j * G;
+      while (cur + 1 < nf && load_index<RING>(args.tile_begin + cur + 1) <= t) ++cur;
+      const FrameDesc* fd = args.frames + cur;
+      const int local = t - load_index<RING>(args.tile_begin + cur);
+      const int tiles_x = fd->tiles_x;
+      const int ty = local / tiles_x;
+      const int gx0 = (local - ty * tiles_x) * kStripX, gy0 = ty * TY;
+      const int eb = fd->in_dtype == NRM_IN_U16_MM ? 2 : 4;
+      unsigned char* st = smem + (size_t)s * SB;
+      if (lane == 0) {
+        if (RING && cur != fenced) {
+          fence_tensormap_acquire(&fd->tmap);
+          fenced = cur;
+        }
+        const int padx = pad_x(ALPHA, eb);
+        const uint32_t bar = smem_u32(&full[s]);
+        mbar_arrive_expect_tx(bar, (uint32_t)((kStripX + 2 * padx) * (TY + 2 * ALPHA) * eb));
+        tma_load_2d(smem_u32(st), &fd->tmap, gx0 - padx, gy0 - ALPHA, bar);
+        StripInfo si;
+        si.a = -g.sign * fd->a;
+        si.b = -g.sign * fd->b;
+        si.c = g.sign * fd->c;
+        si.u16 = eb == 2;
+        si.out_pitch = fd->out_pitch;
+        si.normals = reinterpret_cast<unsigned char*>(fd->normals) + ((long long)gy0 * fd->out_pitch + gx0) * BPP;
+        si.valid = fd->valid + (long long)gy0 * fd->out_pitch + gx0;
+#ifdef NRM_DEBUG_CHECKS
+        si.normals0 = fd->normals;
+        si.valid0 = fd->valid;
+        si.nlen = dbg_span(fd->H, fd->W, fd->out_pitch, BPP);
+        si.mlen = dbg_span(fd->H, fd->W, fd->out_pitch, 1);
+#endif
+        si.cols = fd->W - gx0;
+        si.rows = fd->H - gy0;
+        NRM_STS(reinterpret_cast<StripInfo*>(st + SB - TB), si);
+      }
+      // Column table, two float4 per lane, and row table: the terms of emit_pair.
+      float4* ctab = reinterpret_cast<float4*>(st + SB - TB + kStripInfoBytes);
+      const float cx = fd->cx, cy = fd->cy, ifx = fd->inv_fx, ify = fd->inv_fy;
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const float ua = ((float)(gx0 + 4 * lane + 2 * h) - cx) * ifx;
+        const float ub = ((float)(gx0 + 4 * lane + 2 * h + 1) - cx) * ifx;
+        NRM_STS(ctab + 2 * lane + h, make_float4(-ua, -ub, fmaf(ua, ua, 1.0f), fmaf(ub, ub, 1.0f)));
+      }
+      for (int r = lane; r < TY; r += 32) {
+        const float v1 = ((float)(gy0 + r) - cy) * ify;
+        NRM_STS(ctab + kStripX / 2 + r, make_float4(-v1, -v1, v1 * v1, v1 * v1));
+      }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(smem_u32(&full[s]));
+      if (++s == S) {
+        s = 0;
+        parity ^= 1;
+      }
+    }
+    return;
+  }
+
+  // -------------------------------------------------------------- compute
+  int s = 0;
+  uint32_t parity = 0;
+  for (int i = 0; i < my; ++i) {
+    if (!__all_sync(0xffffffffu, mbar_wait_bounded(smem_u32(&full[s]), parity, g.timeout_ns))) {
+      if (lane == 0) record_error(g.status, NRM_ERR_TIMEOUT);
+      return;
+    }
+    const unsigned char* st = smem + (size_t)s * SB;
+    const StripInfo f = NRM_LDS(StripInfo, reinterpret_cast<const StripInfo*>(st + SB - TB));
+    const float4* ctab = reinterpret_cast<const float4*>(st + SB - TB + kStripInfoBytes);
+    if (f.u16)
+      strip_band<OUT, SECANT, ALPHA>(reinterpret_cast<const uint16_t*>(st), ctab, ctab + kStripX / 2, f, warp, g.tau2);
+    else
+      strip_band<OUT, SECANT, ALPHA>(reinterpret_cast<const float*>(st), ctab, ctab + kStripX / 2, f, warp, g.tau2);
+    __syncwarp();
+    if (lane == 0) mbar_arrive(smem_u32(&empty[s]));
+    if (++s == S) {
+      s = 0;
+      parity ^= 1;
+    }
+  }
+}
+
+template <int OUT, bool SECANT, int ALPHA>
+__global__ void __launch_bounds__(strip_threads(OUT))
+    fwd_strip_param_kernel(const __grid_constant__ ParamBatch pb, const BatchArgs ring, const Globals g) {
+  BatchArgs args = ring;
+  args.hdr = &pb.hdr;
+  args.tile_begin = pb.tile_begin;
+  args.frames = pb.frames;
+  strip_pipeline<OUT, SECANT, ALPHA, false>(args, g);
+}
+
+template <int OUT, bool SECANT, int ALPHA>
+__global__ void __launch_bounds__(strip_threads(OUT)) fwd_strip_kernel(const BatchArgs args, const Globals g) {
+  strip_pipeline<OUT, SECANT, ALPHA, true>(args, g);
+}
+
+}  // namespace nrm

@@ -50,7 +50,9 @@ struct alignas(128) FrameDesc {
 static_assert(sizeof(FrameDesc) == 256, "FrameDesc layout");
 
 // Header of a batch's device descriptor block, followed by tile_begin[n+1]
-// (at kTileBeginOffset) and then the FrameDesc array (at frames_offset()).
+// (at kTileBeginOffset) and then the FrameDesc array (at frames_offset()). A
+// batch that runs as two launches has a second header and its tile_begin
+// after the first ones (second_header_offset()).
 struct BatchHeader {
   int n_frames;
   int total_tiles;
@@ -59,8 +61,14 @@ struct BatchHeader {
 static_assert(sizeof(BatchHeader) == 64, "BatchHeader layout");
 constexpr size_t kTileBeginOffset = 64;
 constexpr size_t frames_offset(int capacity) {
-  size_t b = kTileBeginOffset + sizeof(int) * (size_t)(capacity + 1);
+  size_t b = 2 * kTileBeginOffset + sizeof(int) * (size_t)(capacity + 17);
   return (b + 255) / 256 * 256;
+}
+// The second header of a batch whose first launch takes n frames (64-byte aligned;
+// its tile_begin follows it; both lists together hold at most capacity + 2 entries).
+constexpr size_t second_header_offset(int n) {
+  size_t b = kTileBeginOffset + sizeof(int) * (size_t)(n + 1);
+  return (b + 63) / 64 * 64;
 }
 constexpr size_t block_bytes(int capacity) { return frames_offset(capacity) + sizeof(FrameDesc) * (size_t)capacity; }
 
@@ -106,6 +114,23 @@ const void* fwd_points_kernel(int tile_x, int tile_y, int threads, int out_dtype
 const void* fwd_param_kernel(int tile_x, int tile_y, int threads, int out_dtype);
 size_t param_batch_bytes();
 void pack_param_batch(void* dst, const BatchHeader& hdr, const int* tile_begin, const FrameDesc* frames, int n);
+
+// Strip kernels (nrm_forward_strip.cu): the batched forward pass of frames whose
+// rows TMA can load and whose outputs take whole-vector stores (see
+// strip_frame in nrm_api.cpp), alpha <= kStripMaxAlpha. Descriptors are those of
+// the persistent kernels for tile kStripX x strip_tile_y(out_dtype). param_block: a ParamBatch
+// packed by pack_param_batch, or NULL for the device block in args. u16: every
+// frame is uint16.
+constexpr int kStripX = 128;
+NRM_HD constexpr int strip_rows(int out_dtype) { return out_dtype == NRM_OUT_OCT16 ? 8 : 4; }  // per warp
+NRM_HD constexpr int strip_warps(int out_dtype) {
+  return out_dtype == NRM_OUT_F32X4 ? 6 : out_dtype == NRM_OUT_F16X4 ? 12 : 4;
+}
+NRM_HD constexpr int strip_tile_y(int out_dtype) { return strip_rows(out_dtype) * strip_warps(out_dtype); }
+NRM_HD constexpr int strip_threads(int out_dtype) { return (strip_warps(out_dtype) + 1) * 32; }
+constexpr int kStripMaxAlpha = 4;
+cudaError_t launch_forward_strip(const BatchArgs& args, const Globals& g, int out_dtype, int total_tiles, bool u16,
+                                 cudaStream_t stream, const void* param_block = nullptr);
 
 // Stage buffer bytes for a tile config and alpha: for input elements of eb
 // bytes (2: uint16, 4: float32), or the maximum over both (eb = 0).
