@@ -876,8 +876,8 @@ int nrm_estimate_points(nrm_handle* h, const void* depth, void* normals, uint8_t
   return estimate_single(h, depth, normals, valid, points, cuda_stream);
 }
 
-// The frames of a batched forward call, in two parts: those that the strip
-// kernel takes, then the rest, each with its own work list.
+// The frames of a batched forward (or multi-scale) call, in two parts: those
+// that a strip kernel takes, then the rest, each with its own work list.
 namespace {
 
 struct BatchPart {
@@ -888,27 +888,39 @@ struct BatchPart {
   bool u16 = true;       // uint16 frames only
 };
 
-// True if the handle's batched calls may take the strip kernels.
+// How a call splits its frames: the halo of its tiles, whether a strip kernel
+// may take frames (of tiles kStripX x strip_y), the tiles of the other kernel,
+// and for multi-scale calls K and the divisor q of the form (1 or 4).
+struct BatchPlan {
+  int halo;
+  bool strip;
+  int strip_y;
+  int tile_x, tile_y;
+  int scales = 0;
+  double q = 4.0;
+};
+
+// True if the handle's batched forward calls may take the strip kernels.
 bool strip_handle(const nrm_handle* h) {
   const nrm_tile_config &c = h->cfg, &d = kDefaultConfig;
   return c.tile_x == d.tile_x && c.tile_y == d.tile_y && c.threads == d.threads && c.stages == d.stages &&
          c.ctas_per_sm == d.ctas_per_sm && h->p.alpha <= nrm::kStripMaxAlpha;
 }
 
-// True if the strip kernels can take frame f: whole vectors of four pixels to
-// the right edge, outputs on the alignment of the vector stores, and depth rows
+// True if a strip kernel can take frame f: whole vectors of four pixels to the
+// right edge, outputs on the alignment of the vector stores, and depth rows
 // that TMA can address (make_desc then decides by encoding the map).
-bool strip_frame(const nrm_handle* h, const nrm_frame& f) {
-  if (!strip_handle(h) || f.points) return false;
+bool strip_frame(const nrm_handle* h, const nrm_frame& f, const BatchPlan& plan) {
+  if (!plan.strip || f.points) return false;
   const uintptr_t na = h->p.out_dtype == NRM_OUT_OCT16 ? 16 : 32;
   const int eb = f.in_dtype == NRM_IN_U16_MM ? 2 : 4;
   if (f.in_dtype == NRM_IN_U16_MM) {
-    // The strip kernel leaves out the test q >= FLT_MIN for uint16: with every
-    // depth >= 1 unit, n . ray >= 4 c and so q >= 16 c^2 / |ray|^2.
-    const double a = h->p.alpha, s = h->p.depth_scale;
-    const double c = a * a / (4.0 * f.K.fx * f.K.fy) * s * s;
+    // The strip kernels leave out the test q >= FLT_MIN for uint16: with every
+    // depth >= 1 unit n . ray is at least pmin, and so q >= pmin^2 / |ray|^2.
+    const double s = h->p.depth_scale, a = plan.scales ? 1.0 : (double)h->p.alpha;
+    const double pmin = a * a / (f.K.fx * f.K.fy) * s * s / std::max(plan.scales, 1);
     const double u = (std::fabs(f.K.cx) + f.W) / f.K.fx, v = (std::fabs(f.K.cy) + f.H) / f.K.fy;
-    if (!(16.0 * c * c / (1.0 + u * u + v * v) >= 4.0 * 1.17549435e-38)) return false;
+    if (!(pmin * pmin / (1.0 + u * u + v * v) >= 4.0 * 1.17549435e-38)) return false;
   }
   return f.W % 4 == 0 && f.out_pitch % 4 == 0 && (uintptr_t)f.normals % na == 0 && (uintptr_t)f.valid % 4 == 0 &&
          (uintptr_t)f.depth % 16 == 0 && (f.depth_pitch * eb) % 16 == 0;
@@ -916,25 +928,34 @@ bool strip_frame(const nrm_handle* h, const nrm_frame& f) {
 
 // Descriptors of the n frames into fd: the strip kernel's from the front, the
 // others from the back. Empty frames are left out.
-void split_batch(const nrm_handle* h, const nrm_frame* frames, int n, FrameDesc* fd, BatchPart (&part)[2]) {
-  const int a = h->p.alpha;
-  part[0].tile_y = nrm::strip_tile_y(h->p.out_dtype);
-  part[1].tile_y = h->cfg.tile_y;
+void split_batch(const nrm_handle* h, const nrm_frame* frames, int n, const BatchPlan& plan, FrameDesc* fd,
+                 BatchPart (&part)[2]) {
+  part[0].tile_y = plan.strip_y;
+  part[1].tile_y = plan.tile_y;
   int front = 0, back = n;
   for (int i = 0; i < n; ++i) {
     const nrm_frame& f = frames[i];
     if ((long long)f.H * f.W == 0) continue;
     const int eb = f.in_dtype == NRM_IN_U16_MM ? 2 : 4;
-    bool strip = strip_frame(h, f);
+    bool strip = strip_frame(h, f, plan);
     if (strip) {
       make_desc(&fd[front], f.depth, f.normals, f.valid, f.H, f.W, f.depth_pitch, f.out_pitch, f.K, f.in_dtype, h->p,
-                nrm::kStripX, part[0].tile_y, nrm::kStripX + 2 * nrm::pad_x(a, eb), part[0].tile_y + 2 * a);
+                nrm::kStripX, plan.strip_y, nrm::kStripX + 2 * nrm::pad_x(plan.halo, eb),
+                plan.strip_y + 2 * plan.halo);
       strip = fd[front].use_tma != 0;
     }
     FrameDesc* d = strip ? &fd[front++] : &fd[--back];
     if (!strip)
       make_desc(d, f.depth, f.normals, f.valid, f.H, f.W, f.depth_pitch, f.out_pitch, f.K, f.in_dtype, h->p,
-                h->cfg.tile_x, h->cfg.tile_y, h->cfg.tile_x + 2 * nrm::pad_x(a, eb), h->cfg.tile_y + 2 * a);
+                plan.tile_x, plan.tile_y, plan.tile_x + 2 * nrm::pad_x(plan.halo, eb), plan.tile_y + 2 * plan.halo);
+    if (plan.scales) {
+      // Multi-scale: per-frame bases; the kernel scales them by alpha_i (a, b) and
+      // alpha_i^2 (c).
+      const double sc = f.in_dtype == NRM_IN_U16_MM ? (double)h->p.depth_scale : 1.0;
+      d->a = (float)(sc * sc / (plan.q * f.K.fy * plan.scales));
+      d->b = (float)(sc * sc / (plan.q * f.K.fx * plan.scales));
+      d->c = (float)(sc * sc / (plan.q * f.K.fx * f.K.fy * plan.scales));
+    }
     BatchPart& p = part[strip ? 0 : 1];
     p.u16 = p.u16 && f.in_dtype == NRM_IN_U16_MM;
     p.tiles += d->tiles_x * ((f.H + p.tile_y - 1) / p.tile_y);
@@ -943,6 +964,10 @@ void split_batch(const nrm_handle* h, const nrm_frame* frames, int n, FrameDesc*
   }
   part[0].first = 0;
   part[1].first = back;
+}
+
+BatchPlan forward_plan(const nrm_handle* h) {
+  return {h->p.alpha, strip_handle(h), nrm::strip_tile_y(h->p.out_dtype), h->cfg.tile_x, h->cfg.tile_y};
 }
 
 // One part's header and tile offsets (tile_begin: n + 1 entries).
@@ -958,6 +983,19 @@ void fill_work_list(const BatchPart& p, FrameDesc* fd, nrm::BatchHeader* hdr, in
     acc += d.tiles_x * ((d.H + p.tile_y - 1) / p.tile_y);
   }
   tile_begin[p.n] = acc;
+}
+
+// The 128-byte aligned parameter block of one part's launch, in h's scratch memory.
+void* pack_part(nrm_handle* h, const BatchPart& p, FrameDesc* fd) {
+  std::vector<int>& tb = h->scratch_tb;
+  if (tb.size() < (size_t)p.n + 1) tb.resize((size_t)p.n + 1);
+  std::vector<unsigned char>& raw = h->scratch_param;
+  if (raw.size() < nrm::param_batch_bytes() + 128) raw.resize(nrm::param_batch_bytes() + 128);
+  void* pb = raw.data() + (128 - reinterpret_cast<uintptr_t>(raw.data()) % 128) % 128;
+  nrm::BatchHeader hdr;
+  fill_work_list(p, fd, &hdr, tb.data());
+  nrm::pack_param_batch(pb, hdr, tb.data(), fd + p.first, p.n);
+  return pb;
 }
 
 // Launches one part: its descriptors as the kernel parameter (param_block) or
@@ -1004,11 +1042,9 @@ static int estimate_batched_param(nrm_handle* h, const nrm_frame* frames, int n,
     if (frames[i].points && (long long)frames[i].H * frames[i].W > 0)
       return fail(NRM_ERR_UNSUPPORTED, "frame %d: point clouds are not written during stream capture", i);
   std::vector<FrameDesc>& fd = h->scratch_desc;
-  std::vector<int>& tb = h->scratch_tb;
   if (fd.size() < (size_t)n) fd.resize((size_t)n);
-  if (tb.size() < (size_t)n + 2) tb.resize((size_t)n + 2);
   BatchPart part[2];  // strip kernel, tiled kernel
-  split_batch(h, frames, n, fd.data(), part);
+  split_batch(h, frames, n, forward_plan(h), fd.data(), part);
   Slot* s = nullptr;
   if (!capture) {
     // A ring slot supplies the completion (and, with timing on, the kernel
@@ -1018,15 +1054,9 @@ static int estimate_batched_param(nrm_handle* h, const nrm_frame* frames, int n,
     NRM_CHECK(retire_slot(h, *s));
     if (h->timing) NRM_CUDA(cudaEventRecord(s->ev_start, st), "cudaEventRecord");
   }
-  // The parameter block, 128-byte aligned like the records in it.
-  std::vector<unsigned char>& raw = h->scratch_param;
-  if (raw.size() < nrm::param_batch_bytes() + 128) raw.resize(nrm::param_batch_bytes() + 128);
-  void* pb = raw.data() + (128 - reinterpret_cast<uintptr_t>(raw.data()) % 128) % 128;
   for (int k = 0; k < 2; ++k) {
     if (part[k].tiles == 0) continue;
-    nrm::BatchHeader hdr;
-    fill_work_list(part[k], fd.data(), &hdr, tb.data());
-    nrm::pack_param_batch(pb, hdr, tb.data(), fd.data() + part[k].first, part[k].n);
+    void* pb = pack_part(h, part[k], fd.data());
     nrm::BatchArgs ring;
     std::memset(&ring, 0, sizeof(ring));
     NRM_CHECK(launch_part(h, k == 0, ring, part[k], pb, st));
@@ -1048,7 +1078,7 @@ static int estimate_batched_ring(nrm_handle* h, const nrm_frame* frames, int n, 
   char* base = static_cast<char*>(s.host);
   FrameDesc* fd = reinterpret_cast<FrameDesc*>(base + nrm::frames_offset(s.capacity));
   BatchPart part[2];
-  split_batch(h, frames, n, fd, part);
+  split_batch(h, frames, n, forward_plan(h), fd, part);
   const size_t off[2] = {0, nrm::second_header_offset(part[0].n)};
   for (int k = 0; k < 2; ++k)
     fill_work_list(part[k], fd, reinterpret_cast<nrm::BatchHeader*>(base + off[k]),
@@ -1548,14 +1578,12 @@ int nrm_estimate_batched_multiscale(nrm_handle* h, const nrm_frame* frames, int 
   if (!frames) return fail(NRM_ERR_INVALID_ARG, "frames is NULL");
   const int TX = nrm::kMsTileX, TY = nrm::kMsTileY;
   long long total = 0;
-  bool u16 = true;
   for (int i = 0; i < n; ++i) {
     rc = validate_frame(frames[i], i, h->p.out_dtype);
     if (rc) return rc;
     if (frames[i].points) return fail(NRM_ERR_UNSUPPORTED, "frame %d: the multi-scale variant writes no point clouds", i);
     total += (long long)((frames[i].W + TX - 1) / TX) * ((frames[i].H + TY - 1) / TY);
     if (total >= (1LL << 31) - 1) return fail(NRM_ERR_UNSUPPORTED, "batch exceeds 2^31 tiles");
-    u16 = u16 && (frames[i].in_dtype == NRM_IN_U16_MM || (long long)frames[i].H * frames[i].W == 0);
   }
   if (total == 0) return NRM_OK;
   DeviceGuard guard(h->device);
@@ -1563,78 +1591,45 @@ int nrm_estimate_batched_multiscale(nrm_handle* h, const nrm_frame* frames, int 
   cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
   NRM_CUDA(cudaStreamIsCapturing(st, &capture), "cudaStreamIsCapturing");
   const bool captured = capture == cudaStreamCaptureStatusActive;
-  // Up to kParamMaxFrames frames (and always during capture) the descriptor
-  // block is one kernel parameter; larger batches upload it into a ring slot.
-  const bool param = n <= nrm::kParamMaxFrames;
-  if (captured && !param)
+  if (captured && n > nrm::kParamMaxFrames)
     return fail(NRM_ERR_UNSUPPORTED, "at most %d frames per call during stream capture", nrm::kParamMaxFrames);
+  // A ring slot supplies the completion event; the descriptors travel as the
+  // kernel parameter, kParamMaxFrames frames to a launch.
   Slot* sp = nullptr;
   if (!captured) {
     sp = &h->slots[h->next_slot];
     h->next_slot = (h->next_slot + 1) % kSlots;
     NRM_CHECK(retire_slot(h, *sp));
-    if (!param) NRM_CHECK(ensure_slot_capacity(h, *sp, n));
   }
-  std::vector<FrameDesc> fdv;
-  std::vector<int> tbv;
-  nrm::BatchHeader hdr_local;
-  std::memset(&hdr_local, 0, sizeof(hdr_local));
-  nrm::BatchHeader* hdr = &hdr_local;
-  FrameDesc* fd;
-  int* tb;
-  if (param) {
-    fdv.resize((size_t)n);
-    tbv.resize((size_t)n + 1);
-    fd = fdv.data();
-    tb = tbv.data();
-  } else {
-    char* base = static_cast<char*>(sp->host);
-    hdr = reinterpret_cast<nrm::BatchHeader*>(base);
-    tb = reinterpret_cast<int*>(base + nrm::kTileBeginOffset);
-    fd = reinterpret_cast<FrameDesc*>(base + nrm::frames_offset(sp->capacity));
-  }
-  const double q = scales->form == NRM_MS_QUAD ? 4.0 : 1.0;
-  int acc = 0;
-  for (int i = 0; i < n; ++i) {
-    const nrm_frame& f = frames[i];
-    const int eb = f.in_dtype == NRM_IN_U16_MM ? 2 : 4;
-    make_desc(&fd[i], f.depth, f.normals, f.valid, f.H, f.W, f.depth_pitch, f.out_pitch, f.K, f.in_dtype, h->p,
-              TX, TY, TX + 2 * nrm::pad_x(ms.alpha_max, eb), TY + 2 * ms.alpha_max);
-    // Per-frame bases; the kernel scales them by alpha_i (a, b) and alpha_i^2 (c).
-    const double sc = f.in_dtype == NRM_IN_U16_MM ? (double)h->p.depth_scale : 1.0;
-    fd[i].a = (float)(sc * sc / (q * f.K.fy * ms.K));
-    fd[i].b = (float)(sc * sc / (q * f.K.fx * ms.K));
-    fd[i].c = (float)(sc * sc / (q * f.K.fx * f.K.fy * ms.K));
-    fd[i].tile_begin = acc;
-    tb[i] = acc;
-    acc += fd[i].tiles_x * ((f.H + TY - 1) / TY);
-  }
-  tb[n] = acc;
-  hdr->n_frames = n;
-  hdr->total_tiles = acc;
-  nrm::BatchArgs args;
-  std::memset(&args, 0, sizeof(args));
-  nrm::Globals g = make_globals(h);
-  if (param) {
-    std::vector<unsigned char> raw(nrm::param_batch_bytes() + 128);
-    void* pb = raw.data() + (128 - reinterpret_cast<uintptr_t>(raw.data()) % 128) % 128;
-    nrm::pack_param_batch(pb, *hdr, tb, fd, n);
-    NRM_CUDA(nrm::launch_multiscale_batched(args, ms, g, h->p.out_dtype, scales->form, acc, u16, st, pb),
-             "launch fwd_ms_persistent_param_kernel");
-  } else {
-    const size_t used = nrm::frames_offset(sp->capacity) + sizeof(FrameDesc) * (size_t)n;
-    NRM_CUDA(cudaMemcpyAsync(sp->dev, sp->host, used, cudaMemcpyHostToDevice, st), "cudaMemcpyAsync");
-    args.hdr = reinterpret_cast<const nrm::BatchHeader*>(sp->dev);
-    args.tile_begin = reinterpret_cast<const int*>(static_cast<char*>(sp->dev) + nrm::kTileBeginOffset);
-    args.frames = reinterpret_cast<const FrameDesc*>(static_cast<char*>(sp->dev) + nrm::frames_offset(sp->capacity));
-    NRM_CUDA(nrm::launch_multiscale_batched(args, ms, g, h->p.out_dtype, scales->form, acc, u16, st),
-             "launch fwd_ms_persistent_kernel");
+  bool consecutive = ms.K >= 2 && ms.K <= nrm::kMsStripMaxScales;
+  for (int i = 0; i < ms.K; ++i) consecutive = consecutive && ms.alpha[i] == i + 1;
+  const BatchPlan plan = {ms.alpha_max, consecutive, nrm::ms_strip_tile_y(), TX, TY, ms.K,
+                          scales->form == NRM_MS_QUAD ? 4.0 : 1.0};
+  const nrm::Globals g = make_globals(h);
+  std::vector<FrameDesc>& fd = h->scratch_desc;
+  if (fd.size() < (size_t)std::min(n, nrm::kParamMaxFrames)) fd.resize((size_t)std::min(n, nrm::kParamMaxFrames));
+  int tiles = 0;
+  for (int first = 0; first < n; first += nrm::kParamMaxFrames) {
+    BatchPart part[2];
+    split_batch(h, frames + first, std::min(n - first, nrm::kParamMaxFrames), plan, fd.data(), part);
+    for (int k = 0; k < 2; ++k) {
+      const BatchPart& p = part[k];
+      tiles += p.tiles;
+      if (p.tiles == 0) continue;
+      void* pb = pack_part(h, p, fd.data());
+      if (k == 0)
+        NRM_CUDA(nrm::launch_multiscale_strip(ms, g, h->p.out_dtype, scales->form, p.tiles, p.u16, st, pb),
+                 "launch fwd_ms_strip_kernel");
+      else
+        NRM_CUDA(nrm::launch_multiscale_batched(ms, g, h->p.out_dtype, scales->form, p.tiles, p.u16, st, pb),
+                 "launch fwd_ms_persistent_param_kernel");
+    }
   }
   if (sp) {
     NRM_CUDA(cudaEventRecord(sp->done, st), "cudaEventRecord");
     sp->in_flight = true;
     sp->timed_launch = false;
-    sp->tiles = acc;
+    sp->tiles = tiles;
   }
   return NRM_OK;
 }

@@ -11,13 +11,13 @@
 //   float4: 6 warps x 4 rows, 3 stages   375-380 us (98 %), float32 input 429 us
 //           (96 %), alpha 3 / 4 392 / 379 us; 256 mixed float32 frames 1.05 ms
 //           (98 %)  [8 warps x 8 rows, 3 stages 440; 4 x 4, 4 stages, 409]
-//   half4:  12 warps x 4 rows, 3 stages  227-229 us (94 %), float32 input 260 us
+//   half4:  12 warps x 4 rows, 3 stages  226 us (95 %), float32 input 259 us
 //           (98 %)  [10 warps, 4 stages 222 / 292; 8 x 8, 3 stages 221 / 294]
 // The tiled kernel in its default geometry (128x16, 256 threads) takes 441,
 // 348 and 1283 us on the float4, half4 and mixed batches.
 // The octahedral output is bound by instruction issue (about 40 instructions a
-// pixel), so as many warps as fit run: 4 warps x 8 rows, 197 us (69 %; tiled
-// 341 us); float32 input with 2 stages, 4 CTAs, 200 us (3 stages, 3 CTAs: 205).
+// pixel), so as many warps as fit run: 4 warps x 8 rows, 192 us (71 %; tiled
+// 341 us); float32 input with 2 stages, 4 CTAs, 198 us (3 stages, 3 CTAs: 205).
 // Batches of few tiles take all the CTAs that fit: there the ramp counts, not the
 // steady state (16 x 640x480 float32: 18.8 us with 3 CTAs per SM, 20.9 with one;
 // 2 x 1080p 15.2 against 16.0, 4 x 1080p 30.7 against 29.6 us).
@@ -64,7 +64,7 @@ cudaError_t launch_forward_strip(const BatchArgs& args, const Globals& g, int ou
   if (!fn) return cudaErrorInvalidValue;
   const int eb = u16 ? 2 : 4;
   const int stages = strip_stages(out_dtype, u16);
-  const unsigned smem = strip_smem_bytes(out_dtype, g.alpha, eb, stages);
+  const unsigned smem = strip_smem_bytes(strip_tile_y(out_dtype), g.alpha, eb, stages);
   const int threads = strip_threads(out_dtype);
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
@@ -76,7 +76,7 @@ cudaError_t launch_forward_strip(const BatchArgs& args, const Globals& g, int ou
   std::atomic<int>& occ = fit[out_dtype][secant][g.alpha][param][u16][dev];
   if (occ.load() == 0) {
     int sms = 0, n = 0;
-    e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)strip_smem_bytes(out_dtype, kStripMaxAlpha, 4, 3));
+    e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)strip_smem_bytes(strip_tile_y(out_dtype), kStripMaxAlpha, 4, 3));
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fn, threads, smem);
     if (e != cudaSuccess) return e;
@@ -91,7 +91,7 @@ cudaError_t launch_forward_strip(const BatchArgs& args, const Globals& g, int ou
   const int ctas = per_sm * sms;
   BatchArgs a = args;
   a.stages = stages;
-  a.stage_bytes = strip_stage_bytes(out_dtype, g.alpha, eb);
+  a.stage_bytes = strip_stage_bytes(strip_tile_y(out_dtype), g.alpha, eb);
   Globals gg = g;
   const dim3 grid(std::min(total_tiles, ctas)), block(threads);
   if (param) {

@@ -48,14 +48,14 @@ static_assert(sizeof(StripInfo) <= kStripInfoBytes, "StripInfo must fit its slot
 
 // Shared memory of a stage: raw depth box, record, column table (two float4
 // per lane), row table.
-NRM_HD constexpr unsigned strip_table_bytes(int out_dtype) {
-  return (kStripInfoBytes + (kStripX / 2 + strip_tile_y(out_dtype)) * 16u + 127) / 128 * 128;
+NRM_HD constexpr unsigned strip_table_bytes(int tile_y) {
+  return (kStripInfoBytes + (kStripX / 2 + tile_y) * 16u + 127) / 128 * 128;
 }
-NRM_HD inline unsigned strip_stage_bytes(int out_dtype, int alpha, int eb) {
-  return stage_bytes_for(kStripX, strip_tile_y(out_dtype), alpha, eb) + strip_table_bytes(out_dtype);
+NRM_HD inline unsigned strip_stage_bytes(int tile_y, int halo, int eb) {
+  return stage_bytes_for(kStripX, tile_y, halo, eb) + strip_table_bytes(tile_y);
 }
-NRM_HD inline unsigned strip_smem_bytes(int out_dtype, int alpha, int eb, int stages) {
-  return (strip_stage_bytes(out_dtype, alpha, eb) + 16) * stages;
+NRM_HD inline unsigned strip_smem_bytes(int tile_y, int halo, int eb, int stages) {
+  return (strip_stage_bytes(tile_y, halo, eb) + 16) * stages;
 }
 
 __device__ __forceinline__ float min3_nan(float a, float b, float c) {
@@ -102,24 +102,17 @@ __device__ __forceinline__ float2 load_two(const float* p) {
   return depth_pair(NRM_LDS(float2, reinterpret_cast<const float2*>(p)));
 }
 
-// One pixel pair: the closed form, the statistic and the mask decision, in the
-// operation order of QuadStencil and emit_pair.
+// Section 3.2 for one pixel pair, in the operation order of emit_pair: n_z, q and
+// the mask decisions. mn: the smallest of all depths each pixel uses.
 template <bool SECANT, bool U16>
-__device__ __forceinline__ void strip_pair(float2 d1, float2 d2, float2 d3, float2 d4, float2 d5, float2 A, float2 B,
-                                           float2 C, float2 T, float tau2, float2 nu1, float2 ku, float2 nv1,
-                                           float2 kv, float2& nx, float2& ny, float2& nz, float2& q, bool& ka,
-                                           bool& kb) {
+__device__ __forceinline__ void strip_decide(float2 mn, float2 nx, float2 ny, float2 P, float2 T, float tau2,
+                                             float2 nu1, float2 ku, float2 nv1, float2 kv, float2& nz, float2& q,
+                                             bool& ka, bool& kb) {
   const float kFltMin = 1.17549435e-38f;
-  const float2 M1 = f2(-1.0f, -1.0f);
-  const float2 S24 = __fadd2_rn(d2, d4), D24 = __ffma2_rn(M1, d4, d2);
-  const float2 S35 = __fadd2_rn(d3, d5), D35 = __ffma2_rn(M1, d5, d3);
-  nx = __fmul2_rn(__fmul2_rn(A, S35), D24);
-  ny = __fmul2_rn(__fmul2_rn(B, S24), D35);
-  const float2 P = __fmul2_rn(__fmul2_rn(C, S24), S35);
   nz = __ffma2_rn(nu1, nx, __ffma2_rn(nv1, ny, P));
   q = __ffma2_rn(nx, nx, __ffma2_rn(ny, ny, __fmul2_rn(nz, nz)));
-  ka = min3_nan(min3_nan(d1.x, d2.x, d3.x), d4.x, d5.x) > 0.0f;
-  kb = min3_nan(min3_nan(d1.y, d2.y, d3.y), d4.y, d5.y) > 0.0f;
+  ka = mn.x > 0.0f;
+  kb = mn.y > 0.0f;
   if (!U16) {
     ka = ka & (q.x >= kFltMin);
     kb = kb & (q.y >= kFltMin);
@@ -135,6 +128,24 @@ __device__ __forceinline__ void strip_pair(float2 d1, float2 d2, float2 d3, floa
   }
 }
 
+// The stencil of Eq. 4-6 of one pixel pair, in the operation order of
+// QuadStencil, then strip_decide.
+template <bool SECANT, bool U16>
+__device__ __forceinline__ void strip_pair(float2 d1, float2 d2, float2 d3, float2 d4, float2 d5, float2 A, float2 B,
+                                           float2 C, float2 T, float tau2, float2 nu1, float2 ku, float2 nv1,
+                                           float2 kv, float2& nx, float2& ny, float2& nz, float2& q, bool& ka,
+                                           bool& kb) {
+  const float2 M1 = f2(-1.0f, -1.0f);
+  const float2 S24 = __fadd2_rn(d2, d4), D24 = __ffma2_rn(M1, d4, d2);
+  const float2 S35 = __fadd2_rn(d3, d5), D35 = __ffma2_rn(M1, d5, d3);
+  nx = __fmul2_rn(__fmul2_rn(A, S35), D24);
+  ny = __fmul2_rn(__fmul2_rn(B, S24), D35);
+  const float2 P = __fmul2_rn(__fmul2_rn(C, S24), S35);
+  const float2 mn = f2(min3_nan(min3_nan(d1.x, d2.x, d3.x), d4.x, d5.x),
+                       min3_nan(min3_nan(d1.y, d2.y, d3.y), d4.y, d5.y));
+  strip_decide<SECANT, U16>(mn, nx, ny, P, T, tau2, nu1, ku, nv1, kv, nz, q, ka, kb);
+}
+
 // The octahedral codes of a pixel pair (oct16_code, operation for operation,
 // with the additions, the scale and the rounding steps paired).
 __device__ __forceinline__ void strip_codes(float2 nx, float2 ny, float2 nz, uint32_t& ca, uint32_t& cb) {
@@ -147,6 +158,64 @@ __device__ __forceinline__ void strip_codes(float2 nx, float2 ny, float2 nz, uin
   const float2 x = __ffma2_rn(tx, s, k), y = __ffma2_rn(ty, s, k);
   ca = __byte_perm(__float_as_uint(x.x), __float_as_uint(y.x), 0x5410);
   cb = __byte_perm(__float_as_uint(x.y), __float_as_uint(y.y), 0x5410);
+}
+
+// The normals (or codes) and mask bytes of a lane's four pixels: np, mp point at
+// the first one's; k[i] says whether pixel i is valid.
+template <int OUT>
+__device__ __forceinline__ void strip_store(const float2 (&nx)[2], const float2 (&ny)[2], const float2 (&nz)[2],
+                                            const float2 (&q)[2], const bool (&k)[4], unsigned char* np, uint8_t* mp,
+                                            bool on, [[maybe_unused]] const StripInfo& f) {
+  [[maybe_unused]] constexpr int BPP = OUT == NRM_OUT_F32X4 ? 16 : OUT == NRM_OUT_F16X4 ? 8 : 4;
+  const uint32_t mbits =
+      (k[0] ? 1u : 0u) | (k[1] ? 0x100u : 0u) | (k[2] ? 0x10000u : 0u) | (k[3] ? 0x1000000u : 0u);
+  uint32_t w[4 * BPP / 4];
+  if constexpr (OUT == NRM_OUT_OCT16) {
+    strip_codes(nx[0], ny[0], nz[0], w[0], w[1]);
+    strip_codes(nx[1], ny[1], nz[1], w[2], w[3]);
+    w[0] = k[0] ? w[0] : 0u;
+    w[1] = k[1] ? w[1] : 0u;
+    w[2] = k[2] ? w[2] : 0u;
+    w[3] = k[3] ? w[3] : 0u;
+  } else {
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      const bool ka = k[2 * j], kb = k[2 * j + 1];
+      const float2 inv = f2(rsqrt_ftz(q[j].x), rsqrt_ftz(q[j].y));
+      const float2 ox = __fmul2_rn(nx[j], inv), oy = __fmul2_rn(ny[j], inv), oz = __fmul2_rn(nz[j], inv);
+      if constexpr (OUT == NRM_OUT_F16X4) {
+        w[4 * j] = ka ? h2_bits(__floats2half2_rn(ox.x, oy.x)) : 0u;
+        w[4 * j + 1] = ka ? h2_bits(__floats2half2_rn(oz.x, 0.0f)) : 0u;
+        w[4 * j + 2] = kb ? h2_bits(__floats2half2_rn(ox.y, oy.y)) : 0u;
+        w[4 * j + 3] = kb ? h2_bits(__floats2half2_rn(oz.y, 0.0f)) : 0u;
+      } else {
+        w[8 * j] = __float_as_uint(ka ? ox.x : 0.0f);
+        w[8 * j + 1] = __float_as_uint(ka ? oy.x : 0.0f);
+        w[8 * j + 2] = __float_as_uint(ka ? oz.x : 0.0f);
+        w[8 * j + 3] = 0u;
+        w[8 * j + 4] = __float_as_uint(kb ? ox.y : 0.0f);
+        w[8 * j + 5] = __float_as_uint(kb ? oy.y : 0.0f);
+        w[8 * j + 6] = __float_as_uint(kb ? oz.y : 0.0f);
+        w[8 * j + 7] = 0u;
+      }
+    }
+  }
+#ifdef NRM_DEBUG_CHECKS
+  if (on && !(dbg_gmem_ok(np, 4 * BPP, f.normals0, f.nlen, "strip normals", __LINE__) &&
+              dbg_gmem_ok(mp, 4, f.valid0, f.mlen, "strip mask", __LINE__)))
+    return;
+#endif
+  if (on) {
+    if constexpr (OUT == NRM_OUT_F32X4) {
+      store32(np, w[0], w[1], w[2], w[3], w[4], w[5], w[6], w[7]);
+      store32(np + 32, w[8], w[9], w[10], w[11], w[12], w[13], w[14], w[15]);
+    } else if constexpr (OUT == NRM_OUT_F16X4) {
+      store32(np, w[0], w[1], w[2], w[3], w[4], w[5], w[6], w[7]);
+    } else {
+      __stcs(reinterpret_cast<uint4*>(np), make_uint4(w[0], w[1], w[2], w[3]));
+    }
+    __stcs(reinterpret_cast<unsigned int*>(mp), mbits);
+  }
 }
 
 // One band: strip_rows(OUT) rows of 128 columns from the staged box S (its first
@@ -208,59 +277,12 @@ __device__ __forceinline__ void strip_band(const InT* __restrict__ S, const floa
       const float4 rr = NRM_LDS(float4, rtab + row0 + r);
       const float2 nv1 = f2(rr.x, rr.y), kv = f2(rr.z, rr.w);
       float2 nx[2], ny[2], nz[2], q[2];
-      bool k0, k1, k2, k3;
+      bool keep[4];
       strip_pair<SECANT, EB == 2>(m0, r0, b0, l0, u0, A, B, C, T, tau2, nu1[0], ku[0], nv1, kv, nx[0], ny[0], nz[0],
-                                  q[0], k0, k1);
+                                  q[0], keep[0], keep[1]);
       strip_pair<SECANT, EB == 2>(m1, r1, b1, l1, u1, A, B, C, T, tau2, nu1[1], ku[1], nv1, kv, nx[1], ny[1], nz[1],
-                                  q[1], k2, k3);
-      const uint32_t mbits = (k0 ? 1u : 0u) | (k1 ? 0x100u : 0u) | (k2 ? 0x10000u : 0u) | (k3 ? 0x1000000u : 0u);
-      uint32_t w[4 * BPP / 4];
-      if constexpr (OUT == NRM_OUT_OCT16) {
-        strip_codes(nx[0], ny[0], nz[0], w[0], w[1]);
-        strip_codes(nx[1], ny[1], nz[1], w[2], w[3]);
-        w[0] = k0 ? w[0] : 0u;
-        w[1] = k1 ? w[1] : 0u;
-        w[2] = k2 ? w[2] : 0u;
-        w[3] = k3 ? w[3] : 0u;
-      } else {
-#pragma unroll
-        for (int j = 0; j < 2; ++j) {
-          const bool ka = j ? k2 : k0, kb = j ? k3 : k1;
-          const float2 inv = f2(rsqrt_ftz(q[j].x), rsqrt_ftz(q[j].y));
-          const float2 ox = __fmul2_rn(nx[j], inv), oy = __fmul2_rn(ny[j], inv), oz = __fmul2_rn(nz[j], inv);
-          if constexpr (OUT == NRM_OUT_F16X4) {
-            w[4 * j] = ka ? h2_bits(__floats2half2_rn(ox.x, oy.x)) : 0u;
-            w[4 * j + 1] = ka ? h2_bits(__floats2half2_rn(oz.x, 0.0f)) : 0u;
-            w[4 * j + 2] = kb ? h2_bits(__floats2half2_rn(ox.y, oy.y)) : 0u;
-            w[4 * j + 3] = kb ? h2_bits(__floats2half2_rn(oz.y, 0.0f)) : 0u;
-          } else {
-            w[8 * j] = __float_as_uint(ka ? ox.x : 0.0f);
-            w[8 * j + 1] = __float_as_uint(ka ? oy.x : 0.0f);
-            w[8 * j + 2] = __float_as_uint(ka ? oz.x : 0.0f);
-            w[8 * j + 3] = 0u;
-            w[8 * j + 4] = __float_as_uint(kb ? ox.y : 0.0f);
-            w[8 * j + 5] = __float_as_uint(kb ? oy.y : 0.0f);
-            w[8 * j + 6] = __float_as_uint(kb ? oz.y : 0.0f);
-            w[8 * j + 7] = 0u;
-          }
-        }
-      }
-#ifdef NRM_DEBUG_CHECKS
-      if (on && !(dbg_gmem_ok(np, 4 * BPP, f.normals0, f.nlen, "strip normals", __LINE__) &&
-                  dbg_gmem_ok(mp, 4, f.valid0, f.mlen, "strip mask", __LINE__)))
-        break;
-#endif
-      if (on) {
-        if constexpr (OUT == NRM_OUT_F32X4) {
-          store32(np, w[0], w[1], w[2], w[3], w[4], w[5], w[6], w[7]);
-          store32(np + 32, w[8], w[9], w[10], w[11], w[12], w[13], w[14], w[15]);
-        } else if constexpr (OUT == NRM_OUT_F16X4) {
-          store32(np, w[0], w[1], w[2], w[3], w[4], w[5], w[6], w[7]);
-        } else {
-          __stcs(reinterpret_cast<uint4*>(np), make_uint4(w[0], w[1], w[2], w[3]));
-        }
-        __stcs(reinterpret_cast<unsigned int*>(mp), mbits);
-      }
+                                  q[1], keep[2], keep[3]);
+      strip_store<OUT>(nx, ny, nz, q, keep, np, mp, on, f);
       np += ALPHA * f.out_pitch * BPP;
       mp += ALPHA * f.out_pitch;
       u0 = m0;
@@ -271,14 +293,19 @@ __device__ __forceinline__ void strip_band(const InT* __restrict__ S, const floa
   }
 }
 
-template <int OUT, bool SECANT, int ALPHA, bool RING>
-__device__ __forceinline__ void strip_pipeline(const BatchArgs& args, const Globals& g) {
+// The pipeline of a strip kernel: tiles of kStripX x (ROWS x WARPS) pixels with a halo
+// of HALO; band(stage, column table, row table, record, warp) computes one
+// band, its stage pointer typed by the frame's depth type. RING: the descriptors
+// are in global memory written by the host (each tensor map is fenced before
+// its first use), else in kernel-parameter space.
+template <int OUT, int HALO, int ROWS, int WARPS, bool RING, class Band>
+__device__ __forceinline__ void strip_pipeline(const BatchArgs& args, const Globals& g, const Band& band) {
   extern __shared__ __align__(128) unsigned char smem[];
   constexpr int BPP = OUT == NRM_OUT_F32X4 ? 16 : OUT == NRM_OUT_F16X4 ? 8 : 4;
   const int S = args.stages;
   const unsigned SB = args.stage_bytes;
-  constexpr int WARPS = strip_warps(OUT), TY = strip_tile_y(OUT);
-  constexpr unsigned TB = strip_table_bytes(OUT);
+  constexpr int TY = ROWS * WARPS;
+  constexpr unsigned TB = strip_table_bytes(TY);
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + (size_t)S * SB);
   uint64_t* empty = full + S;
   const int total = args.hdr->total_tiles;
@@ -324,10 +351,10 @@ __device__ __forceinline__ void strip_pipeline(const BatchArgs& args, const Glob
           fence_tensormap_acquire(&fd->tmap);
           fenced = cur;
         }
-        const int padx = pad_x(ALPHA, eb);
+        const int padx = pad_x(HALO, eb);
         const uint32_t bar = smem_u32(&full[s]);
-        mbar_arrive_expect_tx(bar, (uint32_t)((kStripX + 2 * padx) * (TY + 2 * ALPHA) * eb));
-        tma_load_2d(smem_u32(st), &fd->tmap, gx0 - padx, gy0 - ALPHA, bar);
+        mbar_arrive_expect_tx(bar, (uint32_t)((kStripX + 2 * padx) * (TY + 2 * HALO) * eb));
+        tma_load_2d(smem_u32(st), &fd->tmap, gx0 - padx, gy0 - HALO, bar);
         StripInfo si;
         si.a = -g.sign * fd->a;
         si.b = -g.sign * fd->b;
@@ -381,9 +408,9 @@ __device__ __forceinline__ void strip_pipeline(const BatchArgs& args, const Glob
     const StripInfo f = NRM_LDS(StripInfo, reinterpret_cast<const StripInfo*>(st + SB - TB));
     const float4* ctab = reinterpret_cast<const float4*>(st + SB - TB + kStripInfoBytes);
     if (f.u16)
-      strip_band<OUT, SECANT, ALPHA>(reinterpret_cast<const uint16_t*>(st), ctab, ctab + kStripX / 2, f, warp, g.tau2);
+      band(reinterpret_cast<const uint16_t*>(st), ctab, ctab + kStripX / 2, f, warp);
     else
-      strip_band<OUT, SECANT, ALPHA>(reinterpret_cast<const float*>(st), ctab, ctab + kStripX / 2, f, warp, g.tau2);
+      band(reinterpret_cast<const float*>(st), ctab, ctab + kStripX / 2, f, warp);
     __syncwarp();
     if (lane == 0) mbar_arrive(smem_u32(&empty[s]));
     if (++s == S) {
@@ -393,19 +420,27 @@ __device__ __forceinline__ void strip_pipeline(const BatchArgs& args, const Glob
   }
 }
 
+template <int OUT, bool SECANT, int ALPHA, bool RING>
+__device__ __forceinline__ void strip_forward(const BatchArgs& args, const Globals& g) {
+  strip_pipeline<OUT, ALPHA, strip_rows(OUT), strip_warps(OUT), RING>(
+      args, g, [&](const auto* S, const float4* ctab, const float4* rtab, const StripInfo& f, int warp) {
+        strip_band<OUT, SECANT, ALPHA>(S, ctab, rtab, f, warp, g.tau2);
+      });
+}
+
 template <int OUT, bool SECANT, int ALPHA>
-__global__ void __launch_bounds__(strip_threads(OUT))
+__global__ void __launch_bounds__(strip_threads(OUT), OUT == NRM_OUT_OCT16 ? 4 : 1)
     fwd_strip_param_kernel(const __grid_constant__ ParamBatch pb, const BatchArgs ring, const Globals g) {
   BatchArgs args = ring;
   args.hdr = &pb.hdr;
   args.tile_begin = pb.tile_begin;
   args.frames = pb.frames;
-  strip_pipeline<OUT, SECANT, ALPHA, false>(args, g);
+  strip_forward<OUT, SECANT, ALPHA, false>(args, g);
 }
 
 template <int OUT, bool SECANT, int ALPHA>
-__global__ void __launch_bounds__(strip_threads(OUT)) fwd_strip_kernel(const BatchArgs args, const Globals g) {
-  strip_pipeline<OUT, SECANT, ALPHA, true>(args, g);
+__global__ void __launch_bounds__(strip_threads(OUT), OUT == NRM_OUT_OCT16 ? 4 : 1) fwd_strip_kernel(const BatchArgs args, const Globals g) {
+  strip_forward<OUT, SECANT, ALPHA, true>(args, g);
 }
 
 }  // namespace nrm

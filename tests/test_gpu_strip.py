@@ -37,7 +37,8 @@ def both(b, items, outputs=lambda: None):
 
 
 def bits(t):
-    return t.view(torch.int32) if t.dtype == torch.float32 else t.view(torch.int16) if t.element_size() == 2 else t
+    t = t.contiguous()
+    return t.view(torch.int32) if t.dtype == torch.float32 else t.view(torch.int16)
 
 
 def assert_same(one, two, what):
@@ -94,3 +95,26 @@ def test_uint16_frames_whose_statistic_could_underflow_take_the_tiled_kernels():
     items = [(torch.randint(1, 40, (64, 256), generator=gen, device=DEV).to(torch.uint16), (500.0, 500.0, 128.0, 32.0))]
     one, two = both(b, items)
     assert_same(one, two, "underflow")
+
+
+@pytest.mark.parametrize("form", ["pair", "quad"])
+@pytest.mark.parametrize("K", [2, 3, 4, 5, 6])
+def test_multiscale_same_bits_as_the_run_time_distance_kernel(form, K):
+    """Distances 1..K: frames with aligned rows take the strip kernels, the same
+    frames with an odd output pitch the other kernel. More frames than one
+    launch takes, sizes around the tile edges, depth values of every kind."""
+    gen = torch.Generator(device=DEV)
+    gen.manual_seed(K)
+    sizes = SIZES + [(64, 63), (128, 64), (136, 65), (384, 7)]
+    items = [(depth(W, H, dt, gen), (0.8 * W, 0.9 * W, 0.4 * W, 0.6 * H)) for W, H in sizes for dt in ("f32", "u16")]
+    items = items * 5 if K == 4 else items
+    for out, C, dt in (("f32", 4, torch.float32), ("f16", 4, torch.float16), ("oct16", 2, torch.int16)):
+        for mask, tau in (("secant", 12.0), ("raw", 1e-3)):
+            b = nrm.BatchedEstimator(nrm.NormalParams(out_dtype=out, mask_mode=mask, tau=tau))
+            wide = [(torch.zeros((*d.shape[:1], d.shape[1] + 1, C), dtype=dt, device=DEV)[:, :d.shape[1]],
+                     torch.zeros((d.shape[0], d.shape[1] + 1), dtype=torch.uint8, device=DEV)[:, :d.shape[1]])
+                    for d, _ in items]
+            one = b.multiscale(items, range(1, K + 1), form)
+            two = b.multiscale(items, range(1, K + 1), form, outputs=wide)
+            b.sync_status()
+            assert_same(one, two, (form, K, out, mask))
