@@ -32,7 +32,7 @@ LIB = os.path.join(BUILD, "libnrm.so")
 DEBUG_BUILD = os.path.join(BUILD, "debug")
 DEBUG_LIB = os.path.join(BUILD, "libnrm_debug.so")
 
-SOURCES = ["nrm_forward.cu", "nrm_forward_points.cu", "nrm_forward_param.cu", "nrm_forward_strip.cu", "nrm_multiscale_strip.cu", "nrm_multiscale_strip_f16.cu", "nrm_multiscale_strip_oct.cu", "nrm_backward.cu", "nrm_api.cpp", "nrm_noalloc.cu", "nrm_eval.cu", "nrm_planefit.cu", "nrm_multiscale.cu", "nrm_selftest.cu"]
+SOURCES = ["nrm_forward.cu", "nrm_forward_points.cu", "nrm_forward_param.cu", "nrm_forward_strip.cu", "nrm_forward_strip_any.cu", "nrm_multiscale_strip.cu", "nrm_multiscale_strip_f16.cu", "nrm_multiscale_strip_oct.cu", "nrm_backward.cu", "nrm_api.cpp", "nrm_noalloc.cu", "nrm_eval.cu", "nrm_planefit.cu", "nrm_multiscale.cu", "nrm_selftest.cu"]
 HEADERS = ["nrm_internal.h", "nrm_device.cuh", "nrm_forward_kernels.cuh", "nrm_forward_vec.cuh", "nrm_forward_strip.cuh", "nrm_multiscale_strip.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 

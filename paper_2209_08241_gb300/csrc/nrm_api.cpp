@@ -876,8 +876,10 @@ int nrm_estimate_points(nrm_handle* h, const void* depth, void* normals, uint8_t
   return estimate_single(h, depth, normals, valid, points, cuda_stream);
 }
 
-// The frames of a batched forward (or multi-scale) call, in two parts: those
-// that a strip kernel takes, then the rest, each with its own work list.
+// The frames of a batched forward (or multi-scale) call, in two parts, each with
+// its own work list: those that the strip kernel for aligned frames takes, then
+// the rest, which a forward call gives to the strip kernel for any alignment
+// (loader warps in place of TMA) or else to the tiled kernel.
 namespace {
 
 struct BatchPart {
@@ -886,15 +888,16 @@ struct BatchPart {
   int stat_tiles = 0;    // tiles in the handle's geometry (nrm_stats)
   int tile_y = 0;
   bool u16 = true;       // uint16 frames only
+  bool strip = false;    // taken by a strip kernel
 };
 
 // How a call splits its frames: the halo of its tiles, whether a strip kernel
-// may take frames (of tiles kStripX x strip_y), the tiles of the other kernel,
+// may take frames , the tiles of the other kernel,
 // and for multi-scale calls K and the divisor q of the form (1 or 4).
 struct BatchPlan {
   int halo;
   bool strip;
-  int strip_y;
+  int strip_y, any_y;   // rows of a tile of the strip kernel for aligned frames, for any
   int tile_x, tile_y;
   int scales = 0;
   double q = 4.0;
@@ -907,47 +910,55 @@ bool strip_handle(const nrm_handle* h) {
          c.ctas_per_sm == d.ctas_per_sm && h->p.alpha <= nrm::kStripMaxAlpha;
 }
 
-// True if a strip kernel can take frame f: whole vectors of four pixels to the
-// right edge, outputs on the alignment of the vector stores, and depth rows
-// that TMA can address (make_desc then decides by encoding the map).
-bool strip_frame(const nrm_handle* h, const nrm_frame& f, const BatchPlan& plan) {
-  if (!plan.strip || f.points) return false;
-  const uintptr_t na = h->p.out_dtype == NRM_OUT_OCT16 ? 16 : 32;
-  const int eb = f.in_dtype == NRM_IN_U16_MM ? 2 : 4;
-  if (f.in_dtype == NRM_IN_U16_MM) {
-    // The strip kernels leave out the test q >= FLT_MIN for uint16: with every
-    // depth >= 1 unit n . ray is at least pmin, and so q >= pmin^2 / |ray|^2.
-    const double s = h->p.depth_scale, a = plan.scales ? 1.0 : (double)h->p.alpha;
-    const double pmin = a * a / (f.K.fx * f.K.fy) * s * s / std::max(plan.scales, 1);
-    const double u = (std::fabs(f.K.cx) + f.W) / f.K.fx, v = (std::fabs(f.K.cy) + f.H) / f.K.fy;
-    if (!(pmin * pmin / (1.0 + u * u + v * v) >= 4.0 * 1.17549435e-38)) return false;
-  }
-  return f.W % 4 == 0 && f.out_pitch % 4 == 0 && (uintptr_t)f.normals % na == 0 && (uintptr_t)f.valid % 4 == 0 &&
-         (uintptr_t)f.depth % 16 == 0 && (f.depth_pitch * eb) % 16 == 0;
+// True if q >= FLT_MIN for every valid pixel of a uint16 frame, which the strip
+// kernels do not test: with every depth >= 1 unit n . ray is at least pmin, and so
+// q >= pmin^2 / |ray|^2. (float32 depth has no such bound; there they test q.)
+bool strip_domain(const nrm_handle* h, const nrm_frame& f, const BatchPlan& plan) {
+  if (f.in_dtype != NRM_IN_U16_MM) return true;
+  const double s = h->p.depth_scale, a = plan.scales ? 1.0 : (double)h->p.alpha;
+  const double pmin = a * a / (f.K.fx * f.K.fy) * s * s / std::max(plan.scales, 1);
+  const double u = (std::fabs(f.K.cx) + f.W) / f.K.fx, v = (std::fabs(f.K.cy) + f.H) / f.K.fy;
+  return pmin * pmin / (1.0 + u * u + v * v) >= 4.0 * 1.17549435e-38;
 }
 
-// Descriptors of the n frames into fd: the strip kernel's from the front, the
+// True if the strip kernel for aligned frames can take frame f: whole vectors of
+// four pixels to the right edge, outputs on the alignment of the vector stores,
+// and depth rows that TMA can address (make_desc then decides by encoding the map).
+bool strip_aligned(const nrm_handle* h, const nrm_frame& f, const BatchPlan& plan) {
+  const uintptr_t na = h->p.out_dtype == NRM_OUT_OCT16 ? 16 : 32;
+  const int eb = f.in_dtype == NRM_IN_U16_MM ? 2 : 4;
+  return plan.strip && strip_domain(h, f, plan) && f.W % 4 == 0 && f.out_pitch % 4 == 0 &&
+         (uintptr_t)f.normals % na == 0 && (uintptr_t)f.valid % 4 == 0 && (uintptr_t)f.depth % 16 == 0 &&
+         (f.depth_pitch * eb) % 16 == 0;
+}
+
+// Descriptors of the n frames into fd: the aligned ones from the front, the
 // others from the back. Empty frames are left out.
 void split_batch(const nrm_handle* h, const nrm_frame* frames, int n, const BatchPlan& plan, FrameDesc* fd,
                  BatchPart (&part)[2]) {
+  bool any = plan.strip && plan.scales == 0;  // the rest goes to the strip kernel for any alignment
+  for (int i = 0; i < n; ++i) any = any && ((long long)frames[i].H * frames[i].W == 0 || strip_domain(h, frames[i], plan));
+  const int rest_x = any ? nrm::kStripX : plan.tile_x, rest_y = any ? plan.any_y : plan.tile_y;
+  part[0].strip = true;
+  part[1].strip = any;
   part[0].tile_y = plan.strip_y;
-  part[1].tile_y = plan.tile_y;
+  part[1].tile_y = rest_y;
   int front = 0, back = n;
   for (int i = 0; i < n; ++i) {
     const nrm_frame& f = frames[i];
     if ((long long)f.H * f.W == 0) continue;
     const int eb = f.in_dtype == NRM_IN_U16_MM ? 2 : 4;
-    bool strip = strip_frame(h, f, plan);
-    if (strip) {
+    bool aligned = strip_aligned(h, f, plan);
+    if (aligned) {
       make_desc(&fd[front], f.depth, f.normals, f.valid, f.H, f.W, f.depth_pitch, f.out_pitch, f.K, f.in_dtype, h->p,
                 nrm::kStripX, plan.strip_y, nrm::kStripX + 2 * nrm::pad_x(plan.halo, eb),
                 plan.strip_y + 2 * plan.halo);
-      strip = fd[front].use_tma != 0;
+      aligned = fd[front].use_tma != 0;
     }
-    FrameDesc* d = strip ? &fd[front++] : &fd[--back];
-    if (!strip)
+    FrameDesc* d = aligned ? &fd[front++] : &fd[--back];
+    if (!aligned)
       make_desc(d, f.depth, f.normals, f.valid, f.H, f.W, f.depth_pitch, f.out_pitch, f.K, f.in_dtype, h->p,
-                plan.tile_x, plan.tile_y, plan.tile_x + 2 * nrm::pad_x(plan.halo, eb), plan.tile_y + 2 * plan.halo);
+                rest_x, rest_y, rest_x + 2 * nrm::pad_x(plan.halo, eb), rest_y + 2 * plan.halo);
     if (plan.scales) {
       // Multi-scale: per-frame bases; the kernel scales them by alpha_i (a, b) and
       // alpha_i^2 (c).
@@ -956,7 +967,7 @@ void split_batch(const nrm_handle* h, const nrm_frame* frames, int n, const Batc
       d->b = (float)(sc * sc / (plan.q * f.K.fx * plan.scales));
       d->c = (float)(sc * sc / (plan.q * f.K.fx * f.K.fy * plan.scales));
     }
-    BatchPart& p = part[strip ? 0 : 1];
+    BatchPart& p = part[aligned ? 0 : 1];
     p.u16 = p.u16 && f.in_dtype == NRM_IN_U16_MM;
     p.tiles += d->tiles_x * ((f.H + p.tile_y - 1) / p.tile_y);
     p.stat_tiles += ((f.W + h->cfg.tile_x - 1) / h->cfg.tile_x) * ((f.H + h->cfg.tile_y - 1) / h->cfg.tile_y);
@@ -967,7 +978,8 @@ void split_batch(const nrm_handle* h, const nrm_frame* frames, int n, const Batc
 }
 
 BatchPlan forward_plan(const nrm_handle* h) {
-  return {h->p.alpha, strip_handle(h), nrm::strip_tile_y(h->p.out_dtype), h->cfg.tile_x, h->cfg.tile_y};
+  return {h->p.alpha,    strip_handle(h), nrm::strip_tile_y(h->p.out_dtype, true), nrm::strip_tile_y(h->p.out_dtype, false),
+          h->cfg.tile_x, h->cfg.tile_y};
 }
 
 // One part's header and tile offsets (tile_begin: n + 1 entries).
@@ -1000,11 +1012,11 @@ void* pack_part(nrm_handle* h, const BatchPart& p, FrameDesc* fd) {
 
 // Launches one part: its descriptors as the kernel parameter (param_block) or
 // in the device block that args points to.
-int launch_part(nrm_handle* h, bool strip, const nrm::BatchArgs& args, const BatchPart& p, void* param_block,
+int launch_part(nrm_handle* h, bool aligned, const nrm::BatchArgs& args, const BatchPart& p, void* param_block,
                 cudaStream_t st) {
   nrm::Globals g = make_globals(h);
-  if (strip) {
-    NRM_CUDA(nrm::launch_forward_strip(args, g, h->p.out_dtype, p.tiles, p.u16, st, param_block),
+  if (p.strip) {
+    NRM_CUDA(nrm::launch_forward_strip(args, g, h->p.out_dtype, p.tiles, p.u16, aligned, st, param_block),
              "launch strip kernel");
     return NRM_OK;
   }
@@ -1043,7 +1055,7 @@ static int estimate_batched_param(nrm_handle* h, const nrm_frame* frames, int n,
       return fail(NRM_ERR_UNSUPPORTED, "frame %d: point clouds are not written during stream capture", i);
   std::vector<FrameDesc>& fd = h->scratch_desc;
   if (fd.size() < (size_t)n) fd.resize((size_t)n);
-  BatchPart part[2];  // strip kernel, tiled kernel
+  BatchPart part[2];
   split_batch(h, frames, n, forward_plan(h), fd.data(), part);
   Slot* s = nullptr;
   if (!capture) {
@@ -1603,7 +1615,7 @@ int nrm_estimate_batched_multiscale(nrm_handle* h, const nrm_frame* frames, int 
   }
   bool consecutive = ms.K >= 2 && ms.K <= nrm::kMsStripMaxScales;
   for (int i = 0; i < ms.K; ++i) consecutive = consecutive && ms.alpha[i] == i + 1;
-  const BatchPlan plan = {ms.alpha_max, consecutive, nrm::ms_strip_tile_y(), TX, TY, ms.K,
+  const BatchPlan plan = {ms.alpha_max, consecutive, nrm::ms_strip_tile_y(), 0, TX, TY, ms.K,
                           scales->form == NRM_MS_QUAD ? 4.0 : 1.0};
   const nrm::Globals g = make_globals(h);
   std::vector<FrameDesc>& fd = h->scratch_desc;

@@ -21,6 +21,14 @@
 // Batches of few tiles take all the CTAs that fit: there the ramp counts, not the
 // steady state (16 x 640x480 float32: 18.8 us with 3 CTAs per SM, 20.9 with one;
 // 2 x 1080p 15.2 against 16.0, 4 x 1080p 30.7 against 29.6 us).
+//
+// Frames of any alignment (loader warps instead of TMA; nothing comes near
+// saturating HBM): as many CTAs as fit, 6 compute and 4 loader warps (octahedral
+// 4 and 2). 64 x 1921x1081: uint16 -> float4 487 us (76 %; the tiled kernel's plain
+// loads 1092), float32 -> float4 503 (1181), uint16 -> half4 484 (818), octahedral
+// 381 (789); two 3001x2001 uint16 frames 44 us (75). [6 loader warps 521 / 520 /
+// 539; 4 compute warps, 3 CTAs 488 / 504 / 515; 12 and 16 compute warps, 1 CTA 650 /
+// 685 / 566.]
 #include <algorithm>
 #include <atomic>
 
@@ -34,49 +42,33 @@ constexpr int kStripFewTiles = 12;  // tiles per SM
 
 int strip_stages(int out_dtype, bool u16) { return out_dtype == NRM_OUT_OCT16 ? (u16 ? 4 : 2) : 3; }
 
-template <int OUT, bool SECANT>
-const void* strip_kernel_for(int alpha, bool param) {
-  switch (alpha) {
-    case 1: return param ? (const void*)fwd_strip_param_kernel<OUT, SECANT, 1> : (const void*)fwd_strip_kernel<OUT, SECANT, 1>;
-    case 2: return param ? (const void*)fwd_strip_param_kernel<OUT, SECANT, 2> : (const void*)fwd_strip_kernel<OUT, SECANT, 2>;
-    case 3: return param ? (const void*)fwd_strip_param_kernel<OUT, SECANT, 3> : (const void*)fwd_strip_kernel<OUT, SECANT, 3>;
-    case 4: return param ? (const void*)fwd_strip_param_kernel<OUT, SECANT, 4> : (const void*)fwd_strip_kernel<OUT, SECANT, 4>;
-    default: return nullptr;
-  }
-}
-
-const void* strip_kernel(int out_dtype, bool secant, int alpha, bool param) {
-  switch (out_dtype) {
-    case NRM_OUT_F32X4: return secant ? strip_kernel_for<NRM_OUT_F32X4, true>(alpha, param) : strip_kernel_for<NRM_OUT_F32X4, false>(alpha, param);
-    case NRM_OUT_F16X4: return secant ? strip_kernel_for<NRM_OUT_F16X4, true>(alpha, param) : strip_kernel_for<NRM_OUT_F16X4, false>(alpha, param);
-    case NRM_OUT_OCT16: return secant ? strip_kernel_for<NRM_OUT_OCT16, true>(alpha, param) : strip_kernel_for<NRM_OUT_OCT16, false>(alpha, param);
-    default: return nullptr;
-  }
-}
-
 }  // namespace
 
+template const void* strip_kernel<true>(int, bool, int, bool);
+
 cudaError_t launch_forward_strip(const BatchArgs& args, const Globals& g, int out_dtype, int total_tiles, bool u16,
-                                 cudaStream_t stream, const void* param_block) {
+                                 bool aligned, cudaStream_t stream, const void* param_block) {
   const bool param = param_block != nullptr;
   const bool secant = g.mask_mode == NRM_MASK_SECANT;
-  const void* fn = strip_kernel(out_dtype, secant, g.alpha, param);
+  const void* fn = aligned ? strip_kernel<true>(out_dtype, secant, g.alpha, param)
+                           : strip_kernel<false>(out_dtype, secant, g.alpha, param);
   if (!fn) return cudaErrorInvalidValue;
   const int eb = u16 ? 2 : 4;
   const int stages = strip_stages(out_dtype, u16);
-  const unsigned smem = strip_smem_bytes(strip_tile_y(out_dtype), g.alpha, eb, stages);
-  const int threads = strip_threads(out_dtype);
+  const unsigned rowbuf = aligned ? 0 : strip_warps(out_dtype, aligned) * strip_rowbuf(out_dtype);
+  const unsigned smem = strip_smem_bytes(strip_tile_y(out_dtype, aligned), g.alpha, eb, stages) + rowbuf;
+  const int threads = strip_block(out_dtype, aligned);
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
   // CTAs of this kernel and staging size that fit an SM, found once, and the SMs.
-  static std::atomic<int> fit[3][2][kStripMaxAlpha + 1][2][2][64];
+  static std::atomic<int> fit[2][3][2][kStripMaxAlpha + 1][2][2][64];
   static std::atomic<int> sm_count[64];
-  std::atomic<int>& occ = fit[out_dtype][secant][g.alpha][param][u16][dev];
+  std::atomic<int>& occ = fit[aligned][out_dtype][secant][g.alpha][param][u16][dev];
   if (occ.load() == 0) {
     int sms = 0, n = 0;
-    e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)strip_smem_bytes(strip_tile_y(out_dtype), kStripMaxAlpha, 4, 3));
+    e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(strip_smem_bytes(strip_tile_y(out_dtype, aligned), kStripMaxAlpha, 4, 3) + rowbuf));
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fn, threads, smem);
     if (e != cudaSuccess) return e;
@@ -87,11 +79,11 @@ cudaError_t launch_forward_strip(const BatchArgs& args, const Globals& g, int ou
   const int sms = sm_count[dev].load();
   // One CTA per SM once an SM has more than kStripFewTiles tiles (float4 and
   // half4; see the file comment), else as many as fit.
-  const int per_sm = out_dtype != NRM_OUT_OCT16 && total_tiles > kStripFewTiles * sms ? 1 : occ.load();
+  const int per_sm = aligned && out_dtype != NRM_OUT_OCT16 && total_tiles > kStripFewTiles * sms ? 1 : occ.load();
   const int ctas = per_sm * sms;
   BatchArgs a = args;
   a.stages = stages;
-  a.stage_bytes = strip_stage_bytes(strip_tile_y(out_dtype), g.alpha, eb);
+  a.stage_bytes = strip_stage_bytes(strip_tile_y(out_dtype, aligned), g.alpha, eb);
   Globals gg = g;
   const dim3 grid(std::min(total_tiles, ctas)), block(threads);
   if (param) {

@@ -1,6 +1,7 @@
 // The strip kernels: batched forward pass (arXiv 2209.08241, Section 3.1
 // Eq. 4-6 and the Section 3.2 mask) for frames whose rows TMA can load and
-// whose outputs take whole-vector stores, for pixel distance ALPHA = 1..4.
+// whose outputs take whole-vector stores (ALIGNED), or for frames of any pitch
+// and alignment, for pixel distance ALPHA = 1..4.
 //
 // One CTA is strip_warps compute warps and a producer warp. The producer walks
 // the CTA's tiles (128 x strip_tile_y pixels) of the batch's work list and, per
@@ -160,12 +161,105 @@ __device__ __forceinline__ void strip_codes(float2 nx, float2 ny, float2 nz, uin
   cb = __byte_perm(__float_as_uint(x.y), __float_as_uint(y.y), 0x5410);
 }
 
-// The normals (or codes) and mask bytes of a lane's four pixels: np, mp point at
-// the first one's; k[i] says whether pixel i is valid.
+// A row of one band written at any alignment: the lanes' results go to the warp's
+// row buffer at the offset that the row has in memory modulo 16 bytes (mask:
+// modulo 4), and the warp then copies whole 16-byte (4-byte) units with
+// consecutive lanes, the ragged units at the ends element by element. (One store
+// per pixel straight from the lanes, 4 pixels apart, writes part of a 32-byte
+// sector at a time: 64 x 1921x1081 uint16 -> float4 745 us, half4 755 us with one
+// CTA per SM; through the buffer 646 and 492 us, with two CTAs 487 and 484. The
+// octahedral codes, whose ragged ends would be three of four elements, are faster
+// straight from the lanes: 381 against 581 us.) float4: units are pixels, stored
+// with their index's low bits XORed by bits 3-5, so that neither side has bank
+// conflicts.
+constexpr int kRowBufMask = 160;  // the mask's part of a row buffer
+NRM_HD constexpr int strip_rowbuf(int out_dtype) {
+  return kRowBufMask + (out_dtype == NRM_OUT_F32X4 ? 2048 : out_dtype == NRM_OUT_F16X4 ? 1040 : 528);
+}
+
+// Copies bytes [m, m + len) of buf to the same offsets from base, units of U
+// bytes by consecutive lanes, elements of E bytes at the ragged ends.
+template <int U, int E, int BYTES, typename Unit, typename Elem>
+__device__ __forceinline__ void copy_out(const unsigned char* buf, unsigned char* base, int m, int len) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int k = 0; k < (BYTES / U + 1 + 31) / 32; ++k) {
+    const int b = (lane + 32 * k) * U;
+    if (b >= m && b + U <= m + len) {
+      __stcs(reinterpret_cast<Unit*>(base + b), NRM_LDS(Unit, reinterpret_cast<const Unit*>(buf + b)));
+    } else if (b + U > m && b < m + len) {
+#pragma unroll
+      for (int e = 0; e < U; e += E)
+        if (b + e >= m && b + e < m + len)
+          __stcs(reinterpret_cast<Elem*>(base + b + e), NRM_LDS(Elem, reinterpret_cast<const Elem*>(buf + b + e)));
+    }
+  }
+}
+
 template <int OUT>
+__device__ __forceinline__ void store_row(const uint32_t* w, uint32_t mbits, unsigned char* np, uint8_t* mp, int n,
+                                          unsigned char* buf, [[maybe_unused]] const StripInfo& f) {
+  constexpr int BPP = OUT == NRM_OUT_F32X4 ? 16 : OUT == NRM_OUT_F16X4 ? 8 : 4;
+  const int lane = threadIdx.x & 31;
+  unsigned char* row = np - 4 * lane * BPP;  // the row's first pixel in this tile
+  uint8_t* mrow = mp - 4 * lane;
+  const int count = min(f.cols, kStripX);
+#ifdef NRM_DEBUG_CHECKS
+  if (!(dbg_gmem_ok(row, count * BPP, f.normals0, f.nlen, "strip normals", __LINE__) &&
+        dbg_gmem_ok(mrow, count, f.valid0, f.mlen, "strip mask", __LINE__)))
+    return;
+#endif
+  (void)n;
+  unsigned char* nbuf = buf + kRowBufMask;
+  const int mm = (int)(reinterpret_cast<uintptr_t>(mrow) & 3);
+  __syncwarp();  // the previous row has left the buffer
+  if (mm == 0) {
+    NRM_STS(reinterpret_cast<uint32_t*>(buf) + lane, mbits);
+  } else {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) NRM_STS(buf + mm + 4 * lane + i, (unsigned char)(mbits >> (8 * i)));
+  }
+  if constexpr (OUT == NRM_OUT_F32X4) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int c = 4 * lane + i;
+      NRM_STS(reinterpret_cast<uint4*>(nbuf) + (c ^ ((c >> 3) & 7)),
+              make_uint4(w[4 * i], w[4 * i + 1], w[4 * i + 2], w[4 * i + 3]));
+    }
+    __syncwarp();
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int c = lane + 32 * k;
+      if (c < count)
+        __stcs(reinterpret_cast<uint4*>(row) + c, NRM_LDS(uint4, reinterpret_cast<const uint4*>(nbuf) + (c ^ ((c >> 3) & 7))));
+    }
+  } else {
+    const int m = (int)(reinterpret_cast<uintptr_t>(row) & 15);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      if constexpr (OUT == NRM_OUT_F16X4)
+        NRM_STS(reinterpret_cast<uint2*>(nbuf + m) + 4 * lane + i, make_uint2(w[2 * i], w[2 * i + 1]));
+      else
+        NRM_STS(reinterpret_cast<uint32_t*>(nbuf + m) + 4 * lane + i, w[i]);
+    }
+    __syncwarp();
+    if constexpr (OUT == NRM_OUT_F16X4)
+      copy_out<16, 8, 1024, uint4, uint2>(nbuf, row - m, m, count * BPP);
+    else
+      copy_out<16, 4, 512, uint4, uint32_t>(nbuf, row - m, m, count * BPP);
+  }
+  copy_out<4, 1, 128, uint32_t, uint8_t>(buf, mrow - mm, mm, count);
+}
+
+// The normals (or codes) and mask bytes of a lane's four pixels: np, mp point at
+// the first one's; k[i] says whether pixel i is valid; n > 0 of them lie in the
+// frame. ALIGNED: whole vectors, straight to memory (n >= 4); else through the
+// warp's row buffer (store_row).
+template <int OUT, bool ALIGNED>
 __device__ __forceinline__ void strip_store(const float2 (&nx)[2], const float2 (&ny)[2], const float2 (&nz)[2],
                                             const float2 (&q)[2], const bool (&k)[4], unsigned char* np, uint8_t* mp,
-                                            bool on, [[maybe_unused]] const StripInfo& f) {
+                                            int n, [[maybe_unused]] unsigned char* buf,
+                                            [[maybe_unused]] const StripInfo& f) {
   [[maybe_unused]] constexpr int BPP = OUT == NRM_OUT_F32X4 ? 16 : OUT == NRM_OUT_F16X4 ? 8 : 4;
   const uint32_t mbits =
       (k[0] ? 1u : 0u) | (k[1] ? 0x100u : 0u) | (k[2] ? 0x10000u : 0u) | (k[3] ? 0x1000000u : 0u);
@@ -200,29 +294,46 @@ __device__ __forceinline__ void strip_store(const float2 (&nx)[2], const float2 
       }
     }
   }
+  if constexpr (ALIGNED) {
 #ifdef NRM_DEBUG_CHECKS
-  if (on && !(dbg_gmem_ok(np, 4 * BPP, f.normals0, f.nlen, "strip normals", __LINE__) &&
-              dbg_gmem_ok(mp, 4, f.valid0, f.mlen, "strip mask", __LINE__)))
-    return;
+    if (n > 0 && !(dbg_gmem_ok(np, 4 * BPP, f.normals0, f.nlen, "strip normals", __LINE__) &&
+                   dbg_gmem_ok(mp, 4, f.valid0, f.mlen, "strip mask", __LINE__)))
+      return;
 #endif
-  if (on) {
-    if constexpr (OUT == NRM_OUT_F32X4) {
-      store32(np, w[0], w[1], w[2], w[3], w[4], w[5], w[6], w[7]);
-      store32(np + 32, w[8], w[9], w[10], w[11], w[12], w[13], w[14], w[15]);
-    } else if constexpr (OUT == NRM_OUT_F16X4) {
-      store32(np, w[0], w[1], w[2], w[3], w[4], w[5], w[6], w[7]);
-    } else {
-      __stcs(reinterpret_cast<uint4*>(np), make_uint4(w[0], w[1], w[2], w[3]));
+    if (n > 0) {
+      if constexpr (OUT == NRM_OUT_F32X4) {
+        store32(np, w[0], w[1], w[2], w[3], w[4], w[5], w[6], w[7]);
+        store32(np + 32, w[8], w[9], w[10], w[11], w[12], w[13], w[14], w[15]);
+      } else if constexpr (OUT == NRM_OUT_F16X4) {
+        store32(np, w[0], w[1], w[2], w[3], w[4], w[5], w[6], w[7]);
+      } else {
+        __stcs(reinterpret_cast<uint4*>(np), make_uint4(w[0], w[1], w[2], w[3]));
+      }
+      __stcs(reinterpret_cast<unsigned int*>(mp), mbits);
     }
-    __stcs(reinterpret_cast<unsigned int*>(mp), mbits);
+  } else if constexpr (OUT == NRM_OUT_OCT16) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      if (i >= n) break;
+#ifdef NRM_DEBUG_CHECKS
+      if (!(dbg_gmem_ok(np + i * BPP, BPP, f.normals0, f.nlen, "strip normals", __LINE__) &&
+            dbg_gmem_ok(mp + i, 1, f.valid0, f.mlen, "strip mask", __LINE__)))
+        return;
+#endif
+      __stcs(reinterpret_cast<uint32_t*>(np) + i, w[i]);
+      __stcs(mp + i, (uint8_t)(mbits >> (8 * i)));
+    }
+  } else {
+    store_row<OUT>(w, mbits, np, mp, n, buf, f);
   }
 }
 
 // One band: strip_rows(OUT) rows of 128 columns from the staged box S (its first
 // row is ALPHA above the band's, its column PAD the tile's first).
-template <int OUT, bool SECANT, int ALPHA, typename InT>
+template <int OUT, bool SECANT, int ALPHA, bool ALIGNED, typename InT>
 __device__ __forceinline__ void strip_band(const InT* __restrict__ S, const float4* __restrict__ ctab,
-                                           const float4* __restrict__ rtab, const StripInfo& f, int band, float tau2) {
+                                           const float4* __restrict__ rtab, const StripInfo& f, int band, float tau2,
+                                           [[maybe_unused]] unsigned char* buf) {
   constexpr int EB = (int)sizeof(InT);
   constexpr int PAD = EB == 2 ? 8 : 4;        // pad_x(ALPHA, EB) for ALPHA <= 4
   constexpr int SP = kStripX + 2 * PAD;       // staged row pitch
@@ -236,7 +347,7 @@ __device__ __forceinline__ void strip_band(const InT* __restrict__ S, const floa
   const float2 A = f2(f.a, f.a), B = f2(f.b, f.b), C = f2(f.c, f.c), T = f2(tau2, tau2);
   const int row0 = band * ROWS;
   const int rows = min(ROWS, f.rows - row0);
-  const bool on = 4 * lane < f.cols;
+  const int n = f.cols - 4 * lane;  // of the lane's pixels, those in the frame
   const InT* base = S + row0 * SP + PAD + 4 * lane;
 #pragma unroll 1
   for (int c = 0; c < ALPHA; ++c) {
@@ -282,7 +393,7 @@ __device__ __forceinline__ void strip_band(const InT* __restrict__ S, const floa
                                   q[0], keep[0], keep[1]);
       strip_pair<SECANT, EB == 2>(m1, r1, b1, l1, u1, A, B, C, T, tau2, nu1[1], ku[1], nv1, kv, nx[1], ny[1], nz[1],
                                   q[1], keep[2], keep[3]);
-      strip_store<OUT>(nx, ny, nz, q, keep, np, mp, on, f);
+      strip_store<OUT, ALIGNED>(nx, ny, nz, q, keep, np, mp, n, buf, f);
       np += ALPHA * f.out_pitch * BPP;
       mp += ALPHA * f.out_pitch;
       u0 = m0;
@@ -293,12 +404,101 @@ __device__ __forceinline__ void strip_band(const InT* __restrict__ S, const floa
   }
 }
 
+// The record of the tile at (gx0, gy0) of frame fd.
+template <int BPP>
+__device__ __forceinline__ void write_record(StripInfo* dst, const FrameDesc& fd, float sign, int gx0, int gy0) {
+  StripInfo si;
+  si.a = -sign * fd.a;
+  si.b = -sign * fd.b;
+  si.c = sign * fd.c;
+  si.u16 = fd.in_dtype == NRM_IN_U16_MM;
+  si.out_pitch = fd.out_pitch;
+  si.normals = reinterpret_cast<unsigned char*>(fd.normals) + ((long long)gy0 * fd.out_pitch + gx0) * BPP;
+  si.valid = fd.valid + (long long)gy0 * fd.out_pitch + gx0;
+  si.cols = fd.W - gx0;
+  si.rows = fd.H - gy0;
+#ifdef NRM_DEBUG_CHECKS
+  si.normals0 = fd.normals;
+  si.valid0 = fd.valid;
+  si.nlen = dbg_span(fd.H, fd.W, fd.out_pitch, BPP);
+  si.mlen = dbg_span(fd.H, fd.W, fd.out_pitch, 1);
+#endif
+  NRM_STS(dst, si);
+}
+
+// The tile's column table, two float4 per lane, and row table (the terms of
+// emit_pair), by one warp.
+template <int TY>
+__device__ __forceinline__ void write_tables(float4* ctab, const FrameDesc& fd, int gx0, int gy0) {
+  const int lane = threadIdx.x & 31;
+  const float cx = fd.cx, cy = fd.cy, ifx = fd.inv_fx, ify = fd.inv_fy;
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const float ua = ((float)(gx0 + 4 * lane + 2 * h) - cx) * ifx;
+    const float ub = ((float)(gx0 + 4 * lane + 2 * h + 1) - cx) * ifx;
+    NRM_STS(ctab + 2 * lane + h, make_float4(-ua, -ub, fmaf(ua, ua, 1.0f), fmaf(ub, ub, 1.0f)));
+  }
+  for (int r = lane; r < TY; r += 32) {
+    const float v1 = ((float)(gy0 + r) - cy) * ify;
+    NRM_STS(ctab + kStripX / 2 + r, make_float4(-v1, -v1, v1 * v1, v1 * v1));
+  }
+}
+
+// Loads the rows warp, warp + LOADERS, ... of the halo box of a frame without a
+// usable tensor map into its staged layout, in plain loads of one depth per lane
+// (a row may start on any element); 0 outside the frame. These loads are bound by
+// latency, so up to BATCH rows, five loads each (128 columns, then the halo
+// columns), are in flight before the first is stored.
+template <int HALO, int TY, int LOADERS, typename InT>
+__device__ __forceinline__ void load_box(InT* __restrict__ st, const FrameDesc& fd, int gx0, int gy0, int warp) {
+  constexpr int PAD = sizeof(InT) == 2 ? 8 : (HALO + 3) / 4 * 4;
+  constexpr int SP = kStripX + 2 * PAD;
+  constexpr int ROWS = TY + 2 * HALO;
+  constexpr int PER_WARP = (ROWS + LOADERS - 1) / LOADERS;
+  constexpr int BATCH = PER_WARP < 8 ? PER_WARP : 8;
+  const int lane = threadIdx.x & 31;
+  const InT* src = reinterpret_cast<const InT*>(fd.depth);
+  const int H = fd.H, W = fd.W;
+  const long long pitch = fd.depth_pitch;
+  // The lane's five columns of a row; the last is a halo column (lanes < 2 HALO).
+  int col[5];
+  bool in[5];
+#pragma unroll
+  for (int k = 0; k < 5; ++k) {
+    col[k] = k < 4 ? lane + 32 * k : lane < HALO ? lane - HALO : kStripX + lane - HALO;
+    in[k] = (k < 4 || lane < 2 * HALO) && gx0 + col[k] >= 0 && gx0 + col[k] < W;
+  }
+#pragma unroll 1
+  for (int r0 = warp; r0 < ROWS; r0 += BATCH * LOADERS) {
+    InT v[BATCH][5];
+#pragma unroll
+    for (int b = 0; b < BATCH; ++b) {
+      const int y = gy0 - HALO + r0 + b * LOADERS;
+      const bool row = r0 + b * LOADERS < ROWS && y >= 0 && y < H;
+      const InT* p = src + y * pitch + gx0;
+#pragma unroll
+      for (int k = 0; k < 5; ++k) v[b][k] = row && in[k] ? __ldg(p + col[k]) : InT(0);
+    }
+#pragma unroll
+    for (int b = 0; b < BATCH; ++b) {
+      const int r = r0 + b * LOADERS;
+      if (r >= ROWS) break;
+      InT* q = st + r * SP + PAD;
+#pragma unroll
+      for (int k = 0; k < 5; ++k)
+        if (k < 4 || lane < 2 * HALO) NRM_STS(q + col[k], v[b][k]);
+    }
+  }
+}
+
 // The pipeline of a strip kernel: tiles of kStripX x (ROWS x WARPS) pixels with a halo
 // of HALO; band(stage, column table, row table, record, warp) computes one
 // band, its stage pointer typed by the frame's depth type. RING: the descriptors
 // are in global memory written by the host (each tensor map is fenced before
-// its first use), else in kernel-parameter space.
-template <int OUT, int HALO, int ROWS, int WARPS, bool RING, class Band>
+// its first use), else in kernel-parameter space. LOADERS = 0: one producer warp
+// and TMA; LOADERS > 0: that many warps fill the stages with load_box (any pitch
+// and alignment).
+template <int OUT, int HALO, int ROWS, int WARPS, int LOADERS, bool RING, class Band>
 __device__ __forceinline__ void strip_pipeline(const BatchArgs& args, const Globals& g, const Band& band) {
   extern __shared__ __align__(128) unsigned char smem[];
   constexpr int BPP = OUT == NRM_OUT_F32X4 ? 16 : OUT == NRM_OUT_F16X4 ? 8 : 4;
@@ -317,14 +517,14 @@ __device__ __forceinline__ void strip_pipeline(const BatchArgs& args, const Glob
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (threadIdx.x == 0) {
     for (int s = 0; s < S; ++s) {
-      mbar_init(smem_u32(&full[s]), 2);
+      mbar_init(smem_u32(&full[s]), LOADERS ? LOADERS : 2);
       mbar_init(smem_u32(&empty[s]), WARPS);
     }
     fence_barrier_init();
   }
   __syncthreads();
 
-  if (warp == WARPS) {
+  if (warp >= WARPS) {
     // ------------------------------------------------------------ producer
     int cur = 0, fenced = -1, s = 0;
     uint32_t parity = 1;
@@ -346,6 +546,17 @@ __device__ __forceinline__ void strip_pipeline(const BatchArgs& args, const Glob
       const int gx0 = (local - ty * tiles_x) * kStripX, gy0 = ty * TY;
       const int eb = fd->in_dtype == NRM_IN_U16_MM ? 2 : 4;
       unsigned char* st = smem + (size_t)s * SB;
+      if constexpr (LOADERS > 0) {
+        const int w = warp - WARPS;
+        if (eb == 2)
+          load_box<HALO, TY, LOADERS>(reinterpret_cast<uint16_t*>(st), *fd, gx0, gy0, w);
+        else
+          load_box<HALO, TY, LOADERS>(reinterpret_cast<float*>(st), *fd, gx0, gy0, w);
+        if (w == 0) {
+          if (lane == 0) write_record<BPP>(reinterpret_cast<StripInfo*>(st + SB - TB), *fd, g.sign, gx0, gy0);
+          write_tables<TY>(reinterpret_cast<float4*>(st + SB - TB + kStripInfoBytes), *fd, gx0, gy0);
+        }
+      } else {
       if (lane == 0) {
         if (RING && cur != fenced) {
           fence_tensormap_acquire(&fd->tmap);
@@ -355,36 +566,9 @@ __device__ __forceinline__ void strip_pipeline(const BatchArgs& args, const Glob
         const uint32_t bar = smem_u32(&full[s]);
         mbar_arrive_expect_tx(bar, (uint32_t)((kStripX + 2 * padx) * (TY + 2 * HALO) * eb));
         tma_load_2d(smem_u32(st), &fd->tmap, gx0 - padx, gy0 - HALO, bar);
-        StripInfo si;
-        si.a = -g.sign * fd->a;
-        si.b = -g.sign * fd->b;
-        si.c = g.sign * fd->c;
-        si.u16 = eb == 2;
-        si.out_pitch = fd->out_pitch;
-        si.normals = reinterpret_cast<unsigned char*>(fd->normals) + ((long long)gy0 * fd->out_pitch + gx0) * BPP;
-        si.valid = fd->valid + (long long)gy0 * fd->out_pitch + gx0;
-#ifdef NRM_DEBUG_CHECKS
-        si.normals0 = fd->normals;
-        si.valid0 = fd->valid;
-        si.nlen = dbg_span(fd->H, fd->W, fd->out_pitch, BPP);
-        si.mlen = dbg_span(fd->H, fd->W, fd->out_pitch, 1);
-#endif
-        si.cols = fd->W - gx0;
-        si.rows = fd->H - gy0;
-        NRM_STS(reinterpret_cast<StripInfo*>(st + SB - TB), si);
+        write_record<BPP>(reinterpret_cast<StripInfo*>(st + SB - TB), *fd, g.sign, gx0, gy0);
       }
-      // Column table, two float4 per lane, and row table: the terms of emit_pair.
-      float4* ctab = reinterpret_cast<float4*>(st + SB - TB + kStripInfoBytes);
-      const float cx = fd->cx, cy = fd->cy, ifx = fd->inv_fx, ify = fd->inv_fy;
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const float ua = ((float)(gx0 + 4 * lane + 2 * h) - cx) * ifx;
-        const float ub = ((float)(gx0 + 4 * lane + 2 * h + 1) - cx) * ifx;
-        NRM_STS(ctab + 2 * lane + h, make_float4(-ua, -ub, fmaf(ua, ua, 1.0f), fmaf(ub, ub, 1.0f)));
-      }
-      for (int r = lane; r < TY; r += 32) {
-        const float v1 = ((float)(gy0 + r) - cy) * ify;
-        NRM_STS(ctab + kStripX / 2 + r, make_float4(-v1, -v1, v1 * v1, v1 * v1));
+      write_tables<TY>(reinterpret_cast<float4*>(st + SB - TB + kStripInfoBytes), *fd, gx0, gy0);
       }
       __syncwarp();
       if (lane == 0) mbar_arrive(smem_u32(&full[s]));
@@ -420,27 +604,75 @@ __device__ __forceinline__ void strip_pipeline(const BatchArgs& args, const Glob
   }
 }
 
-template <int OUT, bool SECANT, int ALPHA, bool RING>
+// Loader warps of the kernels for frames of any alignment.
+NRM_HD constexpr int strip_loaders(int out_dtype) { return out_dtype == NRM_OUT_OCT16 ? 2 : 4; }
+
+template <int OUT, bool SECANT, int ALPHA, bool ALIGNED, bool RING>
 __device__ __forceinline__ void strip_forward(const BatchArgs& args, const Globals& g) {
-  strip_pipeline<OUT, ALPHA, strip_rows(OUT), strip_warps(OUT), RING>(
+  strip_pipeline<OUT, ALPHA, strip_rows(OUT), strip_warps(OUT, ALIGNED), ALIGNED ? 0 : strip_loaders(OUT), RING>(
       args, g, [&](const auto* S, const float4* ctab, const float4* rtab, const StripInfo& f, int warp) {
-        strip_band<OUT, SECANT, ALPHA>(S, ctab, rtab, f, warp, g.tau2);
+        extern __shared__ __align__(128) unsigned char smem[];
+        unsigned char* buf = smem + args.stages * (args.stage_bytes + 16) + warp * strip_rowbuf(OUT);
+        strip_band<OUT, SECANT, ALPHA, ALIGNED>(S, ctab, rtab, f, warp, g.tau2, buf);
       });
 }
 
-template <int OUT, bool SECANT, int ALPHA>
-__global__ void __launch_bounds__(strip_threads(OUT), OUT == NRM_OUT_OCT16 ? 4 : 1)
+NRM_HD constexpr int strip_block(int out_dtype, bool aligned) {
+  return (strip_warps(out_dtype, aligned) + (aligned ? 1 : strip_loaders(out_dtype))) * 32;
+}
+
+NRM_HD constexpr int strip_min_ctas(int out_dtype, bool aligned) {
+  return out_dtype == NRM_OUT_OCT16 ? (aligned ? 4 : 3) : aligned ? 1 : 2;
+}
+
+template <int OUT, bool SECANT, int ALPHA, bool ALIGNED>
+__global__ void __launch_bounds__(strip_block(OUT, ALIGNED), strip_min_ctas(OUT, ALIGNED))
     fwd_strip_param_kernel(const __grid_constant__ ParamBatch pb, const BatchArgs ring, const Globals g) {
   BatchArgs args = ring;
   args.hdr = &pb.hdr;
   args.tile_begin = pb.tile_begin;
   args.frames = pb.frames;
-  strip_forward<OUT, SECANT, ALPHA, false>(args, g);
+  strip_forward<OUT, SECANT, ALPHA, ALIGNED, false>(args, g);
 }
 
-template <int OUT, bool SECANT, int ALPHA>
-__global__ void __launch_bounds__(strip_threads(OUT), OUT == NRM_OUT_OCT16 ? 4 : 1) fwd_strip_kernel(const BatchArgs args, const Globals g) {
-  strip_forward<OUT, SECANT, ALPHA, true>(args, g);
+template <int OUT, bool SECANT, int ALPHA, bool ALIGNED>
+__global__ void __launch_bounds__(strip_block(OUT, ALIGNED), strip_min_ctas(OUT, ALIGNED))
+    fwd_strip_kernel(const BatchArgs args, const Globals g) {
+  strip_forward<OUT, SECANT, ALPHA, ALIGNED, true>(args, g);
 }
+
+// The kernel of one output type, or NULL (instantiated in a file per ALIGNED).
+template <int OUT, bool SECANT, bool ALIGNED>
+const void* strip_by_alpha(int alpha, bool param) {
+  switch (alpha) {
+    case 1: return param ? (const void*)fwd_strip_param_kernel<OUT, SECANT, 1, ALIGNED>
+                         : (const void*)fwd_strip_kernel<OUT, SECANT, 1, ALIGNED>;
+    case 2: return param ? (const void*)fwd_strip_param_kernel<OUT, SECANT, 2, ALIGNED>
+                         : (const void*)fwd_strip_kernel<OUT, SECANT, 2, ALIGNED>;
+    case 3: return param ? (const void*)fwd_strip_param_kernel<OUT, SECANT, 3, ALIGNED>
+                         : (const void*)fwd_strip_kernel<OUT, SECANT, 3, ALIGNED>;
+    case 4: return param ? (const void*)fwd_strip_param_kernel<OUT, SECANT, 4, ALIGNED>
+                         : (const void*)fwd_strip_kernel<OUT, SECANT, 4, ALIGNED>;
+    default: return nullptr;
+  }
+}
+
+template <bool ALIGNED>
+const void* strip_kernel(int out_dtype, bool secant, int alpha, bool param) {
+  switch (out_dtype) {
+    case NRM_OUT_F32X4:
+      return secant ? strip_by_alpha<NRM_OUT_F32X4, true, ALIGNED>(alpha, param)
+                    : strip_by_alpha<NRM_OUT_F32X4, false, ALIGNED>(alpha, param);
+    case NRM_OUT_F16X4:
+      return secant ? strip_by_alpha<NRM_OUT_F16X4, true, ALIGNED>(alpha, param)
+                    : strip_by_alpha<NRM_OUT_F16X4, false, ALIGNED>(alpha, param);
+    case NRM_OUT_OCT16:
+      return secant ? strip_by_alpha<NRM_OUT_OCT16, true, ALIGNED>(alpha, param)
+                    : strip_by_alpha<NRM_OUT_OCT16, false, ALIGNED>(alpha, param);
+    default: return nullptr;
+  }
+}
+extern template const void* strip_kernel<true>(int, bool, int, bool);
+extern template const void* strip_kernel<false>(int, bool, int, bool);
 
 }  // namespace nrm

@@ -1,0 +1,9 @@
+// Strip kernels for frames of any pitch and alignment (loader warps in place of
+// TMA, one store per pixel).
+#include "nrm_forward_strip.cuh"
+
+namespace nrm {
+
+template const void* strip_kernel<false>(int, bool, int, bool);
+
+}  // namespace nrm

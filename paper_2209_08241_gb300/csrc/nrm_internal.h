@@ -115,22 +115,24 @@ const void* fwd_param_kernel(int tile_x, int tile_y, int threads, int out_dtype)
 size_t param_batch_bytes();
 void pack_param_batch(void* dst, const BatchHeader& hdr, const int* tile_begin, const FrameDesc* frames, int n);
 
-// Strip kernels (nrm_forward_strip.cu): the batched forward pass of frames whose
-// rows TMA can load and whose outputs take whole-vector stores (see
-// strip_frame in nrm_api.cpp), alpha <= kStripMaxAlpha. Descriptors are those of
-// the persistent kernels for tile kStripX x strip_tile_y(out_dtype). param_block: a ParamBatch
-// packed by pack_param_batch, or NULL for the device block in args. u16: every
-// frame is uint16.
+// Strip kernels (nrm_forward_strip.cu): the batched forward pass, alpha <=
+// kStripMaxAlpha, of frames whose rows TMA can load and whose outputs take
+// whole-vector stores (aligned; see strip_frame in nrm_api.cpp), or of any
+// frames. Descriptors are those of the persistent kernels for tile kStripX x
+// strip_tile_y(out_dtype, aligned). param_block: a ParamBatch packed by
+// pack_param_batch, or NULL for the device block in args. u16: every frame is
+// uint16.
 constexpr int kStripX = 128;
 NRM_HD constexpr int strip_rows(int out_dtype) { return out_dtype == NRM_OUT_OCT16 ? 8 : 4; }  // per warp
-NRM_HD constexpr int strip_warps(int out_dtype) {
-  return out_dtype == NRM_OUT_F32X4 ? 6 : out_dtype == NRM_OUT_F16X4 ? 12 : 4;
+NRM_HD constexpr int strip_warps(int out_dtype, bool aligned) {
+  return out_dtype == NRM_OUT_OCT16 ? 4 : out_dtype == NRM_OUT_F16X4 && aligned ? 12 : 6;
 }
-NRM_HD constexpr int strip_tile_y(int out_dtype) { return strip_rows(out_dtype) * strip_warps(out_dtype); }
-NRM_HD constexpr int strip_threads(int out_dtype) { return (strip_warps(out_dtype) + 1) * 32; }
+NRM_HD constexpr int strip_tile_y(int out_dtype, bool aligned) {
+  return strip_rows(out_dtype) * strip_warps(out_dtype, aligned);
+}
 constexpr int kStripMaxAlpha = 4;
 cudaError_t launch_forward_strip(const BatchArgs& args, const Globals& g, int out_dtype, int total_tiles, bool u16,
-                                 cudaStream_t stream, const void* param_block = nullptr);
+                                 bool aligned, cudaStream_t stream, const void* param_block = nullptr);
 
 // Stage buffer bytes for a tile config and alpha: for input elements of eb
 // bytes (2: uint16, 4: float32), or the maximum over both (eb = 0).

@@ -52,7 +52,7 @@ __device__ __forceinline__ void ms_band(const InT* __restrict__ S, const float4*
   const int row0 = band * kRows;
   const int rows = min(kRows, f.rows - row0);
   if (rows <= 0) return;
-  const bool on = 4 * lane < f.cols;
+  const int n = f.cols - 4 * lane;
   const InT* p = S + (row0 + K) * SP + PAD + 4 * lane;  // the band's first row
   unsigned char* np = f.normals + ((long long)row0 * f.out_pitch + 4 * lane) * BPP;
   uint8_t* mp = f.valid + (long long)row0 * f.out_pitch + 4 * lane;
@@ -115,7 +115,7 @@ __device__ __forceinline__ void ms_band(const InT* __restrict__ S, const float4*
       strip_decide<SECANT, EB == 2>(mn, ax, ay, ap, T, tau2, nu1[j], ku[j], nv1, kv, nz[j], q[j], keep[2 * j],
                                     keep[2 * j + 1]);
     }
-    strip_store<OUT>(nx, ny, nz, q, keep, np, mp, on, f);
+    strip_store<OUT, true>(nx, ny, nz, q, keep, np, mp, n, nullptr, f);
     np += f.out_pitch * BPP;
     mp += f.out_pitch;
   }
@@ -128,7 +128,7 @@ __global__ void __launch_bounds__((kWarps + 1) * 32, 1)
   args.hdr = &pb.hdr;
   args.tile_begin = pb.tile_begin;
   args.frames = pb.frames;
-  strip_pipeline<OUT, K, kRows, kWarps, false>(
+  strip_pipeline<OUT, K, kRows, kWarps, 0, false>(
       args, g, [&](const auto* S, const float4* ctab, const float4* rtab, const StripInfo& f, int warp) {
         ms_band<OUT, FORM, SECANT, K>(S, ctab, rtab, f, warp, g.tau2);
       });

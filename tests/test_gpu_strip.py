@@ -1,8 +1,8 @@
 """The strip kernels (batched forward with the default geometry) against the
 tiled kernels (any other geometry): the same bits, over widths and heights
 around the tile edges, every pixel distance they are compiled for, both input
-types, all outputs, both mask modes, depth values of every kind, batches past
-the parameter block and batches of which only some frames qualify."""
+types, all outputs, both mask modes, depth values of every kind, frames of any
+alignment, batches past the parameter block and batches of both kinds."""
 import pytest
 import torch
 
@@ -59,6 +59,36 @@ def test_same_bits_as_the_tiled_kernels(out, alpha, mask):
         items = [(depth(W, H, dt, gen), (0.8 * W, 0.9 * W, 0.4 * W, 0.6 * H)) for W, H in SIZES for dt in ("f32", "u16")]
         assert_same(*both(b, items), (out, alpha, mask, sign))
         assert_same(*both(b, items[1::2]), (out, alpha, mask, sign, "u16 only"))
+
+
+@pytest.mark.parametrize("out", ["f32", "f16", "oct16"])
+@pytest.mark.parametrize("alpha", [1, 2, 3, 4])
+def test_any_alignment_same_bits_as_the_tiled_kernels(out, alpha):
+    """Frames that TMA cannot load (odd widths and pitches, depth starting on any
+    element), outputs of every alignment."""
+    gen = torch.Generator(device=DEV)
+    gen.manual_seed(alpha)
+    C, dt = (2, torch.int16) if out == "oct16" else (4, torch.float16 if out == "f16" else torch.float32)
+    sizes = [(1, 1), (3, 2), (5, 24), (127, 25), (129, 23), (131, 49), (255, 33), (257, 5), (389, 47)]
+    for mask, tau in (("secant", 12.0), ("raw", 1e-3)):
+        b = nrm.BatchedEstimator(nrm.NormalParams(alpha=alpha, out_dtype=out, mask_mode=mask, tau=tau))
+        items, starts = [], []
+        for i, (W, H) in enumerate(sizes):
+            for dtype in ("f32", "u16"):
+                d = depth(W + 2, H, dtype, gen)[:, i % 3:i % 3 + W]
+                items.append((d, (0.8 * W, 0.9 * W, 0.4 * W, 0.6 * H)))
+                starts.append(i % 4)
+
+        def outputs():
+            made = []
+            for (d, _), s in zip(items, starts):
+                H, W = d.shape
+                nb = torch.zeros((H * (W + s) + s, C), dtype=dt, device=DEV)[s:].view(H, W + s, C)
+                vb = torch.zeros(H * (W + s) + s, dtype=torch.uint8, device=DEV)[s:].view(H, W + s)
+                made.append((nb[:, :W], vb[:, :W]))
+            return made
+
+        assert_same(*both(b, items, outputs), (out, alpha, mask))
 
 
 @pytest.mark.parametrize("out", ["f32", "oct16"])
