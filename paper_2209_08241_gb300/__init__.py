@@ -650,7 +650,7 @@ def angle_mse(est, normals, valid, ref_normals, ref_valid, stream=None) -> torch
     _check_map(ref_normals, ref_valid, "ref_normals", est.device)
     if valid.shape != ref_valid.shape or valid.stride(0) != ref_valid.stride(0):
         raise ValueError("the two maps must have one shape and pitch")
-    out = torch.zeros(3, dtype=torch.float64, device=normals.device)
+    out = torch.empty(3, dtype=torch.float64, device=normals.device)
     H, W = valid.shape
     _lib.check(est.lib.nrm_angle_mse(est.h, normals.data_ptr(), valid.data_ptr(), ref_normals.data_ptr(),
                                      ref_valid.data_ptr(), H, W, valid.stride(0), out.data_ptr(),

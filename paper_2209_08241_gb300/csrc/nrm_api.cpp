@@ -276,7 +276,7 @@ struct nrm_handle {
   int persistent_grid_pts[2] = {0, 0};
   const void* param_persistent = nullptr;  // capture-safe kernel (descriptors as a parameter)
   int persistent_grid_param[2] = {0, 0};
-  int* d_status = nullptr;
+  int* d_status = nullptr;               // the status word, then nrm_angle_mse's ticket
   unsigned long long timeout_ns = kDefaultTimeoutNs;
   Slot slots[kSlots];
   int next_slot = 0;
@@ -700,8 +700,8 @@ int nrm_create(const nrm_intrinsics* K, int H, int W, const nrm_params* p, nrm_h
   }
   h->sm_count = prop.multiProcessorCount;
   std::snprintf(h->gpu_name, sizeof(h->gpu_name), "%s", prop.name);
-  if ((e = cudaMalloc(&h->d_status, sizeof(int))) != cudaSuccess ||
-      (e = cudaMemset(h->d_status, 0, sizeof(int))) != cudaSuccess ||
+  if ((e = cudaMalloc(&h->d_status, 2 * sizeof(int))) != cudaSuccess ||
+      (e = cudaMemset(h->d_status, 0, 2 * sizeof(int))) != cudaSuccess ||
       (e = cudaEventCreateWithFlags(&h->last_single, cudaEventDisableTiming)) != cudaSuccess) {
     nrm_destroy(h);
     return cuda_fail(e, "handle allocation");
@@ -1553,9 +1553,10 @@ int nrm_angle_mse(nrm_handle* h, const float* normals, const uint8_t* valid, con
   DeviceGuard guard(h->device);
   if (!h->d_mse_partials)
     NRM_CUDA(cudaMalloc(&h->d_mse_partials, sizeof(double) * 3 * nrm::kMseBlocks), "cudaMalloc");
-  NRM_CUDA(nrm::launch_angle_mse(normals, valid, ref_normals, ref_valid, H, W, pitch, h->d_mse_partials, out,
+  NRM_CUDA(nrm::launch_angle_mse(normals, valid, ref_normals, ref_valid, H, W, pitch, h->d_mse_partials,
+                                 reinterpret_cast<unsigned*>(h->d_status + 1), out, h->d_status, h->timeout_ns,
                                  static_cast<cudaStream_t>(cuda_stream)),
-           "launch mse kernels");
+           "launch mse_kernel");
   NRM_CHECK(mark_single(h, static_cast<cudaStream_t>(cuda_stream)));
   return NRM_OK;
 }

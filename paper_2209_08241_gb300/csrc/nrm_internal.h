@@ -239,12 +239,14 @@ cudaError_t launch_backward_batched_param(const FrameDesc* frames, const BwdMaps
                                           const Globals& g, cudaStream_t stream, const float* scale = nullptr);
 
 // Evaluation kernels (nrm_eval.cu).
-constexpr int kMseBlocks = 2048;  // fixed, so that the reduction order never changes
+constexpr int kMseBlocks = 456;  // fixed, so that the reduction order never changes; three per SM of the GB300
 cudaError_t launch_spherical(const float* normals, const uint8_t* valid, int H, int W, long long pitch, float* phi,
                              float* theta, cudaStream_t stream);
-// partials: 3 kMseBlocks doubles of device scratch; out: 3 doubles.
+// partials: 3 kMseBlocks doubles of device scratch; ticket: a zeroed device word,
+// returned to zero; out: 3 doubles.
 cudaError_t launch_angle_mse(const float* na, const uint8_t* va, const float* nb, const uint8_t* vb, int H, int W,
-                             long long pitch, double* partials, double* out, cudaStream_t stream);
+                             long long pitch, double* partials, unsigned* ticket, double* out, int* status,
+                             unsigned long long timeout_ns, cudaStream_t stream);
 
 // Multi-scale variant (nrm_multiscale.cu): one CTA per kMsTileX x kMsTileY
 // tile, halo of the largest scale. Per scale i the constants of its stencil
