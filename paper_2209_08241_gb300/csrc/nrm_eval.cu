@@ -168,7 +168,9 @@ __device__ __forceinline__ void block_sum3(double& a, double& b, double& c) {
 // are under way while it evaluates four arctangents a pixel (paired: the estimate
 // and the reference in one instruction), and the mask bytes of the next piece are
 // loaded a piece ahead. Three CTAs fill an SM; the grid is one wave, so no SM
-// waits for a last partial one.
+// waits for a last partial one. The pieces are taken from the maps' end: what a
+// call before this one read last (the angle images of the same map) is still in
+// L2 (both calls on 4096 x 3072: 128.4 us, from the start 137.2).
 //
 // Bound by issue (about 115 thread instructions per pixel), HBM (34 B/px) close
 // behind. 4096 x 3072: 76.0 us (83 % of the measured copy); before, with a step's
@@ -205,7 +207,7 @@ __global__ void __launch_bounds__(kThreads, 3)
   const long long mine = first < total ? (total - 1 - first) / step + 1 : 0;
   // Offset of piece i of this warp and its pixels.
   auto piece = [&](long long i, int& n) {
-    const long long u = first + i * step;
+    const long long u = total - 1 - (first + i * step);
     const long long y = u / per_row;
     const int x = (int)(u - y * per_row) * kMsePiece;
     n = min(kMsePiece, W - x);
