@@ -118,9 +118,19 @@ def _in_dtype(t: torch.Tensor) -> int:
     raise TypeError(f"depth must be float32 (metres) or uint16 (depth_scale units), got {t.dtype}")
 
 
+# The current device's current stream as a raw handle, without the Stream object that
+# torch.cuda.current_stream() makes (3.0 us of the 8.5 us that a per-frame call
+# took; this 0.2 us).
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_device = getattr(torch._C, "_cuda_getDevice", None)
+
+
 def _stream_ptr(stream: torch.cuda.Stream | None) -> int:
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return s.cuda_stream
+    if stream is not None:
+        return stream.cuda_stream
+    if _raw_stream is None or _device is None or not torch.cuda.is_initialized():
+        return torch.cuda.current_stream().cuda_stream
+    return _raw_stream(_device())
 
 
 def _intr(K) -> _lib.Intrinsics:
