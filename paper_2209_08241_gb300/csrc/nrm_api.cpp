@@ -181,15 +181,15 @@ int make_desc(FrameDesc* d, const void* depth, void* normals, uint8_t* valid, in
 // set only when the depth, gradient and mask maps can all be made.
 void make_bwd_desc(FrameDesc* d, nrm::BwdMaps* maps, const float* depth, const float* grad_normals,
                    const uint8_t* valid, float* grad_depth, int H, int W, long long depth_pitch,
-                   long long out_pitch, const nrm_intrinsics& K, const nrm_params& p) {
-  const int TX = nrm::kBwdTileX, TY = nrm::kBwdTileY, a = p.alpha;
+                   long long out_pitch, const nrm_intrinsics& K, const nrm_params& p, bool walk) {
+  const nrm::BwdShape b = nrm::bwd_shape(p.alpha, walk);
   make_desc(d, depth, const_cast<float*>(grad_normals), const_cast<uint8_t*>(valid), H, W, depth_pitch, out_pitch,
-            K, NRM_IN_F32_M, p, TX, TY, TX + 2 * nrm::pad_x(2 * a, 4), TY + 4 * a);
+            K, NRM_IN_F32_M, p, b.tx, b.ty, b.dep_w, b.dep_h);
   d->grad_depth = grad_depth;
   std::memset(maps, 0, sizeof(*maps));
   if (d->use_tma) {
-    const bool ok = encode_grad_map(&maps->grad, grad_normals, W, H, out_pitch, TX + 2 * a, TY + 2 * a) &&
-                    encode_mask_map(&maps->mask, valid, W, H, out_pitch, nrm::kBwdMaskBoxW, TY + 2 * a);
+    const bool ok = encode_grad_map(&maps->grad, grad_normals, W, H, out_pitch, b.ex_w, b.ex_h) &&
+                    encode_mask_map(&maps->mask, valid, W, H, out_pitch, nrm::kBwdMaskBoxW, b.ex_h);
     if (!ok) d->use_tma = 0;
   }
 }
@@ -1337,9 +1337,13 @@ int nrm_backward(nrm_handle* h, const void* depth, const float* grad_normals, co
   DeviceGuard guard(h->device);
   FrameDesc d;
   nrm::BwdMaps maps;
+  const int al = h->p.alpha;
+  const bool walk = nrm::bwd_walks(al, nrm::bwd_extended(nrm::bwd_shape(al, true), h->H, h->W),
+                                   nrm::bwd_extended(nrm::bwd_shape(al, false), h->H, h->W));
   make_bwd_desc(&d, &maps, static_cast<const float*>(depth), grad_normals, valid, grad_depth, h->H, h->W, h->W,
-                h->W, h->K, h->p);
-  if ((h->H + nrm::kBwdTileY - 1) / nrm::kBwdTileY > 65535) {
+                h->W, h->K, h->p, walk);
+  const int TY = nrm::bwd_shape(al, walk).ty;
+  if ((h->H + TY - 1) / TY > 65535) {
     // More tile rows than a launch grid holds: a one-frame batched adjoint
     // (one grid row of all the frame's tiles; same per-tile code).
     nrm_grad_frame gf = {};
@@ -1356,7 +1360,7 @@ int nrm_backward(nrm_handle* h, const void* depth, const float* grad_normals, co
   }
   nrm::Globals g = make_globals(h);
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-  NRM_CUDA(nrm::launch_backward(d, maps, g, st), "launch bwd_kernel");
+  NRM_CUDA(nrm::launch_backward(d, maps, g, walk, st), "launch bwd_kernel");
   NRM_CHECK(mark_single(h, st));
   return NRM_OK;
 }
@@ -1420,8 +1424,8 @@ static int backward_batched(nrm_handle* h, const nrm_grad_frame* frames, int n, 
   if (n == 0) return NRM_OK;
   if (!frames) return fail(NRM_ERR_INVALID_ARG, "frames is NULL");
   if (n > 65535) return fail(NRM_ERR_UNSUPPORTED, "at most 65535 frames per batched adjoint");
-  const int TX = nrm::kBwdTileX, TY = nrm::kBwdTileY;
-  long long total = 0;
+  const nrm::BwdShape forms[2] = {nrm::bwd_shape(h->p.alpha, false), nrm::bwd_shape(h->p.alpha, true)};
+  long long total = 0, extended[2] = {0, 0};
   for (int i = 0; i < n; ++i) {
     const nrm_grad_frame& f = frames[i];
     if (f.H < 0 || f.W < 0) return fail(NRM_ERR_INVALID_ARG, "frame %d: negative size", i);
@@ -1434,10 +1438,13 @@ static int backward_batched(nrm_handle* h, const nrm_grad_frame* frames, int n, 
       return fail(NRM_ERR_INVALID_ARG, "frame %d: depth buffers not 4-byte aligned", i);
     if (f.H > (1 << 24) || f.W > (1 << 24)) return fail(NRM_ERR_UNSUPPORTED, "frame %d: dimension above 2^24", i);
     if (validate_intrinsics(f.K)) return fail(NRM_ERR_INVALID_ARG, "frame %d: bad intrinsics", i);
-    total += (long long)((f.W + TX - 1) / TX) * ((f.H + TY - 1) / TY);
+    total += (long long)((f.W + 63) / 64) * ((f.H + 31) / 32);
     if (total >= (1LL << 31) - 1) return fail(NRM_ERR_UNSUPPORTED, "batch exceeds 2^31 tiles");
+    for (int k = 0; k < 2; ++k) extended[k] += nrm::bwd_extended(forms[k], f.H, f.W);
   }
   if (total == 0) return NRM_OK;
+  const bool walk = nrm::bwd_walks(h->p.alpha, extended[1], extended[0]);
+  const int TY = forms[walk].ty;
   DeviceGuard guard(h->device);
   if (n > nrm::kBwdParamMaxFrames) {
     // The descriptor ring is uploaded from host memory that later calls reuse:
@@ -1457,11 +1464,11 @@ static int backward_batched(nrm_handle* h, const nrm_grad_frame* frames, int n, 
     for (int i = 0; i < n; ++i) {
       const nrm_grad_frame& f = frames[i];
       make_bwd_desc(&fdv[i], &mapv[i], f.depth, f.grad_normals, f.valid, f.grad_depth, f.H, f.W, f.depth_pitch,
-                    f.out_pitch, f.K, h->p);
+                    f.out_pitch, f.K, h->p, walk);
       max_tiles = std::max(max_tiles, fdv[i].tiles_x * ((f.H + TY - 1) / TY));
     }
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-    NRM_CUDA(nrm::launch_backward_batched_param(fdv.data(), mapv.data(), n, max_tiles, make_globals(h), st, scale),
+    NRM_CUDA(nrm::launch_backward_batched_param(fdv.data(), mapv.data(), n, max_tiles, make_globals(h), walk, st, scale),
              "launch bwd_batched_param_kernel");
     NRM_CHECK(mark_single(h, st));
     return NRM_OK;
@@ -1493,7 +1500,7 @@ static int backward_batched(nrm_handle* h, const nrm_grad_frame* frames, int n, 
   for (int i = 0; i < n; ++i) {
     const nrm_grad_frame& f = frames[i];
     make_bwd_desc(&fd[i], &maps[i], f.depth, f.grad_normals, f.valid, f.grad_depth, f.H, f.W, f.depth_pitch,
-                  f.out_pitch, f.K, h->p);
+                  f.out_pitch, f.K, h->p, walk);
     fd[i].tile_begin = acc;
     tb[i] = acc;
     acc += fd[i].tiles_x * ((f.H + TY - 1) / TY);
@@ -1513,7 +1520,7 @@ static int backward_batched(nrm_handle* h, const nrm_grad_frame* frames, int n, 
   nrm::Globals g = make_globals(h);
   int max_tiles = 0;
   for (int i = 0; i < n; ++i) max_tiles = std::max(max_tiles, fd[i].tiles_x * ((frames[i].H + TY - 1) / TY));
-  NRM_CUDA(nrm::launch_backward_batched(args, n, max_tiles, g, st, scale), "launch bwd_batched_kernel");
+  NRM_CUDA(nrm::launch_backward_batched(args, n, max_tiles, g, walk, st, scale), "launch bwd_batched_kernel");
   NRM_CUDA(cudaEventRecord(s.done, st), "cudaEventRecord");
   s.in_flight = true;
   return NRM_OK;

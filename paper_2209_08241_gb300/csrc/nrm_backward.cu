@@ -14,17 +14,29 @@
 //   dL/dd_q = w2(q - alpha x) + w4(q + alpha x) + w3(q - alpha y) + w5(q + alpha y),
 // a deterministic gather with no atomics.
 //
-// One CTA per 64 x 32 output tile. Three TMA loads on one mbarrier stage the
-// tile's inputs in shared memory: the depth halo of radius 2 alpha, the upstream
-// gradient of the tile extended by alpha (a 2-D box of 8-byte elements, two per
-// pixel, i.e. float4 per pixel) and the mask of the same region (a
-// uint8 box starting 16 columns left of the tile, the alignment TMA needs).
-// Phase 1 turns each staged gradient into the four weights in place; phase 2
-// gathers. Frames whose buffers cannot be TMA-mapped use plain loads into the
-// same shared-memory layout. bwd_kernel covers one frame (grid = its tiles);
-// bwd_batched_kernel covers a batch (grid = max tiles of a frame x frames).
-// Both are compiled for alpha = 1..4 as constants (shared-memory offsets and
-// loop steps become immediates) and once for any alpha.
+// One CTA per output tile. Three TMA loads on one mbarrier stage the tile's
+// inputs in shared memory: the depth halo, the upstream gradient of the
+// extended region (a 2-D box of 8-byte elements, two per pixel, i.e. float4 per
+// pixel) and the mask of the same region (bwd_shape, nrm_internal.h). Frames
+// whose buffers cannot be TMA-mapped use plain loads into the same shared-memory
+// layout. bwd_kernel covers one frame (grid = its tiles); bwd_batched_kernel
+// covers a batch (grid = max tiles of a frame x frames).
+//
+// Two forms. The walk (bwd_tile, alpha = 2..4): a warp owns kRows rows of a 64 x 32
+// extended region, two columns (x, x + 32) per lane as the pairs of the paired FP32
+// instructions, and keeps the weights in registers: the horizontal sums take w2 and w4
+// from other lanes by shuffles, the vertical ones w3 and w5 from the lane's own
+// registers or, across bands, from a row exchange in shared memory. The gather
+// (bwd_tile_gather, any alpha) stores the four weights of each pixel in shared memory
+// and gathers them: 38 shared-memory wavefronts per 32 pixels, a third of them
+// conflict replays, and 124 thread instructions a pixel, against 21 and 95.
+// alpha 2: 4096 x 3072 walk 60.1 us (77 % of the measured copy), gather 68.1; loss
+// step of 8 x 1920x1080 201 against 205 us, of 32 x 640x480, which the walk's 60 x 28
+// tiles overhang by 8 %, 101 against 99.7: hence the rule on extended pixels
+// (bwd_walks). alpha 3 and 4, 32 x 640x480 and 8 x 1080p: 116 / 205 and 124 / 220
+// against 125 / 223 and 126 / 226; alpha 1, where the gather has the smallest halo,
+// 114 against 112. (Walk with 3 CTAs per SM in place of 4: 69.1 us; 9, 10 or 12
+// warps: 66.9, 64.4, 75.7.)
 #include <algorithm>
 #include <cstring>
 #include <map>
@@ -40,64 +52,32 @@ using namespace dev;
 
 namespace {
 
-constexpr int TX = kBwdTileX;
-constexpr int TY = kBwdTileY;
 constexpr int NT = kBwdThreads;
 constexpr int NW = NT / 32;
 constexpr int MW = kBwdMaskBoxW;   // mask tile pitch (bytes)
-constexpr int MP = kBwdMaskPad;    // mask tile column of global x = gx0 - MP
+constexpr int kMinCtas = 4;        // CTAs per SM (as shared memory allows)
+constexpr int kRows = 4;           // rows of the extended region per warp (bwd_tile)
 
-__host__ __device__ inline unsigned round128(unsigned b) { return (b + 127) / 128 * 128; }
-__host__ __device__ inline unsigned depth_tile_bytes(int alpha) {
-  return round128((unsigned)((TX + 2 * pad_x(2 * alpha, 4)) * (TY + 4 * alpha) * 4));
+__host__ __device__ constexpr unsigned round128(unsigned b) { return (b + 127) / 128 * 128; }
+__host__ __device__ constexpr unsigned depth_tile_bytes(BwdShape s) {
+  return round128((unsigned)(s.dep_w * s.dep_h * 4));
 }
-__host__ __device__ inline unsigned weight_tile_bytes(int alpha) {
-  return round128((unsigned)((TX + 2 * alpha) * (TY + 2 * alpha) * 16));
+__host__ __device__ constexpr unsigned weight_tile_bytes(BwdShape s) {
+  return round128((unsigned)(s.ex_w * s.ex_h * 16));
 }
-__host__ __device__ inline unsigned mask_tile_bytes(int alpha) {
-  return round128((unsigned)(MW * (TY + 2 * alpha)));
-}
-// u1 of each column and v1 of each row of the extended region.
-__host__ __device__ inline unsigned coord_table_bytes(int alpha) {
-  return round128((unsigned)((TX + TY + 4 * alpha) * 4));
+__host__ __device__ constexpr unsigned mask_tile_bytes(BwdShape s) { return round128((unsigned)(MW * s.ex_h)); }
+// Ray coordinates: per row (-v1, -v1, v1, v1) (bwd_tile), or u1 per column and v1
+// per row (bwd_tile_gather).
+__host__ __device__ constexpr unsigned coord_table_bytes(BwdShape s) {
+  return round128((unsigned)(s.ex_h * 16 + s.ex_w * 4));
 }
 
-// One output tile (gx0, gy0) of frame fd. tmap_d/tmap_g/tmap_m: its depth,
-// gradient and mask tensor maps (param or global memory; used only when
-// fd.use_tma). If the bounded wait for the copies runs out, the tile records
-// NRM_ERR_TIMEOUT in the status word and writes nothing.
-// ALPHA > 0 compiles the tile for that pixel distance (offsets and loop steps
-// become constants); ALPHA = 0 takes g.alpha at run time.
-template <int ALPHA>
-__device__ __forceinline__ void bwd_tile(const FrameDesc& fd, const void* tmap_d, const void* tmap_g,
-                                         const void* tmap_m, int gx0, int gy0, const Globals& g,
-                                         unsigned char* smem, const float* __restrict__ scale, int frame) {
-  // Upstream gradient = scale[frame] x the staged float4 when scale is given
-  // (the fused loss entry: the staged values are then target normals).
-  const float sc = scale ? __ldg(scale + frame) : 1.0f;
-  const int alpha = ALPHA > 0 ? ALPHA : g.alpha;
-  const int p2 = pad_x(2 * alpha, 4);
-  const int bw = TX + 2 * p2;       // depth tile pitch
-  const int bh = TY + 4 * alpha;
-  const int ex_w = TX + 2 * alpha;  // extended region (gradient / weight / mask)
-  const int ex_h = TY + 2 * alpha;
-  float* dep = reinterpret_cast<float*>(smem);
-  float4* gw = reinterpret_cast<float4*>(smem + depth_tile_bytes(alpha));
-  uint8_t* msk = smem + depth_tile_bytes(alpha) + weight_tile_bytes(alpha);
-  float* ucol = reinterpret_cast<float*>(msk + mask_tile_bytes(alpha));  // u1 of extended column ex
-  float* vrow = ucol + ex_w;                                              // v1 of extended row ey
-  uint64_t* bar = reinterpret_cast<uint64_t*>(reinterpret_cast<unsigned char*>(ucol) + coord_table_bytes(alpha));
-  const int H = fd.H, W = fd.W;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  // The ray coordinates of the extended region, formed while the copies are
-  // in flight (the barrier that follows them publishes these too).
-  for (int t = threadIdx.x; t < ex_w + ex_h; t += NT) {
-    if (t < ex_w)
-      NRM_STS(ucol + t, ((float)(gx0 - alpha + t) - fd.cx) * fd.inv_fx);
-    else
-      NRM_STS(vrow + t - ex_w, ((float)(gy0 - alpha + t - ex_w) - fd.cy) * fd.inv_fy);
-  }
-
+// Stages the tile's inputs; false if the bounded wait for the copies ran out
+// (thread 0 has then recorded NRM_ERR_TIMEOUT). All threads; ends with a barrier.
+__device__ __forceinline__ bool stage_inputs(const FrameDesc& fd, const BwdShape& sh, int alpha, const void* tmap_d,
+                                             const void* tmap_g, const void* tmap_m, int gx0, int gy0, const Globals& g,
+                                             float* dep, float4* gw, uint8_t* msk, uint64_t* bar) {
+  const int xd = gx0 - sh.dep_x, yd = gy0 - 2 * alpha, xe = gx0 - sh.ex_x, ye = gy0 - alpha, xm = xe & ~15;
   if (fd.use_tma) {
     const uint32_t b = smem_u32(bar);
     if (threadIdx.x == 0) {
@@ -106,10 +86,10 @@ __device__ __forceinline__ void bwd_tile(const FrameDesc& fd, const void* tmap_d
     }
     __syncthreads();
     if (threadIdx.x == 0) {
-      mbar_arrive_expect_tx(b, (uint32_t)(bw * bh * 4 + ex_w * ex_h * 16 + MW * ex_h));
-      tma_load_2d(smem_u32(dep), tmap_d, gx0 - p2, gy0 - 2 * alpha, b);
-      tma_load_2d(smem_u32(gw), tmap_g, 2 * (gx0 - alpha), gy0 - alpha, b);  // x in 8-byte units: even
-      tma_load_2d(smem_u32(msk), tmap_m, gx0 - MP, gy0 - alpha, b);
+      mbar_arrive_expect_tx(b, (uint32_t)(sh.dep_w * sh.dep_h * 4 + sh.ex_w * sh.ex_h * 16 + MW * sh.ex_h));
+      tma_load_2d(smem_u32(dep), tmap_d, xd, yd, b);
+      tma_load_2d(smem_u32(gw), tmap_g, 2 * xe, ye, b);  // x in 8-byte units: even
+      tma_load_2d(smem_u32(msk), tmap_m, xm, ye, b);
     }
     const bool ok = mbar_wait_warp(b, 0, g.timeout_ns);
     if (__syncthreads_or(!ok)) {
@@ -117,23 +97,193 @@ __device__ __forceinline__ void bwd_tile(const FrameDesc& fd, const void* tmap_d
         record_error(g.status, NRM_ERR_TIMEOUT);
         mbar_wait_bounded(b, 0, g.timeout_ns);
       }
-      return;
+      return false;
     }
-  } else {
-    load_tile_plain(dep, bw, bh, fd, gx0 - p2, gy0 - 2 * alpha);
-    const float4* gn = reinterpret_cast<const float4*>(fd.normals);
-    for (int ey = warp; ey < ex_h; ey += NW) {
-      const int py = gy0 - alpha + ey;
-      for (int ex = lane; ex < ex_w; ex += 32) {
-        const int px = gx0 - alpha + ex;
-        const bool in = px >= 0 && py >= 0 && px < W && py < H;
-        const long long o = (long long)py * fd.out_pitch + px;
-        NRM_STS(gw + ey * ex_w + ex, in ? __ldg(gn + o) : make_float4(0.f, 0.f, 0.f, 0.f));
-        NRM_STS(msk + ey * MW + ex + MP - alpha, in ? __ldg(fd.valid + o) : (uint8_t)0);
-      }
-    }
-    __syncthreads();
+    return true;
   }
+  load_tile_plain(dep, sh.dep_w, sh.dep_h, fd, xd, yd);
+  const float4* gn = reinterpret_cast<const float4*>(fd.normals);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int ey = warp; ey < sh.ex_h; ey += NW) {
+    const int py = ye + ey;
+    for (int ex = lane; ex < sh.ex_w; ex += 32) {
+      const int px = xe + ex;
+      const bool in = px >= 0 && py >= 0 && px < fd.W && py < fd.H;
+      const long long o = (long long)py * fd.out_pitch + px;
+      NRM_STS(gw + ey * sh.ex_w + ex, in ? __ldg(gn + o) : make_float4(0.f, 0.f, 0.f, 0.f));
+      NRM_STS(msk + ey * MW + ex + xe - xm, in ? __ldg(fd.valid + o) : (uint8_t)0);
+    }
+  }
+  __syncthreads();
+  return true;
+}
+
+// The depth weights w2..w5 of a pixel pair (Eq. 4-6 differentiated; the file
+// comment) from its stencil and upstream gradient, each operation that of
+// bwd_tile_gather. mx = -n_x and my = -n_y are formed, with -1/||n|| beside 1/||n||,
+// since the paired instructions take no negated operands.
+struct PairWeights {
+  float2 w2, w3, w4, w5;
+};
+__device__ __forceinline__ PairWeights pair_weights(float2 d2, float2 d3, float2 d4, float2 d5, float2 gx, float2 gy,
+                                                    float2 gz, float2 KA, float2 KB, float2 KC, float2 u1, float2 nu1,
+                                                    float2 v1, float2 nv1, float2 sign) {
+  const float2 M1 = f2(-1.0f, -1.0f);
+  const float2 S24 = __fadd2_rn(d2, d4), D24 = __ffma2_rn(M1, d4, d2);
+  const float2 S35 = __fadd2_rn(d3, d5), D35 = __ffma2_rn(M1, d5, d3);
+  const float2 A35 = __fmul2_rn(KA, S35), B35 = __fmul2_rn(KB, D35), C35 = __fmul2_rn(KC, S35);
+  const float2 A24 = __fmul2_rn(KA, D24), B24 = __fmul2_rn(KB, S24), C24 = __fmul2_rn(KC, S24);
+  const float2 mx = __fmul2_rn(A35, D24), my = __fmul2_rn(B24, D35), P = __fmul2_rn(C24, S35);
+  const float2 nz = __ffma2_rn(u1, mx, __ffma2_rn(v1, my, P));
+  const float2 q = __ffma2_rn(mx, mx, __ffma2_rn(my, my, __fmul2_rn(nz, nz)));
+  const float2 inv = f2(rsqrt_ftz(fmaxf(q.x, 1.17549435e-38f)), rsqrt_ftz(fmaxf(q.y, 1.17549435e-38f)));
+  const float2 ninv = __fmul2_rn(M1, inv);
+  const float2 hx0 = __fmul2_rn(mx, ninv), hy0 = __fmul2_rn(my, ninv), hz0 = __fmul2_rn(nz, inv);
+  const float2 ngd = __fmul2_rn(M1, __ffma2_rn(gx, hx0, __ffma2_rn(gy, hy0, __fmul2_rn(gz, hz0))));
+  const float2 si = __fmul2_rn(sign, inv);
+  const float2 hx = __fmul2_rn(__ffma2_rn(ngd, hx0, gx), si);
+  const float2 hy = __fmul2_rn(__ffma2_rn(ngd, hy0, gy), si);
+  const float2 hz = __fmul2_rn(__ffma2_rn(ngd, hz0, gz), si);
+  const float2 ex = __ffma2_rn(nu1, hz, hx), ey = __ffma2_rn(nv1, hz, hy);
+  const float2 nex = __fmul2_rn(M1, ex), ney = __fmul2_rn(M1, ey);
+  const float2 c35 = __ffma2_rn(hz, C35, __fmul2_rn(ney, B35));
+  const float2 c24 = __ffma2_rn(hz, C24, __fmul2_rn(nex, A24));
+  return {__ffma2_rn(nex, A35, c35), __ffma2_rn(ney, B24, c24), __ffma2_rn(ex, A35, c35), __ffma2_rn(ey, B24, c24)};
+}
+
+// One output tile (gx0, gy0) of frame fd for a pixel distance 2..4. scale: the
+// upstream gradient is scale[frame] times the staged float4.
+template <int ALPHA>
+__device__ __forceinline__ void bwd_tile(const FrameDesc& fd, const void* tmap_d, const void* tmap_g,
+                                         const void* tmap_m, int gx0, int gy0, const Globals& g,
+                                         unsigned char* smem, const float* __restrict__ scale, int frame) {
+  constexpr BwdShape SH = bwd_shape(ALPHA, true);
+  static_assert(SH.ex_w == 64 && SH.ex_h == kRows * NW && ALPHA <= kRows && ALPHA <= SH.ex_x, "one band per warp");
+  float* dep = reinterpret_cast<float*>(smem);
+  float4* gw = reinterpret_cast<float4*>(smem + depth_tile_bytes(SH));
+  uint8_t* msk = smem + depth_tile_bytes(SH) + weight_tile_bytes(SH);
+  float4* vtab = reinterpret_cast<float4*>(msk + mask_tile_bytes(SH));
+  uint64_t* bar = reinterpret_cast<uint64_t*>(reinterpret_cast<unsigned char*>(vtab) + coord_table_bytes(SH));
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (threadIdx.x < SH.ex_h) {
+    const float v1 = ((float)(gy0 - ALPHA + (int)threadIdx.x) - fd.cy) * fd.inv_fy;
+    NRM_STS(vtab + threadIdx.x, make_float4(-v1, -v1, v1, v1));
+  }
+  if (!stage_inputs(fd, SH, ALPHA, tmap_d, tmap_g, tmap_m, gx0, gy0, g, dep, gw, msk, bar)) return;
+
+  const int xe = gx0 - SH.ex_x;
+  const float ua = ((float)(xe + lane) - fd.cx) * fd.inv_fx, ub = ((float)(xe + lane + 32) - fd.cx) * fd.inv_fx;
+  const float2 u1 = f2(ua, ub), nu1 = f2(-ua, -ub);
+  const float2 KA = f2(fd.a, fd.a), KB = f2(fd.b, fd.b), KC = f2(fd.c, fd.c), sign = f2(g.sign, g.sign);
+  const float sc = scale ? __ldg(scale + frame) : 1.0f;
+  const int row0 = warp * kRows;  // the band's first row in the extended region
+  // Centre column depths of the band's rows and ALPHA rows above and below.
+  const float* pc = dep + row0 * SH.dep_w + SH.dep_x - SH.ex_x + lane;
+  float2 R[kRows + 2 * ALPHA];
+#pragma unroll
+  for (int i = 0; i < 2 * ALPHA; ++i)
+    R[i] = f2(NRM_LDS(float, pc + i * SH.dep_w), NRM_LDS(float, pc + i * SH.dep_w + 32));
+  const uint8_t* pm = msk + row0 * MW + (xe & 15) + lane;
+  float2 t[kRows], w3[kRows], w5[kRows];
+#pragma unroll
+  for (int r = 0; r < kRows; ++r) {
+    const float* p = pc + (r + ALPHA) * SH.dep_w;
+    R[r + 2 * ALPHA] = f2(NRM_LDS(float, p + ALPHA * SH.dep_w), NRM_LDS(float, p + ALPHA * SH.dep_w + 32));
+    const float2 d2 = f2(NRM_LDS(float, p + ALPHA), NRM_LDS(float, p + ALPHA + 32));
+    const float2 d4 = f2(NRM_LDS(float, p - ALPHA), NRM_LDS(float, p - ALPHA + 32));
+    const float4* pg = gw + (row0 + r) * 64 + lane;
+    const float4 ga = NRM_LDS(float4, pg), gb = NRM_LDS(float4, pg + 32);
+    float2 gx = f2(ga.x, gb.x), gy = f2(ga.y, gb.y), gz = f2(ga.z, gb.z);
+    if (scale) {
+      const float2 s2 = f2(sc, sc);
+      gx = __fmul2_rn(gx, s2);
+      gy = __fmul2_rn(gy, s2);
+      gz = __fmul2_rn(gz, s2);
+    }
+    const float4 vv = NRM_LDS(float4, vtab + row0 + r);
+    PairWeights w = pair_weights(d2, R[r + 2 * ALPHA], d4, R[r], gx, gy, gz, KA, KB, KC, u1, nu1, f2(vv.z, vv.w),
+                                 f2(vv.x, vv.y), sign);
+    // Only valid pixels have weights (elsewhere depth and gradient can be anything).
+    const bool ka = NRM_LDS(uint8_t, pm + r * MW) != 0, kb = NRM_LDS(uint8_t, pm + r * MW + 32) != 0;
+    const float w2a = ka ? w.w2.x : 0.0f, w2b = kb ? w.w2.y : 0.0f;
+    const float w4a = ka ? w.w4.x : 0.0f, w4b = kb ? w.w4.y : 0.0f;
+    w3[r] = f2(ka ? w.w3.x : 0.0f, kb ? w.w3.y : 0.0f);
+    w5[r] = f2(ka ? w.w5.x : 0.0f, kb ? w.w5.y : 0.0f);
+    // w2 from ALPHA columns to the left, w4 from ALPHA to the right (the columns
+    // whose source lies outside the extended region are not in the tile).
+    const float la = __shfl_sync(0xffffffffu, w2a, lane - ALPHA), lb = __shfl_sync(0xffffffffu, w2b, lane - ALPHA);
+    const float ra = __shfl_sync(0xffffffffu, w4a, lane + ALPHA), rb = __shfl_sync(0xffffffffu, w4b, lane + ALPHA);
+    t[r] = __fadd2_rn(f2(la, lane < ALPHA ? la : lb), f2(lane >= 32 - ALPHA ? rb : ra, rb));
+  }
+  // Rows that a neighbouring band needs, in this warp's own part of the gradient
+  // tile (which only it has read): w5 of the first ALPHA rows, then w3 of the last.
+  __syncwarp();
+  float* xch = reinterpret_cast<float*>(gw + row0 * 64);
+#pragma unroll
+  for (int i = 0; i < ALPHA; ++i) {
+    NRM_STS(xch + i * 64 + lane, w5[i].x);
+    NRM_STS(xch + i * 64 + lane + 32, w5[i].y);
+    NRM_STS(xch + (ALPHA + i) * 64 + lane, w3[kRows - ALPHA + i].x);
+    NRM_STS(xch + (ALPHA + i) * 64 + lane + 32, w3[kRows - ALPHA + i].y);
+  }
+  __syncthreads();
+  const float* up = xch - kRows * 64 * 4 + ALPHA * 64 + lane;  // w3 of the band above
+  const float* down = xch + kRows * 64 * 4 + lane;             // w5 of the band below
+  const int xa = xe + lane, xb = xa + 32;
+  const bool oka = lane >= SH.ex_x && xa < fd.W, okb = lane < 32 - SH.ex_x && xb < fd.W;
+#pragma unroll
+  for (int r = 0; r < kRows; ++r) {
+    const int er = row0 + r;
+    const int gy = gy0 - ALPHA + er;
+    if (er < ALPHA || er >= SH.ex_h - ALPHA || gy >= fd.H) continue;
+    const float2 a = r >= ALPHA ? w3[r >= ALPHA ? r - ALPHA : 0]
+                                : f2(NRM_LDS(float, up + r * 64), NRM_LDS(float, up + r * 64 + 32));
+    const float* pd = down + (r + ALPHA - kRows) * 64;
+    const float2 b = r + ALPHA < kRows ? w5[r + ALPHA < kRows ? r + ALPHA : 0]
+                                       : f2(NRM_LDS(float, pd), NRM_LDS(float, pd + 32));
+    const float2 v = __fadd2_rn(__fadd2_rn(t[r], a), b);
+    float* q = fd.grad_depth + (long long)gy * fd.depth_pitch + xa;
+    [[maybe_unused]] const long long len = dbg_span(fd.H, fd.W, fd.depth_pitch, 4);
+    if (oka && NRM_GOK(q, fd.grad_depth, len)) *q = v.x;
+    if (okb && NRM_GOK(q + 32, fd.grad_depth, len)) q[32] = v.y;
+  }
+}
+
+// One output tile (gx0, gy0) of frame fd. tmap_d/tmap_g/tmap_m: its depth,
+// gradient and mask tensor maps (param or global memory; used only when
+// fd.use_tma), for the pixel distance ALPHA or, if that is 0, g.alpha. If the bounded wait for the
+// copies runs out, the tile records NRM_ERR_TIMEOUT in the status word and writes
+// nothing.
+template <int ALPHA>
+__device__ __forceinline__ void bwd_tile_gather(const FrameDesc& fd, const void* tmap_d, const void* tmap_g,
+                                         const void* tmap_m, int gx0, int gy0, const Globals& g,
+                                         unsigned char* smem, const float* __restrict__ scale, int frame) {
+  // Upstream gradient = scale[frame] x the staged float4 when scale is given
+  // (the fused loss entry: the staged values are then target normals).
+  const float sc = scale ? __ldg(scale + frame) : 1.0f;
+  const int alpha = ALPHA > 0 ? ALPHA : g.alpha;
+  const BwdShape sh = bwd_shape(alpha, false);
+  const int bw = sh.dep_w;     // depth tile pitch
+  const int ex_w = sh.ex_w;    // extended region (gradient / weight / mask)
+  const int ex_h = sh.ex_h;
+  const int TX = sh.tx, TY = sh.ty;
+  float* dep = reinterpret_cast<float*>(smem);
+  float4* gw = reinterpret_cast<float4*>(smem + depth_tile_bytes(sh));
+  uint8_t* msk = smem + depth_tile_bytes(sh) + weight_tile_bytes(sh);
+  float* ucol = reinterpret_cast<float*>(msk + mask_tile_bytes(sh));  // u1 of extended column ex
+  float* vrow = ucol + ex_w;                                          // v1 of extended row ey
+  uint64_t* bar = reinterpret_cast<uint64_t*>(reinterpret_cast<unsigned char*>(ucol) + coord_table_bytes(sh));
+  const int H = fd.H, W = fd.W;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  // The ray coordinates of the extended region, formed before the copies are
+  // waited for (the barrier that follows them publishes these too).
+  for (int t = threadIdx.x; t < ex_w + ex_h; t += NT) {
+    if (t < ex_w)
+      NRM_STS(ucol + t, ((float)(gx0 - alpha + t) - fd.cx) * fd.inv_fx);
+    else
+      NRM_STS(vrow + t - ex_w, ((float)(gy0 - alpha + t - ex_w) - fd.cy) * fd.inv_fy);
+  }
+  if (!stage_inputs(fd, sh, alpha, tmap_d, tmap_g, tmap_m, gx0, gy0, g, dep, gw, msk, bar)) return;
 
   // Phase 1: the weights of every pixel p of the extended tile, in place of
   // its staged gradient. Threads walk the ex_w x ex_h elements in row-major
@@ -150,8 +300,8 @@ __device__ __forceinline__ void bwd_tile(const FrameDesc& fd, const void* tmap_d
   const int step_rows = NT / ex_w, step_cols = NT - step_rows * ex_w;
   int ey = threadIdx.x / ex_w;
   int ex = threadIdx.x - ey * ex_w;
-  const float* dep_c = dep + alpha * bw + p2 - alpha;  // depth-tile position of (ey, ex) = (0, 0)
-  const uint8_t* msk_c = msk + MP - alpha;
+  const float* dep_c = dep + alpha * bw + sh.dep_x - alpha;  // depth-tile position of (ey, ex) = (0, 0)
+  const uint8_t* msk_c = msk + ((gx0 - alpha) & 15);
   for (int i = threadIdx.x; i < n_ext; i += NT) {
     float4 w = make_float4(0.f, 0.f, 0.f, 0.f);
     if (NRM_LDS(uint8_t, msk_c + ey * MW + ex)) {
@@ -213,26 +363,40 @@ __device__ __forceinline__ void bwd_tile(const FrameDesc& fd, const void* tmap_d
   }
 }
 
-template <int ALPHA>
-__global__ void __launch_bounds__(NT)
+template <int ALPHA, bool WALK>
+__device__ __forceinline__ void bwd_any_tile(const FrameDesc& fd, const void* tmap_d, const void* tmap_g,
+                                             const void* tmap_m, int gx0, int gy0, const Globals& g,
+                                             unsigned char* smem, const float* __restrict__ scale, int frame) {
+  if constexpr (WALK)
+    bwd_tile<ALPHA>(fd, tmap_d, tmap_g, tmap_m, gx0, gy0, g, smem, scale, frame);
+  else
+    bwd_tile_gather<ALPHA>(fd, tmap_d, tmap_g, tmap_m, gx0, gy0, g, smem, scale, frame);
+}
+
+template <int ALPHA, bool WALK>
+__global__ void __launch_bounds__(NT, kMinCtas)
     bwd_kernel(const __grid_constant__ FrameDesc fd, const __grid_constant__ BwdMaps maps, const Globals g,
                const float* scale) {
   extern __shared__ __align__(128) unsigned char smem[];
   NRM_DEBUG_ENTRY(g.status);
-  bwd_tile<ALPHA>(fd, &fd.tmap, &maps.grad, &maps.mask, blockIdx.x * TX, blockIdx.y * TY, g, smem, scale, 0);
+  const BwdShape sh = bwd_shape(ALPHA > 0 ? ALPHA : g.alpha, WALK);
+  bwd_any_tile<ALPHA, WALK>(fd, &fd.tmap, &maps.grad, &maps.mask, blockIdx.x * sh.tx, blockIdx.y * sh.ty, g, smem,
+                            scale, 0);
 }
 
 // Grid (max tiles of a frame, frames): block (x, f) is tile x of frame f; frames
 // with fewer tiles leave their extra blocks idle.
-template <int ALPHA>
-__global__ void __launch_bounds__(NT) bwd_batched_kernel(const BwdBatchArgs args, const Globals g, const float* scale) {
+template <int ALPHA, bool WALK>
+__global__ void __launch_bounds__(NT, kMinCtas)
+    bwd_batched_kernel(const BwdBatchArgs args, const Globals g, const float* scale) {
   extern __shared__ __align__(128) unsigned char smem[];
   NRM_DEBUG_ENTRY(g.status);
   const int f = (int)blockIdx.y;
   const FrameDesc& fd = args.frames[f];
   const int tiles_x = fd.tiles_x;
   const int local = (int)blockIdx.x;
-  if (tiles_x == 0 || local >= tiles_x * ((fd.H + TY - 1) / TY)) return;
+  const BwdShape sh = bwd_shape(ALPHA > 0 ? ALPHA : g.alpha, WALK);
+  if (tiles_x == 0 || local >= tiles_x * ((fd.H + sh.ty - 1) / sh.ty)) return;
   if (threadIdx.x == 0 && fd.use_tma) {
     fence_tensormap_acquire(&fd.tmap);
     fence_tensormap_acquire(&args.maps[f].grad);
@@ -240,7 +404,8 @@ __global__ void __launch_bounds__(NT) bwd_batched_kernel(const BwdBatchArgs args
   }
   const int ty = local / tiles_x;
   const int tx = local - ty * tiles_x;
-  bwd_tile<ALPHA>(fd, &fd.tmap, &args.maps[f].grad, &args.maps[f].mask, tx * TX, ty * TY, g, smem, scale, f);
+  bwd_any_tile<ALPHA, WALK>(fd, &fd.tmap, &args.maps[f].grad, &args.maps[f].mask, tx * sh.tx, ty * sh.ty, g, smem,
+                            scale, f);
 }
 
 // A batch of at most kBwdParamMaxFrames frames with its records and tensor
@@ -253,8 +418,8 @@ struct alignas(128) BwdParamBatch {
 static_assert(sizeof(BwdParamBatch) <= 32764, "the descriptor block must fit the kernel parameter limit");
 
 // Grid (max tiles of a frame, frames), as bwd_batched_kernel.
-template <int ALPHA>
-__global__ void __launch_bounds__(NT)
+template <int ALPHA, bool WALK>
+__global__ void __launch_bounds__(NT, kMinCtas)
     bwd_batched_param_kernel(const __grid_constant__ BwdParamBatch pb, const Globals g, const float* scale) {
   extern __shared__ __align__(128) unsigned char smem[];
   NRM_DEBUG_ENTRY(g.status);
@@ -262,32 +427,29 @@ __global__ void __launch_bounds__(NT)
   const FrameDesc& fd = pb.frames[f];
   const int tiles_x = fd.tiles_x;
   const int local = (int)blockIdx.x;
-  if (tiles_x == 0 || local >= tiles_x * ((fd.H + TY - 1) / TY)) return;
+  const BwdShape sh = bwd_shape(ALPHA > 0 ? ALPHA : g.alpha, WALK);
+  if (tiles_x == 0 || local >= tiles_x * ((fd.H + sh.ty - 1) / sh.ty)) return;
   const int ty = local / tiles_x;
   const int tx = local - ty * tiles_x;
-  bwd_tile<ALPHA>(fd, &fd.tmap, &pb.maps[f].grad, &pb.maps[f].mask, tx * TX, ty * TY, g, smem, scale, f);
+  bwd_any_tile<ALPHA, WALK>(fd, &fd.tmap, &pb.maps[f].grad, &pb.maps[f].mask, tx * sh.tx, ty * sh.ty, g, smem, scale,
+                            f);
 }
 
-const void* bwd_param_kernel_for(int alpha) {
-  switch (alpha) {
-    case 1: return (const void*)bwd_batched_param_kernel<1>;
-    case 2: return (const void*)bwd_batched_param_kernel<2>;
-    case 3: return (const void*)bwd_batched_param_kernel<3>;
-    case 4: return (const void*)bwd_batched_param_kernel<4>;
-    default: return (const void*)bwd_batched_param_kernel<0>;
-  }
+// The kernel of a launch kind for a distance and form: compiled for alpha = 1..4
+// (constant offsets and loop steps), generic above.
+enum { kOneFrame, kBatch, kBatchParam };
+template <int ALPHA, bool WALK>
+const void* bwd_kernel_of(int kind) {
+  return kind == kOneFrame ? (const void*)bwd_kernel<ALPHA, WALK>
+         : kind == kBatch  ? (const void*)bwd_batched_kernel<ALPHA, WALK>
+                           : (const void*)bwd_batched_param_kernel<ALPHA, WALK>;
 }
-
-// The kernel for alpha: compiled for alpha = 1..4 (constant offsets and loop
-// steps), generic above.
-const void* bwd_kernel_for(int alpha, bool batched) {
-  switch (alpha) {
-    case 1: return batched ? (const void*)bwd_batched_kernel<1> : (const void*)bwd_kernel<1>;
-    case 2: return batched ? (const void*)bwd_batched_kernel<2> : (const void*)bwd_kernel<2>;
-    case 3: return batched ? (const void*)bwd_batched_kernel<3> : (const void*)bwd_kernel<3>;
-    case 4: return batched ? (const void*)bwd_batched_kernel<4> : (const void*)bwd_kernel<4>;
-    default: return batched ? (const void*)bwd_batched_kernel<0> : (const void*)bwd_kernel<0>;
-  }
+const void* bwd_kernel_for(int alpha, bool walk, int kind) {
+  if (walk)
+    return alpha == 2 ? bwd_kernel_of<2, true>(kind) : alpha == 3 ? bwd_kernel_of<3, true>(kind)
+                                                                  : bwd_kernel_of<4, true>(kind);
+  return alpha == 1 ? bwd_kernel_of<1, false>(kind) : alpha == 2 ? bwd_kernel_of<2, false>(kind)
+                                                                 : bwd_kernel_of<0, false>(kind);
 }
 
 // Grants the dynamic shared memory a kernel needs, once per (kernel, device)
@@ -311,10 +473,10 @@ cudaError_t set_smem(const void* fn, unsigned bytes) {
 // per frame count 16 bytes per load, of the whole frame where its rows are
 // contiguous (every thread's two or three loads are then in flight together), else a
 // warp per row. Bound by latency: the loss step of 32 x 640x480 takes 99.7 us with
-// it (one byte per load, a block per row: 112.5). Each block adds its count to the frame's counter, and the last block of the frame
-// to finish (the ordering of a fence and an atomic ticket) writes the scale
-// and returns both counters to zero for the next call. Integer sums: the
-// result does not depend on the order.
+// it (one byte per load, a block per row: 112.5). Each block adds its count to the
+// frame's counter, and the last block of the frame to finish (the ordering of a
+// fence and an atomic ticket) writes the scale and returns both counters to zero
+// for the next call. Integer sums: the result does not depend on the order.
 constexpr int kCountBlocks = 32;
 constexpr int kCountThreads = 256;
 
@@ -392,17 +554,19 @@ cudaError_t launch_loss_scale(const LossCountFrame* frames, int n, unsigned* cou
   return cudaSuccess;
 }
 
-unsigned bwd_smem_bytes(int alpha) {
-  return depth_tile_bytes(alpha) + weight_tile_bytes(alpha) + mask_tile_bytes(alpha) + coord_table_bytes(alpha) + 16;
+unsigned bwd_smem_bytes(int alpha, bool walk) {
+  const BwdShape s = bwd_shape(alpha, walk);
+  return depth_tile_bytes(s) + weight_tile_bytes(s) + mask_tile_bytes(s) + coord_table_bytes(s) + 16;
 }
 
-cudaError_t launch_backward(const FrameDesc& fd, const BwdMaps& maps, const Globals& g, cudaStream_t stream,
-                            const float* scale) {
-  const unsigned smem = bwd_smem_bytes(g.alpha);
-  const void* fn = bwd_kernel_for(g.alpha, false);
+cudaError_t launch_backward(const FrameDesc& fd, const BwdMaps& maps, const Globals& g, bool walk,
+                            cudaStream_t stream, const float* scale) {
+  const unsigned smem = bwd_smem_bytes(g.alpha, walk);
+  const void* fn = bwd_kernel_for(g.alpha, walk, kOneFrame);
   cudaError_t e = set_smem(fn, smem);
   if (e != cudaSuccess) return e;
-  dim3 grid((fd.W + TX - 1) / TX, (fd.H + TY - 1) / TY);
+  const BwdShape s = bwd_shape(g.alpha, walk);
+  dim3 grid((fd.W + s.tx - 1) / s.tx, (fd.H + s.ty - 1) / s.ty);
   FrameDesc d = fd;
   BwdMaps m = maps;
   Globals gg = g;
@@ -413,9 +577,9 @@ cudaError_t launch_backward(const FrameDesc& fd, const BwdMaps& maps, const Glob
 }
 
 cudaError_t launch_backward_batched(const BwdBatchArgs& args, int n_frames, int max_tiles, const Globals& g,
-                                    cudaStream_t stream, const float* scale) {
-  const unsigned smem = bwd_smem_bytes(g.alpha);
-  const void* fn = bwd_kernel_for(g.alpha, true);
+                                    bool walk, cudaStream_t stream, const float* scale) {
+  const unsigned smem = bwd_smem_bytes(g.alpha, walk);
+  const void* fn = bwd_kernel_for(g.alpha, walk, kBatch);
   cudaError_t e = set_smem(fn, smem);
   if (e != cudaSuccess) return e;
   BwdBatchArgs a = args;
@@ -427,10 +591,11 @@ cudaError_t launch_backward_batched(const BwdBatchArgs& args, int n_frames, int 
 }
 
 cudaError_t launch_backward_batched_param(const FrameDesc* frames, const BwdMaps* maps, int n_frames, int max_tiles,
-                                          const Globals& g, cudaStream_t stream, const float* scale) {
+                                          const Globals& g, bool walk, cudaStream_t stream,
+                                          const float* scale) {
   if (n_frames < 1 || n_frames > kBwdParamMaxFrames) return cudaErrorInvalidValue;
-  const unsigned smem = bwd_smem_bytes(g.alpha);
-  const void* fn = bwd_param_kernel_for(g.alpha);
+  const unsigned smem = bwd_smem_bytes(g.alpha, walk);
+  const void* fn = bwd_kernel_for(g.alpha, walk, kBatchParam);
   cudaError_t e = set_smem(fn, smem);
   if (e != cudaSuccess) return e;
   std::vector<unsigned char> raw(sizeof(BwdParamBatch) + 128);

@@ -180,18 +180,28 @@ int host_validate_params(const nrm_params& p);
 int host_validate_frame(const nrm_frame& f, int index, int out_dtype);
 void host_make_forward_desc(FrameDesc* d, const nrm_frame& f, const nrm_params& p, int tile_x, int tile_y);
 
-// Backward (adjoint) kernel for float32 depth: output tile and threads.
-constexpr int kBwdTileX = 64;
-constexpr int kBwdTileY = 32;
+// Backward (adjoint) kernel for float32 depth: threads, and per pixel distance and
+// form (walk: weights in registers, alpha 2..4; else the gather) the output tile and the staged regions: the extended region (the pixels whose
+// weights reach the tile) ex_w x ex_h from (-ex_x, -alpha) of the tile's origin,
+// the depth box dep_w x dep_h from (-dep_x, -2 alpha), and the mask box
+// kBwdMaskBoxW x ex_h from the extended region's left rounded down to 16 (TMA
+// boxes start on 16-byte boundaries).
 constexpr int kBwdThreads = 256;
-// Columns of the mask box to the left of the tile: the TMA box must start on a
-// 16-byte boundary, so the mask halo (alpha <= 16 columns) is read from 16.
-constexpr int kBwdMaskPad = 16;
-constexpr int kBwdMaskBoxW = kBwdTileX + 2 * kBwdMaskPad;
+constexpr int kBwdMaskBoxW = 96;
+struct BwdShape {
+  int tx, ty, ex_x, ex_w, ex_h, dep_x, dep_w, dep_h;
+};
+NRM_HD constexpr BwdShape bwd_shape(int alpha, bool walk) {
+  // walk: a fixed extended region of 64 x 32 (bwd_tile), of which the tile is the
+  // inside; the tile width keeps its origin on 16 bytes of depth.
+  const int hx = alpha <= 2 ? 2 : 4, dx = (hx + alpha + 3) / 4 * 4, p2 = (2 * alpha + 3) / 4 * 4;
+  return walk ? BwdShape{64 - 2 * hx, 32 - 2 * alpha, hx, 64, 32, dx, (dx - hx + 64 + alpha + 3) / 4 * 4, 32 + 2 * alpha}
+                    : BwdShape{64, 32, alpha, 64 + 2 * alpha, 32 + 2 * alpha, p2, 64 + 2 * p2, 32 + 4 * alpha};
+}
 
 // The adjoint's two further tensor maps per frame: the upstream gradient as a
-// 2-D tensor of 8-byte elements (2 W, H), box (2 (TX + 2 alpha), TY + 2 alpha),
-// and the mask as a 2-D uint8 tensor, box (kBwdMaskBoxW, TY + 2 alpha).
+// 2-D tensor of 8-byte elements (2 W, H), box (2 ex_w, ex_h), and the mask as a
+// 2-D uint8 tensor, box (kBwdMaskBoxW, ex_h).
 struct alignas(128) BwdMaps {
   CUtensorMap grad;
   CUtensorMap mask;
@@ -208,18 +218,30 @@ struct BwdBatchArgs {
   const BwdMaps* maps;
 };
 
-unsigned bwd_smem_bytes(int alpha);
-// fd.tmap maps the depth with box (kBwdTileX + 2 pad_x(2 alpha, 4)) x (kBwdTileY + 4 alpha);
+// The extended pixels of a frame's tiles: what either form computes.
+NRM_HD inline long long bwd_extended(const BwdShape& s, int H, int W) {
+  return (long long)((W + s.tx - 1) / s.tx) * ((H + s.ty - 1) / s.ty) * s.ex_w * s.ex_h;
+}
+// Which form a call takes: alpha 3 and 4 walk; alpha 2 where the walk's tiles do not
+// overhang the frames much more than the gather's (extended pixels, both forms');
+// other distances gather. Measured sides: nrm_backward.cu.
+inline bool bwd_walks(int alpha, long long walk_px, long long gather_px) {
+  return alpha == 3 || alpha == 4 || (alpha == 2 && walk_px * 100 <= gather_px * 107);
+}
+
+unsigned bwd_smem_bytes(int alpha, bool walk);
+// walk: the form (bwd_walks), which the descriptors' boxes are for.
+// fd.tmap maps the depth with box dep_w x dep_h of bwd_shape(alpha, walk);
 // fd.normals holds the upstream gradient, fd.valid the mask, fd.grad_depth the output.
 // fd.use_tma = 1 only if all three maps (fd.tmap, maps.grad, maps.mask) are valid.
 // scale (optional, device array indexed by frame): the upstream gradient is
 // scale[frame] times the float4 buffer (then a target normal map).
-cudaError_t launch_backward(const FrameDesc& fd, const BwdMaps& maps, const Globals& g, cudaStream_t stream,
-                            const float* scale = nullptr);
+cudaError_t launch_backward(const FrameDesc& fd, const BwdMaps& maps, const Globals& g, bool walk,
+                            cudaStream_t stream, const float* scale = nullptr);
 // All tiles of a batch in one launch (grid max_tiles x n_frames); the descriptor
 // block is in device memory.
 cudaError_t launch_backward_batched(const BwdBatchArgs& args, int n_frames, int max_tiles, const Globals& g,
-                                    cudaStream_t stream, const float* scale = nullptr);
+                                    bool walk, cudaStream_t stream, const float* scale = nullptr);
 // One frame's mask for the cosine-loss factor (nrm_cosine_loss_scale).
 struct LossCountFrame {
   const uint8_t* valid;
@@ -236,7 +258,8 @@ cudaError_t launch_loss_scale(const LossCountFrame* frames, int n, unsigned* cou
 // (host arrays) passed as one kernel parameter: no upload, no fences.
 constexpr int kBwdParamMaxFrames = 60;
 cudaError_t launch_backward_batched_param(const FrameDesc* frames, const BwdMaps* maps, int n_frames, int max_tiles,
-                                          const Globals& g, cudaStream_t stream, const float* scale = nullptr);
+                                          const Globals& g, bool walk, cudaStream_t stream,
+                                          const float* scale = nullptr);
 
 // Evaluation kernels (nrm_eval.cu).
 constexpr int kMseBlocks = 456;  // fixed, so that the reduction order never changes; three per SM of the GB300
