@@ -825,57 +825,6 @@ void nrm_destroy(nrm_handle* h) {
   delete h;
 }
 
-static int estimate_single(nrm_handle* h, const void* depth, void* normals, uint8_t* valid, float* points,
-                           void* cuda_stream) {
-  g_last_error.clear();
-  if (!h) return fail(NRM_ERR_INVALID_ARG, "handle is NULL");
-  if (h->H == 0 || h->W == 0) return fail(NRM_ERR_INVALID_ARG, "handle was created for batched calls only");
-  nrm_frame f = {};
-  f.depth = depth;
-  f.normals = normals;
-  f.valid = valid;
-  f.H = h->H;
-  f.W = h->W;
-  f.depth_pitch = h->W;
-  f.out_pitch = h->W;
-  f.K = h->K;
-  f.in_dtype = h->p.in_dtype;
-  f.points = points;
-  int rc = validate_frame(f, 0, h->p.out_dtype);
-  if (rc) return rc;
-  DeviceGuard guard(h->device);
-  const int TX = h->cfg.tile_x, TY = h->cfg.tile_y;
-  const int eb = f.in_dtype == NRM_IN_U16_MM ? 2 : 4;
-  FrameDesc d;
-  make_desc(&d, depth, normals, valid, f.H, f.W, f.depth_pitch, f.out_pitch, f.K, f.in_dtype, h->p, TX, TY,
-            TX + 2 * nrm::pad_x(h->p.alpha, eb), TY + 2 * h->p.alpha, points);
-  nrm::Globals g = make_globals(h);
-  dim3 grid((f.W + TX - 1) / TX, (f.H + TY - 1) / TY);
-  // More tile rows than a launch grid holds: the frame runs as a one-frame
-  // batch (the persistent kernel walks a tile list; same per-pixel code).
-  if (grid.y > 65535) return nrm_estimate_batched(h, &f, 1, cuda_stream);
-  void* args[2] = {&d, &g};
-  cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-  NRM_CUDA(cudaLaunchKernel(points ? h->pts_plain : h->ks->plain[h->p.out_dtype], grid, dim3(h->cfg.threads),
-                            args, nrm::plain_smem_bytes(TX, TY, h->p.alpha), st),
-           "launch fwd_plain_kernel");
-  NRM_CHECK(mark_single(h, st));
-  return NRM_OK;
-}
-
-int nrm_estimate(nrm_handle* h, const void* depth, void* normals, uint8_t* valid, void* cuda_stream) {
-  return estimate_single(h, depth, normals, valid, nullptr, cuda_stream);
-}
-
-int nrm_estimate_points(nrm_handle* h, const void* depth, void* normals, uint8_t* valid, float* points,
-                        void* cuda_stream) {
-  if (!points) {
-    g_last_error.clear();
-    return fail(NRM_ERR_INVALID_ARG, "points is NULL");
-  }
-  return estimate_single(h, depth, normals, valid, points, cuda_stream);
-}
-
 // The frames of a batched forward (or multi-scale) call, in two parts, each with
 // its own work list: those that the strip kernel for aligned frames takes, then
 // the rest, which a forward call gives to the strip kernel for any alignment
@@ -973,6 +922,7 @@ void split_batch(const nrm_handle* h, const nrm_frame* frames, int n, const Batc
     p.stat_tiles += ((f.W + h->cfg.tile_x - 1) / h->cfg.tile_x) * ((f.H + h->cfg.tile_y - 1) / h->cfg.tile_y);
     ++p.n;
   }
+  std::reverse(fd + back, fd + n);  // (in the caller's order: it decides how a launch ends)
   part[0].first = 0;
   part[1].first = back;
 }
@@ -997,11 +947,9 @@ void fill_work_list(const BatchPart& p, FrameDesc* fd, nrm::BatchHeader* hdr, in
   tile_begin[p.n] = acc;
 }
 
-// The 128-byte aligned parameter block of one part's launch, in h's scratch memory.
-void* pack_part(nrm_handle* h, const BatchPart& p, FrameDesc* fd) {
-  std::vector<int>& tb = h->scratch_tb;
+// The 128-byte aligned parameter block of one part's launch, in scratch memory.
+void* pack_part(std::vector<int>& tb, std::vector<unsigned char>& raw, const BatchPart& p, FrameDesc* fd) {
   if (tb.size() < (size_t)p.n + 1) tb.resize((size_t)p.n + 1);
-  std::vector<unsigned char>& raw = h->scratch_param;
   if (raw.size() < nrm::param_batch_bytes() + 128) raw.resize(nrm::param_batch_bytes() + 128);
   void* pb = raw.data() + (128 - reinterpret_cast<uintptr_t>(raw.data()) % 128) % 128;
   nrm::BatchHeader hdr;
@@ -1041,6 +989,83 @@ int launch_part(nrm_handle* h, bool aligned, const nrm::BatchArgs& args, const B
 
 }  // namespace
 
+// From this size on one frame takes the strip kernels, as a batch of one whose
+// descriptors travel in the parameter block (built in memory of the calling
+// thread, so that several threads may use one handle's single-frame call). Below it
+// the plain launch is as fast or faster, its host side being shorter (1280x720: plain
+// 5.8-6.6 us, strip 7.3). 1920x1080 float32 -> float4 10.7 / 10.5 us, uint16 ->
+// octahedral 10.0 / 8.3; 4096x3072 51.6 / 44.9 and 35.2 / 22.7; unaligned 1921x1081
+// 14.7 / 12.8, 4095x3071 72.1 / 49.6.
+constexpr long long kStripFramePx = 2000000;
+
+static int estimate_single_strip(nrm_handle* h, const nrm_frame& f, void* cuda_stream) {
+  static thread_local std::vector<int> tb;
+  static thread_local std::vector<unsigned char> raw;
+  cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
+  FrameDesc d[1];
+  BatchPart part[2];
+  split_batch(h, &f, 1, forward_plan(h), d, part);
+  for (int k = 0; k < 2; ++k) {
+    if (part[k].tiles == 0) continue;
+    void* pb = pack_part(tb, raw, part[k], d);
+    const nrm::BatchArgs ring = {};
+    NRM_CHECK(launch_part(h, k == 0, ring, part[k], pb, st));
+  }
+  return mark_single(h, st);
+}
+
+static int estimate_single(nrm_handle* h, const void* depth, void* normals, uint8_t* valid, float* points,
+                           void* cuda_stream) {
+  g_last_error.clear();
+  if (!h) return fail(NRM_ERR_INVALID_ARG, "handle is NULL");
+  if (h->H == 0 || h->W == 0) return fail(NRM_ERR_INVALID_ARG, "handle was created for batched calls only");
+  nrm_frame f = {};
+  f.depth = depth;
+  f.normals = normals;
+  f.valid = valid;
+  f.H = h->H;
+  f.W = h->W;
+  f.depth_pitch = h->W;
+  f.out_pitch = h->W;
+  f.K = h->K;
+  f.in_dtype = h->p.in_dtype;
+  f.points = points;
+  int rc = validate_frame(f, 0, h->p.out_dtype);
+  if (rc) return rc;
+  DeviceGuard guard(h->device);
+  if (!points && (long long)f.H * f.W >= kStripFramePx && strip_handle(h)) return estimate_single_strip(h, f, cuda_stream);
+  const int TX = h->cfg.tile_x, TY = h->cfg.tile_y;
+  const int eb = f.in_dtype == NRM_IN_U16_MM ? 2 : 4;
+  FrameDesc d;
+  make_desc(&d, depth, normals, valid, f.H, f.W, f.depth_pitch, f.out_pitch, f.K, f.in_dtype, h->p, TX, TY,
+            TX + 2 * nrm::pad_x(h->p.alpha, eb), TY + 2 * h->p.alpha, points);
+  nrm::Globals g = make_globals(h);
+  dim3 grid((f.W + TX - 1) / TX, (f.H + TY - 1) / TY);
+  // More tile rows than a launch grid holds: the frame runs as a one-frame
+  // batch (the persistent kernel walks a tile list; same per-pixel code).
+  if (grid.y > 65535) return nrm_estimate_batched(h, &f, 1, cuda_stream);
+  void* args[2] = {&d, &g};
+  cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
+  NRM_CUDA(cudaLaunchKernel(points ? h->pts_plain : h->ks->plain[h->p.out_dtype], grid, dim3(h->cfg.threads),
+                            args, nrm::plain_smem_bytes(TX, TY, h->p.alpha), st),
+           "launch fwd_plain_kernel");
+  NRM_CHECK(mark_single(h, st));
+  return NRM_OK;
+}
+
+int nrm_estimate(nrm_handle* h, const void* depth, void* normals, uint8_t* valid, void* cuda_stream) {
+  return estimate_single(h, depth, normals, valid, nullptr, cuda_stream);
+}
+
+int nrm_estimate_points(nrm_handle* h, const void* depth, void* normals, uint8_t* valid, float* points,
+                        void* cuda_stream) {
+  if (!points) {
+    g_last_error.clear();
+    return fail(NRM_ERR_INVALID_ARG, "points is NULL");
+  }
+  return estimate_single(h, depth, normals, valid, points, cuda_stream);
+}
+
 // nrm_estimate_batched with the descriptor block as one kernel parameter
 // (frame records and tensor maps in parameter space): no descriptor upload and
 // no tensor-map fences. Used for batches of at most kParamMaxFrames frames
@@ -1068,7 +1093,7 @@ static int estimate_batched_param(nrm_handle* h, const nrm_frame* frames, int n,
   }
   for (int k = 0; k < 2; ++k) {
     if (part[k].tiles == 0) continue;
-    void* pb = pack_part(h, part[k], fd.data());
+    void* pb = pack_part(h->scratch_tb, h->scratch_param, part[k], fd.data());
     nrm::BatchArgs ring;
     std::memset(&ring, 0, sizeof(ring));
     NRM_CHECK(launch_part(h, k == 0, ring, part[k], pb, st));
@@ -1636,7 +1661,7 @@ int nrm_estimate_batched_multiscale(nrm_handle* h, const nrm_frame* frames, int 
       const BatchPart& p = part[k];
       tiles += p.tiles;
       if (p.tiles == 0) continue;
-      void* pb = pack_part(h, p, fd.data());
+      void* pb = pack_part(h->scratch_tb, h->scratch_param, p, fd.data());
       if (k == 0)
         NRM_CUDA(nrm::launch_multiscale_strip(ms, g, h->p.out_dtype, scales->form, p.tiles, p.u16, st, pb),
                  "launch fwd_ms_strip_kernel");

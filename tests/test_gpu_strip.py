@@ -148,3 +148,18 @@ def test_multiscale_same_bits_as_the_run_time_distance_kernel(form, K):
             two = b.multiscale(items, range(1, K + 1), form, outputs=wide)
             b.sync_status()
             assert_same(one, two, (form, K, out, mask))
+
+
+@pytest.mark.parametrize("W,H", [(2000, 1001), (1999, 1003), (4096, 489)])
+@pytest.mark.parametrize("dtype,out", [("f32", "f32"), ("u16", "f16"), ("u16", "oct16")])
+def test_large_single_frames_same_bits_as_the_plain_kernel(W, H, dtype, out):
+    """Single-frame calls of two million pixels and more take the strip kernels."""
+    gen = torch.Generator(device=DEV)
+    gen.manual_seed(W)
+    d = depth(W, H, dtype, gen)
+    est = nrm.NormalEstimator((0.8 * W, 0.9 * W, 0.4 * W, 0.6 * H), H, W, nrm.NormalParams(out_dtype=out), dtype)
+    one = est.estimate(d)
+    est.set_config(128, 8, 128, 2, 0)
+    two = est.estimate(d)
+    est.sync_status()
+    assert_same([one], [two], (W, H, dtype, out))
