@@ -992,11 +992,13 @@ int launch_part(nrm_handle* h, bool aligned, const nrm::BatchArgs& args, const B
 // From this size on one frame takes the strip kernels, as a batch of one whose
 // descriptors travel in the parameter block (built in memory of the calling
 // thread, so that several threads may use one handle's single-frame call). Below it
-// the plain launch is as fast or faster, its host side being shorter (1280x720: plain
-// 5.8-6.6 us, strip 7.3). 1920x1080 float32 -> float4 10.7 / 10.5 us, uint16 ->
-// octahedral 10.0 / 8.3; 4096x3072 51.6 / 44.9 and 35.2 / 22.7; unaligned 1921x1081
-// 14.7 / 12.8, 4095x3071 72.1 / 49.6.
-constexpr long long kStripFramePx = 2000000;
+// the plain launch stays: its host side is 3 us shorter, which a caller that makes
+// its tensors per call would see (1280x720: plain 5.8-6.6 us, strip 7.3; 1920x1080:
+// GPU time 12.4 against 10.4, but 13.3 with the views made per call). Plain / strip
+// over rotating buffers: 2560x1440 float32 -> float4 18.6 / 16.5 us, uint16 ->
+// half4 14.7 / 12.3; 4096x3072 52.1 / 45.6, 41.2 / 27.3 and uint16 -> octahedral
+// 39.6 / 25.1; unaligned 2561x1441 27.5 / 20.6, 4095x3071 74.8 / 50.9.
+constexpr long long kStripFramePx = 3000000;
 
 static int estimate_single_strip(nrm_handle* h, const nrm_frame& f, void* cuda_stream) {
   static thread_local std::vector<int> tb;

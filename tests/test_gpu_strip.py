@@ -150,10 +150,10 @@ def test_multiscale_same_bits_as_the_run_time_distance_kernel(form, K):
             assert_same(one, two, (form, K, out, mask))
 
 
-@pytest.mark.parametrize("W,H", [(2000, 1001), (1999, 1003), (4096, 489)])
+@pytest.mark.parametrize("W,H", [(2400, 1251), (1999, 1503), (4096, 735)])
 @pytest.mark.parametrize("dtype,out", [("f32", "f32"), ("u16", "f16"), ("u16", "oct16")])
 def test_large_single_frames_same_bits_as_the_plain_kernel(W, H, dtype, out):
-    """Single-frame calls of two million pixels and more take the strip kernels."""
+    """Single-frame calls of three million pixels and more take the strip kernels."""
     gen = torch.Generator(device=DEV)
     gen.manual_seed(W)
     d = depth(W, H, dtype, gen)
