@@ -1364,12 +1364,12 @@ int nrm_backward(nrm_handle* h, const void* depth, const float* grad_normals, co
   DeviceGuard guard(h->device);
   FrameDesc d;
   nrm::BwdMaps maps;
-  const int al = h->p.alpha;
-  const bool walk = nrm::bwd_walks(al, nrm::bwd_extended(nrm::bwd_shape(al, true), h->H, h->W),
-                                   nrm::bwd_extended(nrm::bwd_shape(al, false), h->H, h->W));
+  nrm::BwdChoice choice(h->p.alpha);
+  choice.add(h->H, h->W);
+  const bool walk = choice.walks();
   make_bwd_desc(&d, &maps, static_cast<const float*>(depth), grad_normals, valid, grad_depth, h->H, h->W, h->W,
                 h->W, h->K, h->p, walk);
-  const int TY = nrm::bwd_shape(al, walk).ty;
+  const int TY = nrm::bwd_shape(h->p.alpha, walk).ty;
   if ((h->H + TY - 1) / TY > 65535) {
     // More tile rows than a launch grid holds: a one-frame batched adjoint
     // (one grid row of all the frame's tiles; same per-tile code).
@@ -1451,8 +1451,8 @@ static int backward_batched(nrm_handle* h, const nrm_grad_frame* frames, int n, 
   if (n == 0) return NRM_OK;
   if (!frames) return fail(NRM_ERR_INVALID_ARG, "frames is NULL");
   if (n > 65535) return fail(NRM_ERR_UNSUPPORTED, "at most 65535 frames per batched adjoint");
-  const nrm::BwdShape forms[2] = {nrm::bwd_shape(h->p.alpha, false), nrm::bwd_shape(h->p.alpha, true)};
-  long long total = 0, extended[2] = {0, 0};
+  nrm::BwdChoice choice(h->p.alpha);
+  long long total = 0;
   for (int i = 0; i < n; ++i) {
     const nrm_grad_frame& f = frames[i];
     if (f.H < 0 || f.W < 0) return fail(NRM_ERR_INVALID_ARG, "frame %d: negative size", i);
@@ -1467,11 +1467,11 @@ static int backward_batched(nrm_handle* h, const nrm_grad_frame* frames, int n, 
     if (validate_intrinsics(f.K)) return fail(NRM_ERR_INVALID_ARG, "frame %d: bad intrinsics", i);
     total += (long long)((f.W + 63) / 64) * ((f.H + 31) / 32);
     if (total >= (1LL << 31) - 1) return fail(NRM_ERR_UNSUPPORTED, "batch exceeds 2^31 tiles");
-    for (int k = 0; k < 2; ++k) extended[k] += nrm::bwd_extended(forms[k], f.H, f.W);
+    choice.add(f.H, f.W);
   }
   if (total == 0) return NRM_OK;
-  const bool walk = nrm::bwd_walks(h->p.alpha, extended[1], extended[0]);
-  const int TY = forms[walk].ty;
+  const bool walk = choice.walks();
+  const int TY = nrm::bwd_shape(h->p.alpha, walk).ty;
   DeviceGuard guard(h->device);
   if (n > nrm::kBwdParamMaxFrames) {
     // The descriptor ring is uploaded from host memory that later calls reuse:

@@ -33,7 +33,7 @@
 // alpha 2: 4096 x 3072 walk 60.1 us (77 % of the measured copy), gather 68.1; loss
 // step of 8 x 1920x1080 201 against 205 us, of 32 x 640x480, which the walk's 60 x 28
 // tiles overhang by 8 %, 101 against 99.7: hence the rule on extended pixels
-// (bwd_walks). alpha 3 and 4, 32 x 640x480 and 8 x 1080p: 116 / 205 and 124 / 220
+// (BwdChoice). alpha 3 and 4, 32 x 640x480 and 8 x 1080p: 116 / 205 and 124 / 220
 // against 125 / 223 and 126 / 226; alpha 1, where the gather has the smallest halo,
 // 114 against 112. (Walk with 3 CTAs per SM in place of 4: 69.1 us; 9, 10 or 12
 // warps: 66.9, 64.4, 75.7.)

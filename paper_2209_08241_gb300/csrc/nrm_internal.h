@@ -181,16 +181,18 @@ int host_validate_frame(const nrm_frame& f, int index, int out_dtype);
 void host_make_forward_desc(FrameDesc* d, const nrm_frame& f, const nrm_params& p, int tile_x, int tile_y);
 
 // Backward (adjoint) kernel for float32 depth: threads, and per pixel distance and
-// form (walk: weights in registers, alpha 2..4; else the gather) the output tile and the staged regions: the extended region (the pixels whose
-// weights reach the tile) ex_w x ex_h from (-ex_x, -alpha) of the tile's origin,
-// the depth box dep_w x dep_h from (-dep_x, -2 alpha), and the mask box
-// kBwdMaskBoxW x ex_h from the extended region's left rounded down to 16 (TMA
+// form (walk: weights in registers, for the distances of bwd_has_walk only; else
+// the gather) the output tile and the staged regions: the extended region (the
+// pixels whose weights reach the tile) ex_w x ex_h from (-ex_x, -alpha) of the
+// tile's origin, the depth box dep_w x dep_h from (-dep_x, -2 alpha), and the mask
+// box kBwdMaskBoxW x ex_h from the extended region's left rounded down to 16 (TMA
 // boxes start on 16-byte boundaries).
 constexpr int kBwdThreads = 256;
 constexpr int kBwdMaskBoxW = 96;
 struct BwdShape {
   int tx, ty, ex_x, ex_w, ex_h, dep_x, dep_w, dep_h;
 };
+NRM_HD constexpr bool bwd_has_walk(int alpha) { return alpha >= 2 && alpha <= 4; }
 NRM_HD constexpr BwdShape bwd_shape(int alpha, bool walk) {
   // walk: a fixed extended region of 64 x 32 (bwd_tile), of which the tile is the
   // inside; the tile width keeps its origin on 16 bytes of depth.
@@ -222,15 +224,27 @@ struct BwdBatchArgs {
 NRM_HD inline long long bwd_extended(const BwdShape& s, int H, int W) {
   return (long long)((W + s.tx - 1) / s.tx) * ((H + s.ty - 1) / s.ty) * s.ex_w * s.ex_h;
 }
-// Which form a call takes: alpha 3 and 4 walk; alpha 2 where the walk's tiles do not
-// overhang the frames much more than the gather's (extended pixels, both forms');
-// other distances gather. Measured sides: nrm_backward.cu.
-inline bool bwd_walks(int alpha, long long walk_px, long long gather_px) {
-  return alpha == 3 || alpha == 4 || (alpha == 2 && walk_px * 100 <= gather_px * 107);
-}
+// Which form a call over frames takes: alpha 3 and 4 walk; alpha 2 where the walk's
+// tiles do not overhang the frames much more than the gather's (the extended pixels
+// of all frames, both forms'); other distances gather. Measured sides:
+// nrm_backward.cu.
+class BwdChoice {
+ public:
+  explicit BwdChoice(int alpha) : alpha_(alpha) {}
+  void add(int H, int W) {
+    if (!bwd_has_walk(alpha_)) return;
+    walk_px_ += bwd_extended(bwd_shape(alpha_, true), H, W);
+    gather_px_ += bwd_extended(bwd_shape(alpha_, false), H, W);
+  }
+  bool walks() const { return bwd_has_walk(alpha_) && (alpha_ != 2 || walk_px_ * 100 <= gather_px_ * 107); }
+
+ private:
+  int alpha_;
+  long long walk_px_ = 0, gather_px_ = 0;
+};
 
 unsigned bwd_smem_bytes(int alpha, bool walk);
-// walk: the form (bwd_walks), which the descriptors' boxes are for.
+// walk: the form (BwdChoice), which the descriptors' boxes are for.
 // fd.tmap maps the depth with box dep_w x dep_h of bwd_shape(alpha, walk);
 // fd.normals holds the upstream gradient, fd.valid the mask, fd.grad_depth the output.
 // fd.use_tma = 1 only if all three maps (fd.tmap, maps.grad, maps.mask) are valid.
