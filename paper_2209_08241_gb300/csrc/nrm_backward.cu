@@ -471,14 +471,19 @@ cudaError_t set_smem(const void* fn, unsigned bytes) {
 // The per-frame factor of the cosine loss, scale = -1 / max(N_valid, 1), with
 // N_valid the number of nonzero mask bytes of the frame: kCountBlocks blocks
 // per frame count 16 bytes per load, of the whole frame where its rows are
-// contiguous (every thread's two or three loads are then in flight together), else a
-// warp per row. Bound by latency: the loss step of 32 x 640x480 takes 99.7 us with
+// contiguous (at 640x480 every thread's two or three loads are then in flight
+// together), else a warp per row, or several warps per row where the rows are fewer
+// than the warps (one 1,000,000-pixel row with a gap behind it: 4.3 us, with one warp
+// for it 184, one byte per load 92; four rows of 100,000: 4.2, 22.2 and 12.5).
+// Bound by latency: the loss step of 32 x 640x480 takes 99.7 us with
 // it (one byte per load, a block per row: 112.5). Each block adds its count to the
 // frame's counter, and the last block of the frame to finish (the ordering of a
 // fence and an atomic ticket) writes the scale and returns both counters to zero
 // for the next call. Integer sums: the result does not depend on the order.
 constexpr int kCountBlocks = 32;
 constexpr int kCountThreads = 256;
+constexpr int kCountWarps = kCountBlocks * kCountThreads / 32;
+constexpr int kCountSegment = 512;  // a row's parts hold at least about this many bytes: one load per lane
 
 // Nonzero bytes among those of p[0, n) that are worker i's of `workers` (>= 16).
 __device__ __forceinline__ unsigned count_nonzero(const uint8_t* __restrict__ p, long long n, int i, int workers) {
@@ -498,10 +503,20 @@ __device__ __forceinline__ unsigned count_nonzero(const uint8_t* __restrict__ p,
   return c + (tail < n && __ldg(p + tail) != 0 ? 1u : 0u);
 }
 
+// The parts that a row is counted in, a warp each: as many as there are warps for,
+// of kCountSegment bytes or more. Rows without gaps are counted as one row.
+__host__ __device__ inline int count_segments(const LossCountFrame& f) {
+  if (f.pitch == f.W || f.H <= 0 || f.H >= kCountWarps) return 1;
+  const int fit = kCountWarps / f.H, of = f.W / kCountSegment;
+  return fit < of ? fit : of > 1 ? of : 1;
+}
+
 struct CountArgs {
   LossCountFrame f[kLossCountMaxFrames];
 };
 
+// LONG_ROWS: a batch with frames of fewer rows than warps.
+template <bool LONG_ROWS>
 __global__ void __launch_bounds__(kCountThreads)
     loss_scale_kernel(const __grid_constant__ CountArgs a, unsigned* __restrict__ counts,
                       unsigned* __restrict__ tickets, float* __restrict__ scale) {
@@ -513,9 +528,18 @@ __global__ void __launch_bounds__(kCountThreads)
     c = count_nonzero(fr.valid, (long long)fr.H * fr.W, (int)(blockIdx.x * kCountThreads + threadIdx.x),
                       kCountBlocks * kCountThreads);
   } else {
-    constexpr int kWarps = kCountThreads / 32;
-    for (int y = blockIdx.x * kWarps + (threadIdx.x >> 5); y < fr.H; y += kCountBlocks * kWarps)
-      c += count_nonzero(fr.valid + (long long)y * fr.pitch, fr.W, threadIdx.x & 31, 32);
+    const int first = blockIdx.x * (kCountThreads / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if constexpr (!LONG_ROWS) {
+      for (int y = first; y < fr.H; y += kCountWarps)
+        c += count_nonzero(fr.valid + (long long)y * fr.pitch, fr.W, lane, 32);
+    } else {
+      const int segs = count_segments(fr);
+      const long long len = ((long long)fr.W + 16 * segs - 1) / (16 * segs) * 16;  // (whole 16-byte units)
+      for (long long u = first; u < (long long)fr.H * segs; u += kCountWarps) {
+        const long long y = u / segs, x = (u - y * segs) * len;
+        c += count_nonzero(fr.valid + y * fr.pitch + x, max(0LL, min(len, fr.W - x)), lane, 32);
+      }
+    }
   }
   c = __reduce_add_sync(0xffffffffu, c);
   __shared__ unsigned part[kCountThreads / 32];
@@ -547,8 +571,10 @@ cudaError_t launch_loss_scale(const LossCountFrame* frames, int n, unsigned* cou
     unsigned* t = tickets + first;
     float* sc = scale + first;
     void* args[4] = {&a, &c, &t, &sc};
-    cudaError_t e = cudaLaunchKernel((const void*)loss_scale_kernel, dim3(kCountBlocks, m), dim3(kCountThreads), args,
-                                     0, stream);
+    bool long_rows = false;
+    for (int i = 0; i < m; ++i) long_rows = long_rows || count_segments(a.f[i]) > 1;
+    const void* fn = long_rows ? (const void*)loss_scale_kernel<true> : (const void*)loss_scale_kernel<false>;
+    cudaError_t e = cudaLaunchKernel(fn, dim3(kCountBlocks, m), dim3(kCountThreads), args, 0, stream);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
