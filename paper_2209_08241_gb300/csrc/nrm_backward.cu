@@ -104,13 +104,16 @@ __device__ __forceinline__ bool stage_inputs(const FrameDesc& fd, const BwdShape
   load_tile_plain(dep, sh.dep_w, sh.dep_h, fd, xd, yd);
   const float4* gn = reinterpret_cast<const float4*>(fd.normals);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int ey = warp; ey < sh.ex_h; ey += NW) {
+  // (In registers: read from the descriptor in the loop, 8 x 641x481 at alpha 1 takes
+  // 36.9 us instead of 33.1, at alpha 5 55.6 instead of 50.2.)
+  const int W = fd.W, H = fd.H, w = sh.ex_w, h = sh.ex_h;
+  for (int ey = warp; ey < h; ey += NW) {
     const int py = ye + ey;
-    for (int ex = lane; ex < sh.ex_w; ex += 32) {
+    for (int ex = lane; ex < w; ex += 32) {
       const int px = xe + ex;
-      const bool in = px >= 0 && py >= 0 && px < fd.W && py < fd.H;
+      const bool in = px >= 0 && py >= 0 && px < W && py < H;
       const long long o = (long long)py * fd.out_pitch + px;
-      NRM_STS(gw + ey * sh.ex_w + ex, in ? __ldg(gn + o) : make_float4(0.f, 0.f, 0.f, 0.f));
+      NRM_STS(gw + ey * w + ex, in ? __ldg(gn + o) : make_float4(0.f, 0.f, 0.f, 0.f));
       NRM_STS(msk + ey * MW + ex + xe - xm, in ? __ldg(fd.valid + o) : (uint8_t)0);
     }
   }
