@@ -828,7 +828,8 @@ void nrm_destroy(nrm_handle* h) {
 // The frames of a batched forward (or multi-scale) call, in two parts, each with
 // its own work list: those that the strip kernel for aligned frames takes, then
 // the rest, which a forward call gives to the strip kernel for any alignment
-// (loader warps in place of TMA) or else to the tiled kernel.
+// (loader warps in place of TMA) or to the tiled kernel. Either part may be empty
+// (forward_plan).
 namespace {
 
 struct BatchPart {
@@ -840,13 +841,14 @@ struct BatchPart {
   bool strip = false;    // taken by a strip kernel
 };
 
-// How a call splits its frames: the halo of its tiles, whether a strip kernel
-// may take frames , the tiles of the other kernel,
-// and for multi-scale calls K and the divisor q of the form (1 or 4).
+// How a call splits its frames: the halo of its tiles, whether the strip kernel for
+// aligned frames takes those, whether the one for any alignment takes the rest (else
+// the tiled kernel does), the rows of a tile of either, the tiled kernel's tiles, and
+// for multi-scale calls K and the divisor q of the form (1 or 4).
 struct BatchPlan {
   int halo;
-  bool strip;
-  int strip_y, any_y;   // rows of a tile of the strip kernel for aligned frames, for any
+  bool strip, any;
+  int strip_y, any_y;
   int tile_x, tile_y;
   int scales = 0;
   double q = 4.0;
@@ -870,26 +872,29 @@ bool strip_domain(const nrm_handle* h, const nrm_frame& f, const BatchPlan& plan
   return pmin * pmin / (1.0 + u * u + v * v) >= 4.0 * 1.17549435e-38;
 }
 
+// True if TMA can load the frame's depth rows (make_desc then decides by encoding
+// the map).
+bool tma_rows(const nrm_frame& f) {
+  const int eb = f.in_dtype == NRM_IN_U16_MM ? 2 : 4;
+  return (uintptr_t)f.depth % 16 == 0 && (f.depth_pitch * eb) % 16 == 0;
+}
+
 // True if the strip kernel for aligned frames can take frame f: whole vectors of
 // four pixels to the right edge, outputs on the alignment of the vector stores,
-// and depth rows that TMA can address (make_desc then decides by encoding the map).
+// and depth rows that TMA can address.
 bool strip_aligned(const nrm_handle* h, const nrm_frame& f, const BatchPlan& plan) {
   const uintptr_t na = h->p.out_dtype == NRM_OUT_OCT16 ? 16 : 32;
-  const int eb = f.in_dtype == NRM_IN_U16_MM ? 2 : 4;
-  return plan.strip && strip_domain(h, f, plan) && f.W % 4 == 0 && f.out_pitch % 4 == 0 &&
-         (uintptr_t)f.normals % na == 0 && (uintptr_t)f.valid % 4 == 0 && (uintptr_t)f.depth % 16 == 0 &&
-         (f.depth_pitch * eb) % 16 == 0;
+  return strip_domain(h, f, plan) && f.W % 4 == 0 && f.out_pitch % 4 == 0 && (uintptr_t)f.normals % na == 0 &&
+         (uintptr_t)f.valid % 4 == 0 && tma_rows(f);
 }
 
 // Descriptors of the n frames into fd: the aligned ones from the front, the
 // others from the back. Empty frames are left out.
 void split_batch(const nrm_handle* h, const nrm_frame* frames, int n, const BatchPlan& plan, FrameDesc* fd,
                  BatchPart (&part)[2]) {
-  bool any = plan.strip && plan.scales == 0;  // the rest goes to the strip kernel for any alignment
-  for (int i = 0; i < n; ++i) any = any && ((long long)frames[i].H * frames[i].W == 0 || strip_domain(h, frames[i], plan));
-  const int rest_x = any ? nrm::kStripX : plan.tile_x, rest_y = any ? plan.any_y : plan.tile_y;
+  const int rest_x = plan.any ? nrm::kStripX : plan.tile_x, rest_y = plan.any ? plan.any_y : plan.tile_y;
   part[0].strip = true;
-  part[1].strip = any;
+  part[1].strip = plan.any;
   part[0].tile_y = plan.strip_y;
   part[1].tile_y = rest_y;
   int front = 0, back = n;
@@ -897,7 +902,7 @@ void split_batch(const nrm_handle* h, const nrm_frame* frames, int n, const Batc
     const nrm_frame& f = frames[i];
     if ((long long)f.H * f.W == 0) continue;
     const int eb = f.in_dtype == NRM_IN_U16_MM ? 2 : 4;
-    bool aligned = strip_aligned(h, f, plan);
+    bool aligned = plan.strip && strip_aligned(h, f, plan);
     if (aligned) {
       make_desc(&fd[front], f.depth, f.normals, f.valid, f.H, f.W, f.depth_pitch, f.out_pitch, f.K, f.in_dtype, h->p,
                 nrm::kStripX, plan.strip_y, nrm::kStripX + 2 * nrm::pad_x(plan.halo, eb),
@@ -927,9 +932,98 @@ void split_batch(const nrm_handle* h, const nrm_frame* frames, int n, const Batc
   part[1].first = back;
 }
 
-BatchPlan forward_plan(const nrm_handle* h) {
-  return {h->p.alpha,    strip_handle(h), nrm::strip_tile_y(h->p.out_dtype, true), nrm::strip_tile_y(h->p.out_dtype, false),
-          h->cfg.tile_x, h->cfg.tile_y};
+// GPU time of one launch of a forward kernel: what it takes however small it is (a
+// launch that follows another in its stream adds all of it, and kSecondLaunch on the
+// host), and per million pixels of frames that the aligned strip kernel could take,
+// of others that TMA can load ("ragged": widths or pitches not in fours, outputs off
+// the vector stores' alignment), and of frames with plain loads only. Microseconds,
+// measured by graph replay from 320x240 to 64 x 1920x1080; a call takes the cheapest
+// of the four ways below, so an error of the model costs what the ways differ by
+// where they cross.
+struct LaunchCost {
+  double ramp, aligned, ragged, plain;
+};
+struct ForwardCosts {
+  LaunchCost strip, any, tiled;
+};
+
+// What they rest on (u16 input, alpha 2 where not said): strip 1 x 640x480 3.8 / 4.0 /
+// 3.7 us (float4 / half4 / octahedral), 16 x 1080p 97 / 60 / 51. Any alignment:
+// 321x241 4.9 / 5.4 / 5.9, 16 x 641x481 24.0 / 25.0 / 21.4, 16 x 1921x1081
+// 124 / 125 / 113, ragged 64 x 1918x1078 430-442 / 391-417 / 390-404. Tiled:
+// 318x238 ragged 3.9 / 3.9 / 4.0, 64 x 1918x1078 442-485 / 361 / 355-445, plain
+// loads 321x241 4.9 / 5.0 / 5.0, 16 x 1921x1081 275 / 208 / 212; its vector loops (alpha
+// 1 and 2; octahedral: rows of codes on 16 bytes) make half4 and octahedral tiles
+// cheaper, at alpha 3 and 4 64 x 1918x1078 take 540 / 466 / 497.
+ForwardCosts forward_costs(int out_dtype, int alpha, bool vector_rows) {
+  const bool vec = alpha <= 2;
+  switch (out_dtype) {
+    case NRM_OUT_F16X4: {
+      const double t = vec ? 2.7 : alpha == 3 ? 3.2 : 3.3;
+      return {{3.6, 1.7, 0, 0}, {5.1, 3.0, 3.0, 3.7}, {3.7, t, t, 5.2}};
+    }
+    case NRM_OUT_OCT16: {
+      const double a = alpha == 1 ? 2.3 : 2.75, scalar = vec ? 3.2 : 3.45;
+      return {{3.6, 1.45, 0, 0}, {5.8, a, a, 3.1}, {3.7, vec ? 2.55 : scalar, vec && vector_rows ? 2.55 : scalar, 5.5}};
+    }
+    default: return {{3.6, 2.85, 0, 0}, {4.7, 3.15, 3.0, 3.6}, {3.7, 3.4, 3.6, 7.0}};
+  }
+}
+
+constexpr double kSecondLaunch = 1.5;
+
+// The plan of a forward call. Two launches where both parts are worth one (a batch of
+// 24 aligned and 24 other VGA frames), else one kernel takes all frames: one 640x480
+// and one 641x481 frame, float4: two launches 8.4 us, any alignment 6.2, tiled 7.6.
+BatchPlan forward_plan(const nrm_handle* h, const nrm_frame* frames, int n) {
+  BatchPlan plan = {h->p.alpha,
+                    false,
+                    false,
+                    nrm::strip_tile_y(h->p.out_dtype, true),
+                    nrm::strip_tile_y(h->p.out_dtype, false),
+                    h->cfg.tile_x,
+                    h->cfg.tile_y};
+  if (!strip_handle(h)) return plan;
+  bool any_ok = true;
+  double strip = 0, any[2] = {0, 0}, tiled[2] = {0, 0};  // us beyond the ramps: aligned frames, the rest
+  int count[2] = {0, 0};
+  bool plain_loads = false;
+  ForwardCosts c = {};
+  for (int i = 0; i < n; ++i) {
+    const nrm_frame& f = frames[i];
+    const double mpx = 1e-6 * f.H * f.W;
+    if (mpx == 0) continue;
+    any_ok = any_ok && strip_domain(h, f, plan);
+    c = forward_costs(h->p.out_dtype, h->p.alpha,
+                      (uintptr_t)f.normals % 16 == 0 && f.out_pitch % 4 == 0 && (uintptr_t)f.valid % 4 == 0);
+    const bool aligned = strip_aligned(h, f, plan), tma = tma_rows(f);
+    const int k = aligned ? 0 : 1;
+    ++count[k];
+    strip += aligned ? mpx * c.strip.aligned : 0;
+    any[k] += mpx * (aligned ? c.any.aligned : tma ? c.any.ragged : c.any.plain);
+    tiled[k] += mpx * (aligned ? c.tiled.aligned : tma ? c.tiled.ragged : c.tiled.plain);
+    plain_loads = plain_loads || !tma;
+  }
+  if (count[1] == 0) {
+    plan.strip = true;
+    return plan;
+  }
+  const double tiled_ramp = c.tiled.ramp + (plain_loads ? 0.6 : 0.0);
+  const double split = count[0] ? c.strip.ramp + strip + kSecondLaunch : INFINITY;  // the aligned part of two launches
+  double best = tiled_ramp + tiled[0] + tiled[1];
+  auto take = [&](double us, bool to_strip, bool to_any) {
+    if (us < best) {
+      best = us;
+      plan.strip = to_strip;
+      plan.any = to_any;
+    }
+  };
+  take(split + tiled_ramp + tiled[1], true, false);
+  if (any_ok) {
+    take(c.any.ramp + any[0] + any[1], false, true);
+    take(split + c.any.ramp + any[1], true, true);
+  }
+  return plan;
 }
 
 // One part's header and tile offsets (tile_begin: n + 1 entries).
@@ -997,16 +1091,26 @@ int launch_part(nrm_handle* h, bool aligned, const nrm::BatchArgs& args, const B
 // GPU time 12.4 against 10.4, but 13.3 with the views made per call). Plain / strip
 // over rotating buffers: 2560x1440 float32 -> float4 18.6 / 16.5 us, uint16 ->
 // half4 14.7 / 12.3; 4096x3072 52.1 / 45.6, 41.2 / 27.3 and uint16 -> octahedral
-// 39.6 / 25.1; unaligned 2561x1441 27.5 / 20.6, 4095x3071 74.8 / 50.9.
-constexpr long long kStripFramePx = 3000000;
+// 39.6 / 25.1; unaligned 2561x1441 27.5 / 20.6, 4095x3071 74.8 / 50.9. Half4 frames of
+// no alignment gain later: 2001x1503 14.4-15.8 / 15.0.
+constexpr long long kStripFramePx = 3000000, kStripPlainHalfPx = 5000000;
 
-static int estimate_single_strip(nrm_handle* h, const nrm_frame& f, void* cuda_stream) {
+// True if a single frame goes to a strip kernel, with its plan.
+static bool single_takes_strip(const nrm_handle* h, const nrm_frame& f, BatchPlan* plan) {
+  const long long px = (long long)f.H * f.W;
+  if (px < kStripFramePx || !strip_handle(h)) return false;
+  *plan = forward_plan(h, &f, 1);
+  return plan->strip ||
+         (plan->any && (h->p.out_dtype != NRM_OUT_F16X4 || tma_rows(f) || px >= kStripPlainHalfPx));
+}
+
+static int estimate_single_strip(nrm_handle* h, const nrm_frame& f, const BatchPlan& plan, void* cuda_stream) {
   static thread_local std::vector<int> tb;
   static thread_local std::vector<unsigned char> raw;
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   FrameDesc d[1];
   BatchPart part[2];
-  split_batch(h, &f, 1, forward_plan(h), d, part);
+  split_batch(h, &f, 1, plan, d, part);
   for (int k = 0; k < 2; ++k) {
     if (part[k].tiles == 0) continue;
     void* pb = pack_part(tb, raw, part[k], d);
@@ -1035,7 +1139,8 @@ static int estimate_single(nrm_handle* h, const void* depth, void* normals, uint
   int rc = validate_frame(f, 0, h->p.out_dtype);
   if (rc) return rc;
   DeviceGuard guard(h->device);
-  if (!points && (long long)f.H * f.W >= kStripFramePx && strip_handle(h)) return estimate_single_strip(h, f, cuda_stream);
+  BatchPlan plan;
+  if (!points && single_takes_strip(h, f, &plan)) return estimate_single_strip(h, f, plan, cuda_stream);
   const int TX = h->cfg.tile_x, TY = h->cfg.tile_y;
   const int eb = f.in_dtype == NRM_IN_U16_MM ? 2 : 4;
   FrameDesc d;
@@ -1083,7 +1188,7 @@ static int estimate_batched_param(nrm_handle* h, const nrm_frame* frames, int n,
   std::vector<FrameDesc>& fd = h->scratch_desc;
   if (fd.size() < (size_t)n) fd.resize((size_t)n);
   BatchPart part[2];
-  split_batch(h, frames, n, forward_plan(h), fd.data(), part);
+  split_batch(h, frames, n, forward_plan(h, frames, n), fd.data(), part);
   Slot* s = nullptr;
   if (!capture) {
     // A ring slot supplies the completion (and, with timing on, the kernel
@@ -1117,7 +1222,7 @@ static int estimate_batched_ring(nrm_handle* h, const nrm_frame* frames, int n, 
   char* base = static_cast<char*>(s.host);
   FrameDesc* fd = reinterpret_cast<FrameDesc*>(base + nrm::frames_offset(s.capacity));
   BatchPart part[2];
-  split_batch(h, frames, n, forward_plan(h), fd, part);
+  split_batch(h, frames, n, forward_plan(h, frames, n), fd, part);
   const size_t off[2] = {0, nrm::second_header_offset(part[0].n)};
   for (int k = 0; k < 2; ++k)
     fill_work_list(part[k], fd, reinterpret_cast<nrm::BatchHeader*>(base + off[k]),
@@ -1650,7 +1755,7 @@ int nrm_estimate_batched_multiscale(nrm_handle* h, const nrm_frame* frames, int 
   }
   bool consecutive = ms.K >= 2 && ms.K <= nrm::kMsStripMaxScales;
   for (int i = 0; i < ms.K; ++i) consecutive = consecutive && ms.alpha[i] == i + 1;
-  const BatchPlan plan = {ms.alpha_max, consecutive, nrm::ms_strip_tile_y(), 0, TX, TY, ms.K,
+  const BatchPlan plan = {ms.alpha_max, consecutive, false, nrm::ms_strip_tile_y(), 0, TX, TY, ms.K,
                           scales->form == NRM_MS_QUAD ? 4.0 : 1.0};
   const nrm::Globals g = make_globals(h);
   std::vector<FrameDesc>& fd = h->scratch_desc;
