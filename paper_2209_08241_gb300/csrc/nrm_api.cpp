@@ -1026,6 +1026,30 @@ BatchPlan forward_plan(const nrm_handle* h, const nrm_frame* frames, int n) {
   return plan;
 }
 
+// True if the multi-scale strip kernel pays for the aligned frames of a batch (plan:
+// of scales 1..K). Its tiles are large (128 x 64, one CTA per SM) and fully unrolled
+// over the scales, so it needs most of an SM each before it is ahead of the run-time
+// kernel (float4, us, strip / run-time: one 640x480 frame, 40 tiles, pair of 4 scales
+// 6.4 / 4.9, quad of 6 8.1 / 5.6; two 6.7 / 6.1, 8.0 / 7.0; one 1280x720, 120 tiles,
+// 6.6 / 7.3, 8.2 / 8.8; four 640x480, 160 tiles, 9.1 / 9.9, quad of 6 from float32
+// 11.8 / 10.7; sixteen 19.8 / 26.7, 27.9 / 35.5), and more in a batch with other
+// frames, where it is a second launch (7 of 640x480 and one of 641x481, 280 tiles, pair
+// of 2 scales 15.0 / 14.2; one of 1920x1080 and one of 1921x1081 19.2 / 18.1).
+bool ms_strip_pays(const nrm_handle* h, const nrm_frame* frames, int n, const BatchPlan& plan) {
+  long long tiles = 0;
+  bool rest = false;
+  for (int i = 0; i < n; ++i) {
+    const nrm_frame& f = frames[i];
+    if ((long long)f.H * f.W == 0) continue;
+    if (strip_aligned(h, f, plan))
+      tiles += (long long)((f.W + nrm::kStripX - 1) / nrm::kStripX) * ((f.H + plan.strip_y - 1) / plan.strip_y);
+    else
+      rest = true;
+  }
+  const bool wide = plan.q == 4.0 && plan.scales >= 5;  // four directions, five scales and more
+  return 3 * tiles >= (long long)h->sm_count * (rest ? 8 : wide ? 6 : 2);
+}
+
 // One part's header and tile offsets (tile_begin: n + 1 entries).
 void fill_work_list(const BatchPart& p, FrameDesc* fd, nrm::BatchHeader* hdr, int* tile_begin) {
   std::memset(hdr, 0, sizeof(*hdr));
@@ -1755,7 +1779,7 @@ int nrm_estimate_batched_multiscale(nrm_handle* h, const nrm_frame* frames, int 
   }
   bool consecutive = ms.K >= 2 && ms.K <= nrm::kMsStripMaxScales;
   for (int i = 0; i < ms.K; ++i) consecutive = consecutive && ms.alpha[i] == i + 1;
-  const BatchPlan plan = {ms.alpha_max, consecutive, false, nrm::ms_strip_tile_y(), 0, TX, TY, ms.K,
+  BatchPlan plan = {ms.alpha_max, false, false, nrm::ms_strip_tile_y(), 0, TX, TY, ms.K,
                           scales->form == NRM_MS_QUAD ? 4.0 : 1.0};
   const nrm::Globals g = make_globals(h);
   std::vector<FrameDesc>& fd = h->scratch_desc;
@@ -1763,7 +1787,9 @@ int nrm_estimate_batched_multiscale(nrm_handle* h, const nrm_frame* frames, int 
   int tiles = 0;
   for (int first = 0; first < n; first += nrm::kParamMaxFrames) {
     BatchPart part[2];
-    split_batch(h, frames + first, std::min(n - first, nrm::kParamMaxFrames), plan, fd.data(), part);
+    const int m = std::min(n - first, nrm::kParamMaxFrames);
+    plan.strip = consecutive && ms_strip_pays(h, frames + first, m, plan);
+    split_batch(h, frames + first, m, plan, fd.data(), part);
     for (int k = 0; k < 2; ++k) {
       const BatchPart& p = part[k];
       tiles += p.tiles;
