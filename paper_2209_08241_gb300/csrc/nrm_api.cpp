@@ -1034,7 +1034,8 @@ BatchPlan forward_plan(const nrm_handle* h, const nrm_frame* frames, int n) {
 // 6.6 / 7.3, 8.2 / 8.8; four 640x480, 160 tiles, 9.1 / 9.9, quad of 6 from float32
 // 11.8 / 10.7; sixteen 19.8 / 26.7, 27.9 / 35.5), and more in a batch with other
 // frames, where it is a second launch (7 of 640x480 and one of 641x481, 280 tiles, pair
-// of 2 scales 15.0 / 14.2; one of 1920x1080 and one of 1921x1081 19.2 / 18.1).
+// of 2 scales 15.0 / 14.2; one of 1920x1080 and one of 1921x1081 19.2 / 18.1) or, past
+// the parameter block's frames, several.
 bool ms_strip_pays(const nrm_handle* h, const nrm_frame* frames, int n, const BatchPlan& plan) {
   long long tiles = 0;
   bool rest = false;
@@ -1047,7 +1048,7 @@ bool ms_strip_pays(const nrm_handle* h, const nrm_frame* frames, int n, const Ba
       rest = true;
   }
   const bool wide = plan.q == 4.0 && plan.scales >= 5;  // four directions, five scales and more
-  return 3 * tiles >= (long long)h->sm_count * (rest ? 8 : wide ? 6 : 2);
+  return 3 * tiles >= (long long)h->sm_count * (rest || n > nrm::kParamMaxFrames ? 8 : wide ? 6 : 2);
 }
 
 // One part's header and tile offsets (tile_begin: n + 1 entries).
@@ -1769,45 +1770,69 @@ int nrm_estimate_batched_multiscale(nrm_handle* h, const nrm_frame* frames, int 
   const bool captured = capture == cudaStreamCaptureStatusActive;
   if (captured && n > nrm::kParamMaxFrames)
     return fail(NRM_ERR_UNSUPPORTED, "at most %d frames per call during stream capture", nrm::kParamMaxFrames);
-  // A ring slot supplies the completion event; the descriptors travel as the
-  // kernel parameter, kParamMaxFrames frames to a launch.
+  // A ring slot supplies the completion event and, past the parameter block's frames,
+  // the memory for the descriptors.
+  const bool ring = n > nrm::kParamMaxFrames;
   Slot* sp = nullptr;
   if (!captured) {
     sp = &h->slots[h->next_slot];
     h->next_slot = (h->next_slot + 1) % kSlots;
     NRM_CHECK(retire_slot(h, *sp));
+    if (ring) NRM_CHECK(ensure_slot_capacity(h, *sp, n));
+  }
+  char* base = ring ? static_cast<char*>(sp->host) : nullptr;
+  FrameDesc* fd = nullptr;
+  if (ring) {
+    fd = reinterpret_cast<FrameDesc*>(base + nrm::frames_offset(sp->capacity));
+  } else {
+    if (h->scratch_desc.size() < (size_t)n) h->scratch_desc.resize((size_t)n);
+    fd = h->scratch_desc.data();
   }
   bool consecutive = ms.K >= 2 && ms.K <= nrm::kMsStripMaxScales;
   for (int i = 0; i < ms.K; ++i) consecutive = consecutive && ms.alpha[i] == i + 1;
   BatchPlan plan = {ms.alpha_max, false, false, nrm::ms_strip_tile_y(), 0, TX, TY, ms.K,
-                          scales->form == NRM_MS_QUAD ? 4.0 : 1.0};
+                    scales->form == NRM_MS_QUAD ? 4.0 : 1.0};
+  plan.strip = consecutive && ms_strip_pays(h, frames, n, plan);
+  BatchPart part[2];
+  split_batch(h, frames, n, plan, fd, part);
   const nrm::Globals g = make_globals(h);
-  std::vector<FrameDesc>& fd = h->scratch_desc;
-  if (fd.size() < (size_t)std::min(n, nrm::kParamMaxFrames)) fd.resize((size_t)std::min(n, nrm::kParamMaxFrames));
-  int tiles = 0;
-  for (int first = 0; first < n; first += nrm::kParamMaxFrames) {
-    BatchPart part[2];
-    const int m = std::min(n - first, nrm::kParamMaxFrames);
-    plan.strip = consecutive && ms_strip_pays(h, frames + first, m, plan);
-    split_batch(h, frames + first, m, plan, fd.data(), part);
-    for (int k = 0; k < 2; ++k) {
-      const BatchPart& p = part[k];
-      tiles += p.tiles;
-      if (p.tiles == 0) continue;
-      void* pb = pack_part(h->scratch_tb, h->scratch_param, p, fd.data());
-      if (k == 0)
-        NRM_CUDA(nrm::launch_multiscale_strip(ms, g, h->p.out_dtype, scales->form, p.tiles, p.u16, st, pb),
-                 "launch fwd_ms_strip_kernel");
-      else
-        NRM_CUDA(nrm::launch_multiscale_batched(ms, g, h->p.out_dtype, scales->form, p.tiles, p.u16, st, pb),
-                 "launch fwd_ms_persistent_param_kernel");
+  // The strip kernel's frames, a parameter block at a time.
+  for (int first = 0; first < part[0].n; first += nrm::kParamMaxFrames) {
+    BatchPart p = part[0];
+    p.first = first;
+    p.n = std::min(part[0].n - first, nrm::kParamMaxFrames);
+    p.tiles = 0;
+    for (int i = 0; i < p.n; ++i) p.tiles += fd[first + i].tiles_x * ((fd[first + i].H + p.tile_y - 1) / p.tile_y);
+    void* pb = pack_part(h->scratch_tb, h->scratch_param, p, fd);
+    NRM_CUDA(nrm::launch_multiscale_strip(ms, g, h->p.out_dtype, scales->form, p.tiles, p.u16, st, pb),
+             "launch fwd_ms_strip_kernel");
+  }
+  // The others: one launch, their descriptors as the parameter block or uploaded.
+  const BatchPart& rest = part[1];
+  if (rest.tiles > 0) {
+    nrm::BatchArgs args;
+    std::memset(&args, 0, sizeof(args));
+    void* pb = nullptr;
+    if (ring) {
+      fill_work_list(rest, fd, reinterpret_cast<nrm::BatchHeader*>(base),
+                     reinterpret_cast<int*>(base + nrm::kTileBeginOffset));
+      const size_t used = nrm::frames_offset(sp->capacity) + sizeof(FrameDesc) * (size_t)n;
+      NRM_CUDA(cudaMemcpyAsync(sp->dev, sp->host, used, cudaMemcpyHostToDevice, st), "cudaMemcpyAsync");
+      const char* dbase = static_cast<const char*>(sp->dev);
+      args.hdr = reinterpret_cast<const nrm::BatchHeader*>(dbase);
+      args.tile_begin = reinterpret_cast<const int*>(dbase + nrm::kTileBeginOffset);
+      args.frames = reinterpret_cast<const FrameDesc*>(dbase + nrm::frames_offset(sp->capacity)) + rest.first;
+    } else {
+      pb = pack_part(h->scratch_tb, h->scratch_param, rest, fd);
     }
+    NRM_CUDA(nrm::launch_multiscale_batched(args, ms, g, h->p.out_dtype, scales->form, rest.tiles, rest.u16, st, pb),
+             "launch fwd_ms_persistent_kernel");
   }
   if (sp) {
     NRM_CUDA(cudaEventRecord(sp->done, st), "cudaEventRecord");
     sp->in_flight = true;
     sp->timed_launch = false;
-    sp->tiles = tiles;
+    sp->tiles = part[0].tiles + rest.tiles;
   }
   return NRM_OK;
 }

@@ -303,14 +303,17 @@ struct MsConsts {
 // (kMsTileY + 2 alpha_max) (or fd.use_tma = 0).
 cudaError_t launch_multiscale(const FrameDesc& fd, const MsConsts& ms, const Globals& g, int out_dtype, int form,
                               cudaStream_t stream);
-// The batched form: one persistent launch over the work list of a ParamBatch
-// packed by pack_param_batch. Each frame's a, b, c hold its bases
-// s^2 / (q fy K), s^2 / (q fx K), s^2 / (q fx fy K) (s the depth scale, q = 1 for
-// NRM_MS_PAIR and 4 for NRM_MS_QUAD); ms.A, ms.B, ms.C are not used. u16: every
-// frame is uint16.
+// The batched form: one persistent launch over a work list (stages and stage bytes are
+// set here). Each frame's a, b, c hold its bases s^2 / (q fy K), s^2 / (q fx K),
+// s^2 / (q fx fy K) (s the depth scale, q = 1 for NRM_MS_PAIR and 4 for
+// NRM_MS_QUAD); ms.A, ms.B, ms.C are not used. u16: every frame is uint16.
 constexpr int kMsStages = 3;
-cudaError_t launch_multiscale_batched(const MsConsts& ms, const Globals& g, int out_dtype, int form, int total_tiles,
-                                      bool u16, cudaStream_t stream, void* param_block);
+// param_block: a ParamBatch packed by pack_param_batch (batches of at most
+// kParamMaxFrames frames; args' pointers are then unused), or NULL for the
+// device descriptor block in args.
+cudaError_t launch_multiscale_batched(const BatchArgs& args, const MsConsts& ms, const Globals& g, int out_dtype,
+                                      int form, int total_tiles, bool u16, cudaStream_t stream,
+                                      const void* param_block = nullptr);
 // The same by the strip kernels (nrm_multiscale_strip.cu), for the distances
 // 1..K, 2 <= K <= kMsStripMaxScales, and tiles of kStripX x ms_strip_tile_y().
 constexpr int kMsStripMaxScales = 6;

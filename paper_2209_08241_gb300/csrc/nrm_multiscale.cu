@@ -15,12 +15,14 @@
 // fwd_ms_kernel: one CTA per 128 x 16 tile of one frame, with a halo of the
 // largest scale, staged by TMA (or plain loads) and decoded once; the
 // per-pixel work is K stencil evaluations from shared memory.
-// fwd_ms_persistent_param_kernel: the batched form, on the persistent pipeline
-// of the single-scale batched kernel (producer warp, TMA stage ring), with the
-// descriptor block as the kernel parameter; each frame's descriptor carries its
-// base constants a, b, c (see launch_multiscale_batched), scaled per scale by
-// alpha_i and alpha_i^2. It takes what the strip kernels (nrm_multiscale_strip.cu)
-// do not: other distance sets and frames without aligned rows.
+// fwd_ms_persistent_param_kernel / fwd_ms_persistent_kernel: the batched form, on the
+// persistent pipeline of the single-scale batched kernel (producer warp, TMA stage
+// ring), with the descriptor block as the kernel parameter or, past its 100 frames,
+// in global memory (one launch: 256 frames of 64x48 or 65x49 29-32 us a call, as
+// launches of 100 frames 33-39); each frame's descriptor carries its base constants
+// a, b, c (see launch_multiscale_batched), scaled per scale by alpha_i and
+// alpha_i^2. They take what the strip kernels (nrm_multiscale_strip.cu) do not: other
+// distance sets, frames without aligned rows, and batches too small for their tiles.
 #include <algorithm>
 #include <atomic>
 
@@ -209,6 +211,15 @@ __global__ void __launch_bounds__(NT + 32, kMsCtasPerSm)
   persistent_pipeline<TX, TY, NT, decltype(compute), false>(args, g, compute);
 }
 
+template <int OUT, int FORM>
+__global__ void __launch_bounds__(NT + 32, kMsCtasPerSm)
+    fwd_ms_persistent_kernel(const BatchArgs args, const __grid_constant__ MsConsts ms, const Globals g) {
+  persistent_pipeline<TX, TY, NT>(args, g,
+                                  [&](const float* F, int fw, int pad4, const TileFrame& tf, int gx0, int gy0) {
+                                    ms_tile<OUT, FORM>(ms, g, F, fw, pad4, tf, gx0, gy0);
+                                  });
+}
+
 const void* ms_persistent_param_kernel(int out_dtype, int form) {
   static const void* k[3][2] = {
       {(const void*)fwd_ms_persistent_param_kernel<NRM_OUT_F32X4, NRM_MS_PAIR>,
@@ -217,6 +228,17 @@ const void* ms_persistent_param_kernel(int out_dtype, int form) {
        (const void*)fwd_ms_persistent_param_kernel<NRM_OUT_F16X4, NRM_MS_QUAD>},
       {(const void*)fwd_ms_persistent_param_kernel<NRM_OUT_OCT16, NRM_MS_PAIR>,
        (const void*)fwd_ms_persistent_param_kernel<NRM_OUT_OCT16, NRM_MS_QUAD>}};
+  return k[out_dtype][form];
+}
+
+const void* ms_persistent_kernel(int out_dtype, int form) {
+  static const void* k[3][2] = {
+      {(const void*)fwd_ms_persistent_kernel<NRM_OUT_F32X4, NRM_MS_PAIR>,
+       (const void*)fwd_ms_persistent_kernel<NRM_OUT_F32X4, NRM_MS_QUAD>},
+      {(const void*)fwd_ms_persistent_kernel<NRM_OUT_F16X4, NRM_MS_PAIR>,
+       (const void*)fwd_ms_persistent_kernel<NRM_OUT_F16X4, NRM_MS_QUAD>},
+      {(const void*)fwd_ms_persistent_kernel<NRM_OUT_OCT16, NRM_MS_PAIR>,
+       (const void*)fwd_ms_persistent_kernel<NRM_OUT_OCT16, NRM_MS_QUAD>}};
   return k[out_dtype][form];
 }
 
@@ -256,19 +278,21 @@ cudaError_t launch_multiscale(const FrameDesc& fd, const MsConsts& ms, const Glo
   return e;
 }
 
-cudaError_t launch_multiscale_batched(const MsConsts& ms, const Globals& g, int out_dtype, int form, int total_tiles,
-                                      bool u16, cudaStream_t stream, void* param_block) {
+cudaError_t launch_multiscale_batched(const BatchArgs& args, const MsConsts& ms, const Globals& g, int out_dtype,
+                                      int form, int total_tiles, bool u16, cudaStream_t stream,
+                                      const void* param_block) {
   if (out_dtype < 0 || out_dtype > 2 || form < 0 || form > 1) return cudaErrorInvalidValue;
-  const void* fn = ms_persistent_param_kernel(out_dtype, form);
-  static std::atomic<bool> granted[3][2][64];
+  const bool param = param_block != nullptr;
+  const void* fn = param ? ms_persistent_param_kernel(out_dtype, form) : ms_persistent_kernel(out_dtype, form);
+  static std::atomic<bool> granted[2][3][2][64];
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   if (dev < 0 || dev >= 64) dev = 63;
-  if (!granted[out_dtype][form][dev].load()) {
+  if (!granted[param][out_dtype][form][dev].load()) {
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)persistent_smem_bytes(TX, TY, NRM_MAX_ALPHA, kMsStages));
     if (e != cudaSuccess) return e;
-    granted[out_dtype][form][dev].store(true);
+    granted[param][out_dtype][form][dev].store(true);
   }
   const unsigned smem = persistent_smem_bytes(TX, TY, ms.alpha_max, kMsStages, u16 ? 2 : 0);
   int occ = 0;
@@ -280,14 +304,18 @@ cudaError_t launch_multiscale_batched(const MsConsts& ms, const Globals& g, int 
   // stencils per pixel make this kernel issue-bound rather than HBM-bound, and
   // the extra warps hide the shared-memory and arithmetic latencies.
   const int grid = std::min(total_tiles, std::min(occ, kMsCtasPerSm) * sms);
-  BatchArgs a = {};
+  BatchArgs a = args;
   a.stages = kMsStages;
   a.stage_bytes = stage_bytes_for(TX, TY, ms.alpha_max, u16 ? 2 : 0);
   MsConsts m = ms;
   Globals gg = g;
   gg.alpha = ms.alpha_max;
-  void* pargs[4] = {param_block, &a, &m, &gg};
-  return cudaLaunchKernel(fn, dim3(grid), dim3(persistent_threads(NT)), pargs, smem, stream);
+  if (param) {
+    void* pargs[4] = {const_cast<void*>(param_block), &a, &m, &gg};
+    return cudaLaunchKernel(fn, dim3(grid), dim3(persistent_threads(NT)), pargs, smem, stream);
+  }
+  void* kargs[3] = {&a, &m, &gg};
+  return cudaLaunchKernel(fn, dim3(grid), dim3(persistent_threads(NT)), kargs, smem, stream);
 }
 
 }  // namespace nrm

@@ -185,9 +185,9 @@ cudaError_t launch_forward_strip(const BatchArgs& a, const Globals&, int, int ti
 cudaError_t launch_multiscale(const FrameDesc&, const MsConsts&, const Globals&, int, int, cudaStream_t) {
   return launched("ms_plain");
 }
-cudaError_t launch_multiscale_batched(const MsConsts&, const Globals&, int, int, int tiles, bool, cudaStream_t,
-                                      void* pb) {
-  const BatchHeader* hdr = static_cast<const BatchHeader*>(pb);
+cudaError_t launch_multiscale_batched(const BatchArgs& a, const MsConsts&, const Globals&, int, int, int tiles, bool,
+                                      cudaStream_t, const void* pb) {
+  const BatchHeader* hdr = pb ? static_cast<const BatchHeader*>(pb) : a.hdr;
   if (hdr->total_tiles != tiles) abort();
   return launched(describe("ms_tiled", hdr));
 }

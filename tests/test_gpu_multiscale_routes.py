@@ -6,7 +6,7 @@ import pytest
 import torch
 
 import paper_2209_08241_gb300 as nrm
-from test_gpu_strip import DEV, depth
+from test_gpu_strip import DEV, assert_same, depth
 from test_gpu_strip_routes import OUT, Buffers, bits, cameras
 
 pytestmark = pytest.mark.gpu
@@ -33,3 +33,24 @@ def test_same_bits(form, K, out):
             buf.check_gaps((form, K, out, mask))
         for i, ((n1, m1), (n2, m2)) in enumerate(zip(*got)):
             assert torch.equal(m1, m2) and torch.equal(n1, n2), (form, K, out, mask, i)
+
+
+@pytest.mark.parametrize("form", ["pair", "quad"])
+@pytest.mark.parametrize("big", [False, True])
+def test_more_frames_than_the_parameter_block(form, big):
+    """Aligned and other frames, empty ones among them: the run-time kernel alone, or
+    strip launches of 100 frames and one launch for the rest, against the same frames
+    in batches of one."""
+    gen = torch.Generator(device=DEV)
+    gen.manual_seed(11)
+    sizes = [(64 + 8 * (i % 5) + (i % 3 == 0), 20 + i % 29 if i % 31 else 0) for i in range(230)]
+    items = [(depth(W, max(H, 1), "u16" if i % 2 else "f32", gen)[:H], cameras(W, max(H, 1)))
+             for i, (W, H) in enumerate(sizes)]
+    if big:
+        items.insert(150, (depth(2048, 2049, "u16", gen), cameras(2048, 2049)))
+        items.insert(7, (depth(1920, 1081, "f32", gen), cameras(1920, 1081)))
+    b = nrm.BatchedEstimator()
+    one = b.multiscale(items, (1, 2, 3), form)
+    two = [b.multiscale([it], (1, 2, 3), form)[0] for it in items]
+    b.sync_status()
+    assert_same(one, two, (form, big))

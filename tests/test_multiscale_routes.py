@@ -48,6 +48,17 @@ def test_mixed_batches(capture, other):
     assert launches(batch, range(1, 5), "quad", capture=capture) == [("ms_strip", 7), ("ms_tiled", 1)]
 
 
+def test_batches_past_the_parameter_block():
+    """The run-time kernel takes any number of frames in one launch, the strip kernel
+    100 a launch."""
+    assert launches([aligned(64, 48)] * 256, (1, 3)) == [("ms_tiled", 256)]
+    assert launches([aligned(64, 48)] * 256, range(1, 5)) == [("ms_tiled", 256)]
+    assert launches([plain(65, 49)] * 101, range(1, 5)) == [("ms_tiled", 101)]
+    assert launches([aligned()] * 130, range(1, 5)) == [("ms_strip", 100), ("ms_strip", 30)]
+    assert launches(([aligned()] * 2 + [plain()]) * 60, range(1, 5)) == [("ms_strip", 100), ("ms_strip", 20),
+                                                                        ("ms_tiled", 60)]
+
+
 def test_other_distances_and_frames():
     big = [aligned(1920, 1080)] * 4
     for alphas in ((1, 3), (2, 1), (1,), (2, 3, 4), range(1, 8), range(1, 9)):
@@ -64,5 +75,8 @@ def test_the_bit_comparisons_reach_the_strip_kernel(form):
     for K in range(2, 7):
         batch = [aligned(W, H, F32 if t == "f32" else 1) for W, H in gpu.SIZES for t in eb if W * eb[t] % 16 == 0]
         assert launches(batch, range(1, K + 1), form) == [("ms_strip", len(batch))]
+        times = -(-101 // len(batch))
+        got = launches(batch * times, range(1, K + 1), form)
+        assert {k for k, _ in got} == {"ms_strip"} and sum(n for _, n in got) == len(batch) * times
         small = [aligned(W, H) for W, H in gpu.SMALL]
         assert launches(small, range(1, K + 1), form) == [("ms_tiled", len(small))]
