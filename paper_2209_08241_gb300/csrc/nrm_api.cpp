@@ -1240,6 +1240,18 @@ static int estimate_batched_param(nrm_handle* h, const nrm_frame* frames, int n,
   return NRM_OK;
 }
 
+// Ends a call that uploaded slot s's block on st (rc: how its launches went): the slot
+// stays in use until st has come this far, also after a failed launch, since the upload
+// and launches before it may still read the block.
+static int finish_slot(Slot& s, cudaStream_t st, int rc, bool timed, int tiles) {
+  const cudaError_t e = cudaEventRecord(s.done, st);
+  s.in_flight = e == cudaSuccess;
+  s.timed_launch = rc == NRM_OK && timed;
+  s.tiles = tiles;
+  if (rc) return rc;
+  return e == cudaSuccess ? NRM_OK : cuda_fail(e, "cudaEventRecord");
+}
+
 // A batch of more than kParamMaxFrames frames of which the strip kernel may take
 // some: one upload of the descriptors into slot s (retired, with capacity n),
 // then a launch per part.
@@ -1254,23 +1266,22 @@ static int estimate_batched_ring(nrm_handle* h, const nrm_frame* frames, int n, 
                    reinterpret_cast<int*>(base + off[k] + nrm::kTileBeginOffset));
   const size_t used = nrm::frames_offset(s.capacity) + sizeof(FrameDesc) * (size_t)n;
   NRM_CUDA(cudaMemcpyAsync(s.dev, s.host, used, cudaMemcpyHostToDevice, st), "cudaMemcpyAsync");
-  if (h->timing) NRM_CUDA(cudaEventRecord(s.ev_start, st), "cudaEventRecord");
-  char* dbase = static_cast<char*>(s.dev);
-  for (int k = 0; k < 2; ++k) {
-    if (part[k].tiles == 0) continue;
-    nrm::BatchArgs args;
-    std::memset(&args, 0, sizeof(args));
-    args.hdr = reinterpret_cast<const nrm::BatchHeader*>(dbase + off[k]);
-    args.tile_begin = reinterpret_cast<const int*>(dbase + off[k] + nrm::kTileBeginOffset);
-    args.frames = reinterpret_cast<const FrameDesc*>(dbase + nrm::frames_offset(s.capacity)) + part[k].first;
-    NRM_CHECK(launch_part(h, k == 0, args, part[k], nullptr, st));
-  }
-  if (h->timing) NRM_CUDA(cudaEventRecord(s.ev_end, st), "cudaEventRecord");
-  NRM_CUDA(cudaEventRecord(s.done, st), "cudaEventRecord");
-  s.in_flight = true;
-  s.timed_launch = h->timing;
-  s.tiles = part[0].stat_tiles + part[1].stat_tiles;
-  return NRM_OK;
+  auto launch = [&]() -> int {
+    if (h->timing) NRM_CUDA(cudaEventRecord(s.ev_start, st), "cudaEventRecord");
+    char* dbase = static_cast<char*>(s.dev);
+    for (int k = 0; k < 2; ++k) {
+      if (part[k].tiles == 0) continue;
+      nrm::BatchArgs args;
+      std::memset(&args, 0, sizeof(args));
+      args.hdr = reinterpret_cast<const nrm::BatchHeader*>(dbase + off[k]);
+      args.tile_begin = reinterpret_cast<const int*>(dbase + off[k] + nrm::kTileBeginOffset);
+      args.frames = reinterpret_cast<const FrameDesc*>(dbase + nrm::frames_offset(s.capacity)) + part[k].first;
+      NRM_CHECK(launch_part(h, k == 0, args, part[k], nullptr, st));
+    }
+    if (h->timing) NRM_CUDA(cudaEventRecord(s.ev_end, st), "cudaEventRecord");
+    return NRM_OK;
+  };
+  return finish_slot(s, st, launch(), h->timing, part[0].stat_tiles + part[1].stat_tiles);
 }
 
 int nrm_estimate_batched(nrm_handle* h, const nrm_frame* frames, int n, void* cuda_stream) {
@@ -1825,16 +1836,11 @@ int nrm_estimate_batched_multiscale(nrm_handle* h, const nrm_frame* frames, int 
     } else {
       pb = pack_part(h->scratch_tb, h->scratch_param, rest, fd);
     }
-    NRM_CUDA(nrm::launch_multiscale_batched(args, ms, g, h->p.out_dtype, scales->form, rest.tiles, rest.u16, st, pb),
-             "launch fwd_ms_persistent_kernel");
+    const cudaError_t e = nrm::launch_multiscale_batched(args, ms, g, h->p.out_dtype, scales->form, rest.tiles,
+                                                         rest.u16, st, pb);
+    if (e != cudaSuccess) rc = cuda_fail(e, "launch fwd_ms_persistent_kernel");
   }
-  if (sp) {
-    NRM_CUDA(cudaEventRecord(sp->done, st), "cudaEventRecord");
-    sp->in_flight = true;
-    sp->timed_launch = false;
-    sp->tiles = part[0].tiles + rest.tiles;
-  }
-  return NRM_OK;
+  return sp ? finish_slot(*sp, st, rc, false, part[0].tiles + rest.tiles) : rc;
 }
 
 int nrm_estimate_multiscale(nrm_handle* h, const void* depth, void* normals, uint8_t* valid,
