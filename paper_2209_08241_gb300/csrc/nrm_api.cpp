@@ -1930,7 +1930,7 @@ int nrm_plane_fit(nrm_handle* h, const void* depth, float* normals, uint8_t* val
   d.cy = (float)f.K.cy;
   d.in_dtype = f.in_dtype;
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-  NRM_CUDA(nrm::launch_plane_fit(d, radius, h->p.orient_to_camera ? -1.0f : 1.0f, st), "launch plane_fit_kernel");
+  NRM_CUDA(nrm::launch_plane_fit(d, radius, h->p.orient_to_camera ? -1.0f : 1.0f, h->sm_count, st), "launch plane_fit_kernel");
   NRM_CHECK(mark_single(h, st));
   return NRM_OK;
 }

@@ -331,7 +331,7 @@ cudaError_t launch_bounds_selftest(int* results, int* status, cudaStream_t strea
 // Plane-fitting ground truth (nrm_planefit.cu): FP32 normals (w = 0) and the
 // validity mask of the (2 radius + 1)^2 window fit; fd.depth, fd.normals,
 // fd.valid, pitches, H, W, cx, cy, inv_fx, inv_fy and in_dtype are used;
-// radius 1..4 (compiled per radius).
-cudaError_t launch_plane_fit(const FrameDesc& fd, int radius, float sign, cudaStream_t stream);
+// radius 1..4 (compiled per radius); sms: the device's SMs.
+cudaError_t launch_plane_fit(const FrameDesc& fd, int radius, float sign, int sms, cudaStream_t stream);
 
 }  // namespace nrm

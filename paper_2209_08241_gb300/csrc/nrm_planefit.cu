@@ -24,56 +24,93 @@
 // one pixel, and the rotations are free of branches: a pixel that is done rotates by
 // zero, which leaves its bits. 1920x1080 float32, R = 2: 49.8 us (one pixel per
 // thread with branching rotations: 68.1); ~31 us is the FMA pipe's time for
-// these operations.
+// these operations. Frames that do not fill the GPU are bound by the chain of one
+// thread, which is shorter with one pixel per thread (launch_plane_fit):
+// 160x120 at R = 1 / 2 / 3 / 4 3.7 / 3.7 / 4.2 / 4.5 us with one, 4.8 / 5.0 / 5.4 / 6.2 with two;
+// 320x240 5.0 / 5.6 / 6.0 / 7.0 and 4.8 / 5.5 / 5.8 / 6.6.
+#include <type_traits>
+
 #include "nrm_device.cuh"
 
 namespace nrm {
 
 namespace {
 
-constexpr int PX = 64, PY = 8, PT = PX / 2 * PY;
+constexpr int PY = 8, PT = 32 * PY;  // rows and threads of a CTA
 
 using dev::f2;
-
 using dev::rsqrt_ftz;
-__device__ __forceinline__ float2 neg(float2 x) { return __fmul2_rn(x, f2(-1.0f, -1.0f)); }
 
-// One Jacobi rotation zeroing a[p][q] of the symmetric matrices a of a pixel
-// pair, accumulated into the eigenvector columns of v. A pixel that is done
+// The values of a thread's N pixels, and the operations on them.
+template <int N>
+using Px = std::conditional_t<N == 2, float2, float>;
+template <int N>
+__device__ __forceinline__ Px<N> all(float x) {
+  if constexpr (N == 2)
+    return f2(x, x);
+  else
+    return x;
+}
+__device__ __forceinline__ float2 add(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float add(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ float2 mul(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float mul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ float2 fma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float fma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ float2 neg(float2 x) { return __fmul2_rn(x, f2(-1.0f, -1.0f)); }
+__device__ __forceinline__ float neg(float x) { return -x; }
+__device__ __forceinline__ float& px(float2& v, int i) { return i ? v.y : v.x; }
+__device__ __forceinline__ float px(const float2& v, int i) { return i ? v.y : v.x; }
+__device__ __forceinline__ float& px(float& v, int) { return v; }
+__device__ __forceinline__ float px(const float& v, int) { return v; }
+
+// One Jacobi rotation zeroing a[p][q] of the symmetric matrices a of a thread's
+// pixels, accumulated into the eigenvector columns of v. A pixel that is done
 // (!on) or whose a[p][q] is nothing takes t = 0, which leaves it bit for bit as it
 // is. Approximate reciprocal and square root suffice: c and s are formed from t
 // so that c^2 + s^2 = 1 to rounding whatever t's last bits, and an error of a few
 // ulp in t only leaves an off-diagonal residue of a few ulp of |a_pq|, the size
 // of the rounding already in S. (|theta| is capped at 1e18, where theta^2 would
 // come near overflow and t is nothing beside 1.)
-template <int p, int q>
-__device__ __forceinline__ void jacobi_rotate(float2 (&a)[3][3], float2 (&v)[3][3], bool on0, bool on1) {
-  const float2 apq = a[p][q];
+template <int p, int q, int N>
+__device__ __forceinline__ void jacobi_rotate(Px<N> (&a)[3][3], Px<N> (&v)[3][3], const bool (&on)[N]) {
+  using V = Px<N>;
+  const V apq = a[p][q], one = all<N>(1.0f);
   // t = tan of the rotation angle, the smaller root of t^2 + 2 theta t - 1 = 0.
-  const float2 den = __fadd2_rn(apq, apq);
-  const float2 num = __ffma2_rn(f2(-1.0f, -1.0f), a[p][p], a[q][q]);
-  const float2 theta = __fmul2_rn(num, f2(dev::rcp_ftz(den.x), dev::rcp_ftz(den.y)));
-  const float2 at = f2(fminf(fabsf(theta.x), 1e18f), fminf(fabsf(theta.y), 1e18f));
-  const float2 h = __ffma2_rn(at, at, f2(1.0f, 1.0f));
-  const float2 d = __ffma2_rn(h, f2(rsqrt_ftz(h.x), rsqrt_ftz(h.y)), at);
-  float2 t = f2(copysignf(dev::rcp_ftz(d.x), theta.x), copysignf(dev::rcp_ftz(d.y), theta.y));
-  t.x = on0 && fabsf(apq.x) >= 1e-35f ? t.x : 0.0f;
-  t.y = on1 && fabsf(apq.y) >= 1e-35f ? t.y : 0.0f;
-  const float2 g = __ffma2_rn(t, t, f2(1.0f, 1.0f));
-  const float2 c = f2(rsqrt_ftz(g.x), rsqrt_ftz(g.y));
-  const float2 s = __fmul2_rn(t, c), ns = neg(s);
-  a[p][p] = __ffma2_rn(neg(t), apq, a[p][p]);
-  a[q][q] = __ffma2_rn(t, apq, a[q][q]);
-  a[p][q] = a[q][p] = f2(0.0f, 0.0f);
-  constexpr int r = 3 - p - q;
-  const float2 arp = a[r][p], arq = a[r][q];
-  a[r][p] = a[p][r] = __ffma2_rn(c, arp, __fmul2_rn(ns, arq));
-  a[r][q] = a[q][r] = __ffma2_rn(c, arq, __fmul2_rn(s, arp));
+  const V den = add(apq, apq);
+  const V num = fma(all<N>(-1.0f), a[p][p], a[q][q]);
+  V r, at, t;
+#pragma unroll
+  for (int i = 0; i < N; ++i) px(r, i) = dev::rcp_ftz(px(den, i));
+  const V theta = mul(num, r);
+#pragma unroll
+  for (int i = 0; i < N; ++i) px(at, i) = fminf(fabsf(px(theta, i)), 1e18f);
+  const V h = fma(at, at, one);
+#pragma unroll
+  for (int i = 0; i < N; ++i) px(r, i) = rsqrt_ftz(px(h, i));
+  const V d = fma(h, r, at);
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    px(t, i) = copysignf(dev::rcp_ftz(px(d, i)), px(theta, i));
+    px(t, i) = on[i] && fabsf(px(apq, i)) >= 1e-35f ? px(t, i) : 0.0f;
+  }
+  const V g = fma(t, t, one);
+  V c;
+#pragma unroll
+  for (int i = 0; i < N; ++i) px(c, i) = rsqrt_ftz(px(g, i));
+  const V s = mul(t, c), ns = neg(s);
+  a[p][p] = fma(neg(t), apq, a[p][p]);
+  a[q][q] = fma(t, apq, a[q][q]);
+  a[p][q] = a[q][p] = all<N>(0.0f);
+  constexpr int o = 3 - p - q;
+  const V aop = a[o][p], aoq = a[o][q];
+  a[o][p] = a[p][o] = fma(c, aop, mul(ns, aoq));
+  a[o][q] = a[q][o] = fma(c, aoq, mul(s, aop));
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
-    const float2 vkp = v[k][p], vkq = v[k][q];
-    v[k][p] = __ffma2_rn(c, vkp, __fmul2_rn(ns, vkq));
-    v[k][q] = __ffma2_rn(s, vkp, __fmul2_rn(c, vkq));
+    const V vkp = v[k][p], vkq = v[k][q];
+    v[k][p] = fma(c, vkp, mul(ns, vkq));
+    v[k][q] = fma(s, vkp, mul(c, vkq));
   }
 }
 
@@ -98,13 +135,16 @@ __device__ __forceinline__ float4 smallest(const float (&d)[3], const float (&v)
   return valid ? make_float4(nx * o, ny * o, nz * o, 0.0f) : make_float4(0.f, 0.f, 0.f, 0.f);
 }
 
-template <int R>
+// N adjacent pixels per thread.
+template <int R, int N>
 __global__ void __launch_bounds__(PT)
     plane_fit_kernel(const __grid_constant__ FrameDesc fd, float sign) {
-  // The decoded halo tile, and the same shifted by one column: a thread's two
-  // depths at any offset are one aligned 8-byte load of one of the two.
+  using V = Px<N>;
+  constexpr int PX = 32 * N;
+  // The decoded halo tile and, for two pixels, the same shifted by one column: a
+  // thread's two depths at any offset are one aligned 8-byte load of one of the two.
   constexpr int tw = PX + 2 * R, th = PY + 2 * R;
-  __shared__ __align__(16) float tile[2][th * tw];
+  __shared__ __align__(16) float tile[N][th * tw];
   NRM_DEBUG_ENTRY(nullptr);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int x0 = blockIdx.x * PX - R, y0 = blockIdx.y * PY - R;
@@ -122,106 +162,120 @@ __global__ void __launch_bounds__(PT)
                 : dev::decode_depth(__ldg(reinterpret_cast<const float*>(fd.depth) + o + lx));
       if (NRM_IOK(ly * tw + lx, tw * th)) {
         tile[0][ly * tw + lx] = z;
-        if (lx > 0) tile[1][ly * tw + lx - 1] = z;
+        if (N == 2 && lx > 0) tile[N - 1][ly * tw + lx - 1] = z;
       }
     }
   }
   __syncthreads();
-  const int px = blockIdx.x * PX + 2 * lane, py = blockIdx.y * PY + warp;
-  if (px >= fd.W || py >= fd.H) return;
-  // Depths of the pixel pair at window offset (dx, dy).
+  const int col = blockIdx.x * PX + N * lane, py = blockIdx.y * PY + warp;
+  if (col >= fd.W || py >= fd.H) return;
+  // Depths of the thread's pixels at window offset (dx, dy).
   auto at = [&](int dx, int dy) {
-    const int c = R + dx, odd = c & 1;
-    const int i = (warp + R + dy) * tw + 2 * lane + c - odd;
-    if (!NRM_IOK(i + 1, tw * th)) return f2(0.0f, 0.0f);
-    return *reinterpret_cast<const float2*>(&tile[odd][i]);
+    const int c = R + dx, odd = N == 2 ? c & 1 : 0;
+    const int i = (warp + R + dy) * tw + N * lane + c - odd;
+    if (!NRM_IOK(i + N - 1, tw * th)) return all<N>(0.0f);
+    return *reinterpret_cast<const V*>(&tile[odd][i]);
   };
-  const float2 z0 = at(0, 0), nz0 = neg(z0);
-  const float2 u0 = f2(((float)px - fd.cx) * fd.inv_fx, ((float)(px + 1) - fd.cx) * fd.inv_fx);
+  const V z0 = at(0, 0), nz0 = neg(z0);
+  V u0;
+#pragma unroll
+  for (int i = 0; i < N; ++i) px(u0, i) = ((float)(col + i) - fd.cx) * fd.inv_fx;
   const float v0 = ((float)py - fd.cy) * fd.inv_fy;
-  float2 sx = f2(0.f, 0.f), sy = sx, sz = sx;
-  float2 a00 = sx, a01 = sx, a02 = sx, a11 = sx, a12 = sx, a22 = sx;
+  V sx = all<N>(0.f), sy = sx, sz = sx;
+  V a00 = sx, a01 = sx, a02 = sx, a11 = sx, a12 = sx, a22 = sx;
 #pragma unroll
   for (int dy = -R; dy <= R; ++dy) {
     const float e1 = (float)dy * fd.inv_fy, v1 = __fadd_rn(v0, e1);
-    const float2 v = f2(v1, v1), ey = __fmul2_rn(z0, f2(e1, e1));
+    const V v = all<N>(v1), ey = mul(z0, all<N>(e1));
 #pragma unroll
     for (int dx = -R; dx <= R; ++dx) {
-      const float e = (float)dx * fd.inv_fx;
-      const float2 u = __fadd2_rn(u0, f2(e, e));
-      const float2 dz = __fadd2_rn(at(dx, dy), nz0);
-      const float2 qx = __ffma2_rn(dz, u, __fmul2_rn(z0, f2(e, e)));
-      const float2 qy = __ffma2_rn(dz, v, ey);
-      sx = __fadd2_rn(sx, qx);
-      sy = __fadd2_rn(sy, qy);
-      sz = __fadd2_rn(sz, dz);
-      a00 = __ffma2_rn(qx, qx, a00);
-      a01 = __ffma2_rn(qx, qy, a01);
-      a02 = __ffma2_rn(qx, dz, a02);
-      a11 = __ffma2_rn(qy, qy, a11);
-      a12 = __ffma2_rn(qy, dz, a12);
-      a22 = __ffma2_rn(dz, dz, a22);
+      const V e = all<N>((float)dx * fd.inv_fx);
+      const V u = add(u0, e);
+      const V dz = add(at(dx, dy), nz0);
+      const V qx = fma(dz, u, mul(z0, e));
+      const V qy = fma(dz, v, ey);
+      sx = add(sx, qx);
+      sy = add(sy, qy);
+      sz = add(sz, dz);
+      a00 = fma(qx, qx, a00);
+      a01 = fma(qx, qy, a01);
+      a02 = fma(qx, dz, a02);
+      a11 = fma(qy, qy, a11);
+      a12 = fma(qy, dz, a12);
+      a22 = fma(dz, dz, a22);
     }
   }
   // A NaN depth in the window leaves a NaN in the sums.
-  const bool ok0 = fabsf(sx.x) + fabsf(sy.x) + fabsf(sz.x) <= 3.402823466e38f;
-  const bool ok1 = fabsf(sx.y) + fabsf(sy.y) + fabsf(sz.y) <= 3.402823466e38f;
+  bool ok[N], on[N], any = false;
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    ok[i] = on[i] = fabsf(px(sx, i)) + fabsf(px(sy, i)) + fabsf(px(sz, i)) <= 3.402823466e38f;
+    any = any || on[i];
+  }
   constexpr float kInvN = 1.0f / (float)((2 * R + 1) * (2 * R + 1));
-  const float2 inv_n = f2(-kInvN, -kInvN);
-  const float2 mx = __fmul2_rn(sx, inv_n), my = __fmul2_rn(sy, inv_n), mz = __fmul2_rn(sz, inv_n);
-  float2 a[3][3];
-  a[0][0] = __ffma2_rn(mx, sx, a00);
-  a[0][1] = a[1][0] = __ffma2_rn(mx, sy, a01);
-  a[0][2] = a[2][0] = __ffma2_rn(mx, sz, a02);
-  a[1][1] = __ffma2_rn(my, sy, a11);
-  a[1][2] = a[2][1] = __ffma2_rn(my, sz, a12);
-  a[2][2] = __ffma2_rn(mz, sz, a22);
-  float2 vec[3][3];
+  const V inv_n = all<N>(-kInvN);
+  const V mx = mul(sx, inv_n), my = mul(sy, inv_n), mz = mul(sz, inv_n);
+  V a[3][3];
+  a[0][0] = fma(mx, sx, a00);
+  a[0][1] = a[1][0] = fma(mx, sy, a01);
+  a[0][2] = a[2][0] = fma(mx, sz, a02);
+  a[1][1] = fma(my, sy, a11);
+  a[1][2] = a[2][1] = fma(my, sz, a12);
+  a[2][2] = fma(mz, sz, a22);
+  V vec[3][3];
 #pragma unroll
-  for (int k = 0; k < 9; ++k) vec[k / 3][k % 3] = k % 4 ? f2(0.f, 0.f) : f2(1.f, 1.f);
-  bool on0 = ok0, on1 = ok1;
+  for (int k = 0; k < 9; ++k) vec[k / 3][k % 3] = all<N>(k % 4 ? 0.f : 1.f);
 #pragma unroll 1
-  for (int sweep = 0; sweep < 6 && (on0 || on1); ++sweep) {
-    jacobi_rotate<0, 1>(a, vec, on0, on1);
-    jacobi_rotate<0, 2>(a, vec, on0, on1);
-    jacobi_rotate<1, 2>(a, vec, on0, on1);
-    const float2 off = __ffma2_rn(a[0][1], a[0][1], __ffma2_rn(a[0][2], a[0][2], __fmul2_rn(a[1][2], a[1][2])));
-    const float2 diag = __ffma2_rn(a[0][0], a[0][0], __ffma2_rn(a[1][1], a[1][1], __fmul2_rn(a[2][2], a[2][2])));
-    on0 = on0 && !(off.x <= 1e-14f * diag.x);
-    on1 = on1 && !(off.y <= 1e-14f * diag.y);
-  }
-  const float d0[3] = {a[0][0].x, a[1][1].x, a[2][2].x}, d1[3] = {a[0][0].y, a[1][1].y, a[2][2].y};
-  float w0[3][3], w1[3][3];
+  for (int sweep = 0; sweep < 6 && any; ++sweep) {
+    jacobi_rotate<0, 1, N>(a, vec, on);
+    jacobi_rotate<0, 2, N>(a, vec, on);
+    jacobi_rotate<1, 2, N>(a, vec, on);
+    const V off = fma(a[0][1], a[0][1], fma(a[0][2], a[0][2], mul(a[1][2], a[1][2])));
+    const V diag = fma(a[0][0], a[0][0], fma(a[1][1], a[1][1], mul(a[2][2], a[2][2])));
+    any = false;
 #pragma unroll
-  for (int k = 0; k < 9; ++k) {
-    w0[k / 3][k % 3] = vec[k / 3][k % 3].x;
-    w1[k / 3][k % 3] = vec[k / 3][k % 3].y;
+    for (int i = 0; i < N; ++i) {
+      on[i] = on[i] && !(px(off, i) <= 1e-14f * px(diag, i));
+      any = any || on[i];
+    }
   }
-  const long long oo = (long long)py * fd.out_pitch + px;
+  const long long oo = (long long)py * fd.out_pitch + col;
   float4* out = reinterpret_cast<float4*>(fd.normals) + oo;
   uint8_t* mask = fd.valid + oo;
   [[maybe_unused]] const long long nlen = dev::dbg_span(fd.H, fd.W, fd.out_pitch, 16);
   [[maybe_unused]] const long long mlen = dev::dbg_span(fd.H, fd.W, fd.out_pitch, 1);
-  if (NRM_GOK(out, fd.normals, nlen)) *out = smallest(d0, w0, u0.x, v0, sign, ok0);
-  if (NRM_GOK(mask, fd.valid, mlen)) *mask = ok0;
-  if (px + 1 < fd.W) {
-    if (NRM_GOK(out + 1, fd.normals, nlen)) out[1] = smallest(d1, w1, u0.y, v0, sign, ok1);
-    if (NRM_GOK(mask + 1, fd.valid, mlen)) mask[1] = ok1;
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    if (col + i >= fd.W) break;
+    const float d[3] = {px(a[0][0], i), px(a[1][1], i), px(a[2][2], i)};
+    float w[3][3];
+#pragma unroll
+    for (int k = 0; k < 9; ++k) w[k / 3][k % 3] = px(vec[k / 3][k % 3], i);
+    if (NRM_GOK(out + i, fd.normals, nlen)) out[i] = smallest(d, w, px(u0, i), v0, sign, ok[i]);
+    if (NRM_GOK(mask + i, fd.valid, mlen)) mask[i] = ok[i];
+  }
+}
+
+template <int N>
+const void* kernel_for(int radius) {
+  switch (radius) {
+    case 1: return (const void*)plane_fit_kernel<1, N>;
+    case 2: return (const void*)plane_fit_kernel<2, N>;
+    case 3: return (const void*)plane_fit_kernel<3, N>;
+    case 4: return (const void*)plane_fit_kernel<4, N>;
+    default: return nullptr;
   }
 }
 
 }  // namespace
 
-cudaError_t launch_plane_fit(const FrameDesc& fd, int radius, float sign, cudaStream_t stream) {
-  dim3 grid((fd.W + PX - 1) / PX, (fd.H + PY - 1) / PY);
-  const void* fn = nullptr;
-  switch (radius) {
-    case 1: fn = (const void*)plane_fit_kernel<1>; break;
-    case 2: fn = (const void*)plane_fit_kernel<2>; break;
-    case 3: fn = (const void*)plane_fit_kernel<3>; break;
-    case 4: fn = (const void*)plane_fit_kernel<4>; break;
-    default: return cudaErrorInvalidValue;
-  }
+cudaError_t launch_plane_fit(const FrameDesc& fd, int radius, float sign, int sms, cudaStream_t stream) {
+  const int rows = (fd.H + PY - 1) / PY;
+  // One pixel per thread while its CTAs are at most one per SM (see the file comment).
+  const int n = (long long)((fd.W + 31) / 32) * rows <= sms ? 1 : 2;
+  const void* fn = n == 1 ? kernel_for<1>(radius) : kernel_for<2>(radius);
+  if (!fn) return cudaErrorInvalidValue;
+  dim3 grid((fd.W + 32 * n - 1) / (32 * n), rows);
   FrameDesc d = fd;
   float sg = sign;
   void* args[2] = {&d, &sg};

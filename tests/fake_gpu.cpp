@@ -221,6 +221,6 @@ cudaError_t launch_angle_mse(const float*, const uint8_t*, const float*, const u
 }
 cudaError_t launch_wait_expiry(unsigned long long, int*, cudaStream_t) { return cudaErrorNotSupported; }
 cudaError_t launch_bounds_selftest(int*, int*, cudaStream_t) { return cudaErrorNotSupported; }
-cudaError_t launch_plane_fit(const FrameDesc&, int, float, cudaStream_t) { return launched("plane_fit"); }
+cudaError_t launch_plane_fit(const FrameDesc&, int, float, int, cudaStream_t) { return launched("plane_fit"); }
 
 }  // namespace nrm
