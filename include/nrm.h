@@ -375,11 +375,14 @@ NRM_API int nrm_set_config(nrm_handle* h, const nrm_tile_config* cfg);
 /* Times every supported configuration on the given batch (which must stay
  * valid during the call; outputs are overwritten), keeps the fastest in the
  * handle and records it in the JSON cache file cache_path, keyed by GPU name,
- * SM count, frame-size class, dtypes and alpha. cache_path = NULL takes the
+ * SM count, the generation of the library's kernels, frame-size class, dtypes,
+ * alpha and whether the batch writes point clouds. cache_path = NULL takes the
  * process-wide cache file (nrm_set_autotune_cache), if any. If the cache
  * already holds the key, loads it without timing. The tuned configuration is
- * also recorded under the handle's own key (nrm_autotune_key), which
- * nrm_create looks up. Synchronous. */
+ * also recorded under the handle's own key (nrm_autotune_key; "|points" after
+ * it for a batch with point clouds), which nrm_create looks up. Tuning on a
+ * batch with point clouds does not decide which kernels calls without them
+ * take. Synchronous. */
 NRM_API int nrm_autotune(nrm_handle* h, const nrm_frame* frames, int n, void* cuda_stream,
                  const char* cache_path);
 
@@ -403,8 +406,8 @@ NRM_API int nrm_reset_stats(nrm_handle* h);
  * With a cache file set, nrm_create configures a new handle from the entry of
  * its key, if there is one, instead of the default geometry, so a process
  * that tuned a workload once lets later processes skip the sweep.
- * nrm_autotune_key writes a handle's key (GPU name, SM count, input and output
- * dtypes, alpha, H x W of the handle) to buf (NUL-terminated; NRM_ERR_INVALID_ARG
+ * nrm_autotune_key writes a handle's key (GPU name, SM count, kernel generation,
+ * input and output dtypes, alpha, H x W of the handle) to buf (NUL-terminated; NRM_ERR_INVALID_ARG
  * if it does not fit in len bytes). nrm_autotune_cache_get reads the entry of
  * key from the file at path (NRM_ERR_INVALID_ARG if the file or the key is
  * absent or malformed); nrm_autotune_cache_put adds or replaces it (written to

@@ -218,9 +218,17 @@ int validate_intrinsics(const nrm_intrinsics& K) {
 }
 
 constexpr int kSlots = 3;
-// A handle's geometry unless another is asked for. Batched calls of a handle
-// with this geometry take the strip kernels wherever those apply.
+// A handle's geometry unless another is asked for. Asking for this one, or no other,
+// lets calls without point clouds take the strip kernels wherever those apply.
 constexpr nrm_tile_config kDefaultConfig = {128, 16, 256, 3, 0};
+bool is_default(const nrm_tile_config& c) {
+  const nrm_tile_config& d = kDefaultConfig;
+  return c.tile_x == d.tile_x && c.tile_y == d.tile_y && c.threads == d.threads && c.stages == d.stages &&
+         c.ctas_per_sm == d.ctas_per_sm;
+}
+// Part of the autotune cache's keys: raised when the kernels behind a geometry change,
+// so that entries timed on older kernels are not used. 2: the strip kernels.
+constexpr int kKernelGeneration = 2;
 constexpr unsigned long long kDefaultTimeoutNs = 2000000000ull;  // 2 s
 
 struct Slot {
@@ -267,6 +275,7 @@ struct nrm_handle {
   nrm_intrinsics K = {1, 1, 0, 0};
   nrm_params p;
   nrm_tile_config cfg = kDefaultConfig;
+  bool strips = true;  // calls may take the strip kernels: cfg is the default, or was tuned for point clouds
   const FwdKernelSet* ks = nullptr;
   // Persistent grids [u16]: u16 = 1 for batches of uint16 frames only, whose
   // smaller staging buffers let more CTAs share an SM.
@@ -556,6 +565,15 @@ bool write_cache(const char* path, const std::map<std::string, std::string>& m) 
   return std::rename(tmp.c_str(), path) == 0;
 }
 
+bool writes_points(const nrm_frame* f, int n) {
+  for (int i = 0; i < n; ++i)
+    if (f[i].points && (long long)f[i].H * f[i].W > 0) return true;
+  return false;
+}
+constexpr const char* kPointsSuffix = "|points";  // of the keys of geometries tuned for point clouds
+
+// The key of a batch: GPU, SM count, kernel generation, dtypes, alpha, size classes and
+// whether point clouds are written (other kernels write those).
 std::string tune_key(const nrm_handle* h, const nrm_frame* f, int n) {
   long long px = 0;
   int maxw = 0, dtypes = 0;
@@ -572,20 +590,20 @@ std::string tune_key(const nrm_handle* h, const nrm_frame* f, int n) {
   for (auto& ch : name)
     if (ch == '"' || ch == '\\') ch = '_';
   std::ostringstream k;
-  k << name << "|sm" << h->sm_count << "|in" << dtypes << "|out" << h->p.out_dtype << "|a" << h->p.alpha
-    << "|px2^" << lpx << "|w2^" << lw;
+  k << name << "|sm" << h->sm_count << "|k" << kKernelGeneration << "|in" << dtypes << "|out" << h->p.out_dtype << "|a"
+    << h->p.alpha << "|px2^" << lpx << "|w2^" << lw << (writes_points(f, n) ? kPointsSuffix : "");
   return k.str();
 }
 
-// The key of a handle as created: GPU, SM count, input dtype of its params,
-// output dtype, alpha and the handle's frame size (0 x 0 for batch handles).
+// The key of a handle as created: GPU, SM count, kernel generation, input dtype of its
+// params, output dtype, alpha and the handle's frame size (0 x 0 for batch handles).
 std::string handle_key(const nrm_handle* h) {
   std::string name = h->gpu_name;
   for (auto& ch : name)
     if (ch == '"' || ch == '\\') ch = '_';
   std::ostringstream k;
-  k << name << "|sm" << h->sm_count << "|in" << (1 << h->p.in_dtype) << "|out" << h->p.out_dtype << "|a"
-    << h->p.alpha << "|handle" << h->H << "x" << h->W;
+  k << name << "|sm" << h->sm_count << "|k" << kKernelGeneration << "|in" << (1 << h->p.in_dtype) << "|out"
+    << h->p.out_dtype << "|a" << h->p.alpha << "|handle" << h->H << "x" << h->W;
   return k.str();
 }
 
@@ -735,11 +753,18 @@ int nrm_create(const nrm_intrinsics* K, int H, int W, const nrm_params* p, nrm_h
       std::lock_guard<std::mutex> lock(g_tune_mu);
       cache = read_cache(path.c_str());
     }
+    // (A geometry tuned for point clouds leaves the strip kernels to calls without.)
     auto it = cache.find(handle_key(h));
+    const bool points = it == cache.end();
+    if (points) it = cache.find(handle_key(h) + kPointsSuffix);
     nrm_tile_config tuned;
-    if (it != cache.end() && parse_config(it->second, &tuned) && configure(h, tuned) != NRM_OK) {
-      configure(h, c);  // a stale or foreign entry: keep the default geometry
-      g_last_error.clear();
+    if (it != cache.end() && parse_config(it->second, &tuned)) {
+      if (configure(h, tuned) == NRM_OK) {
+        h->strips = points || is_default(tuned);
+      } else {
+        configure(h, c);  // a stale or foreign entry: keep the default geometry
+        g_last_error.clear();
+      }
     }
   }
   *out = h;
@@ -855,11 +880,7 @@ struct BatchPlan {
 };
 
 // True if the handle's batched forward calls may take the strip kernels.
-bool strip_handle(const nrm_handle* h) {
-  const nrm_tile_config &c = h->cfg, &d = kDefaultConfig;
-  return c.tile_x == d.tile_x && c.tile_y == d.tile_y && c.threads == d.threads && c.stages == d.stages &&
-         c.ctas_per_sm == d.ctas_per_sm && h->p.alpha <= nrm::kStripMaxAlpha;
-}
+bool strip_handle(const nrm_handle* h) { return h->strips && h->p.alpha <= nrm::kStripMaxAlpha; }
 
 // True if q >= FLT_MIN for every valid pixel of a uint16 frame, which the strip
 // kernels do not test: with every depth >= 1 unit n . ray is at least pmin, and so
@@ -2004,7 +2025,9 @@ int nrm_get_config(const nrm_handle* h, nrm_tile_config* cfg) {
 int nrm_set_config(nrm_handle* h, const nrm_tile_config* cfg) {
   if (!h || !cfg) return fail(NRM_ERR_INVALID_ARG, "NULL argument");
   DeviceGuard guard(h->device);
-  return configure(h, *cfg);
+  NRM_CHECK(configure(h, *cfg));
+  h->strips = is_default(*cfg);
+  return NRM_OK;
 }
 
 int nrm_enable_timing(nrm_handle* h, int enable) {
@@ -2038,6 +2061,9 @@ int nrm_autotune(nrm_handle* h, const nrm_frame* frames, int n, void* cuda_strea
   DeviceGuard guard(h->device);
   const std::string key = tune_key(h, frames, n);
   const std::string path = tune_path(cache_path);
+  // Batches with point clouds never take the strip kernels, so tuning for them does
+  // not decide about those.
+  const bool points = writes_points(frames, n), strips_before = h->strips;
   std::map<std::string, std::string> cache;
   if (!path.empty()) {
     {
@@ -2046,7 +2072,10 @@ int nrm_autotune(nrm_handle* h, const nrm_frame* frames, int n, void* cuda_strea
     }
     auto it = cache.find(key);
     nrm_tile_config c;
-    if (it != cache.end() && parse_config(it->second, &c) && configure(h, c) == NRM_OK) return NRM_OK;
+    if (it != cache.end() && parse_config(it->second, &c) && configure(h, c) == NRM_OK) {
+      if (!points) h->strips = is_default(c);
+      return NRM_OK;
+    }
   }
   const bool timing_was = h->timing;
   h->timing = false;
@@ -2059,9 +2088,8 @@ int nrm_autotune(nrm_handle* h, const nrm_frame* frames, int n, void* cuda_strea
   float best_ms = INFINITY;
   int rc = NRM_OK;
   // The batch decides which staging size (and so which occupancy) applies.
-  bool points = false, u16 = true;
+  bool u16 = true;
   for (int i = 0; i < n; ++i) {
-    points = points || frames[i].points;
     u16 = u16 && (frames[i].in_dtype == NRM_IN_U16_MM || (long long)frames[i].H * frames[i].W == 0);
   }
   // Candidates: every compiled tile shape x pipeline depth x CTAs per SM from
@@ -2085,6 +2113,7 @@ int nrm_autotune(nrm_handle* h, const nrm_frame* frames, int n, void* cuda_strea
     {
       const nrm_tile_config c = cands[ci];
       if (configure(h, c) != NRM_OK) continue;
+      h->strips = is_default(c);
       for (int w = 0; w < 2 && rc == NRM_OK; ++w) rc = nrm_estimate_batched(h, frames, n, cuda_stream);
       if (rc) break;
       const int reps = 5;
@@ -2108,13 +2137,14 @@ int nrm_autotune(nrm_handle* h, const nrm_frame* frames, int n, void* cuda_strea
   cudaEventDestroy(e1);
   h->timing = timing_was;
   int rc2 = configure(h, rc == NRM_OK ? best : start);
+  h->strips = rc != NRM_OK || points ? strips_before : is_default(best);
   if (rc) return rc;
   if (rc2) return rc2;
   if (!path.empty()) {
     std::lock_guard<std::mutex> lock(g_tune_mu);
     cache = read_cache(path.c_str());  // entries other processes added meanwhile
     cache[key] = format_config(best);
-    cache[handle_key(h)] = format_config(best);
+    cache[handle_key(h) + (points ? kPointsSuffix : "")] = format_config(best);
     write_cache(path.c_str(), cache);
   }
   return NRM_OK;
