@@ -79,22 +79,30 @@ __device__ __forceinline__ float2 atan2_fit2(float2 y, float2 x) {
   return f2(copysignf(r.x, y.x), copysignf(r.y, y.y));
 }
 
-// Hardware square root, flush-to-zero.
-__device__ __forceinline__ float sqrt_ftz(float x) {
-  float y;
-  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
+// Square roots of two values: the hardware's reciprocal square root y, then one Newton
+// step for s^2 = x from s = x y, s + (x - s^2) y / 2, whose residual one FMA gives exactly.
+// The same bits as sqrtf for 0 and for every float from 2^-100 to the largest
+// (compared one by one); below that the angle is off by at most 1.1e-19 rad, and
+// infinity counts as the largest float (the angle is pi / 2 either way). So the MSE is
+// that of the angle images as spherical_kernel forms them, without sqrtf's branch per
+// value: the MSE kernel at 4096 x 3072 takes 77.4 us, with sqrtf 94, with the hardware's
+// approximate square root (other bits for one float in six) 72.8.
+__device__ __forceinline__ float2 sqrt2(float2 x) {
+  using dev::f2;
+  const float kFltMin = 1.17549435e-38f, kFltMax = 3.402823466e38f;
+  x = f2(fminf(x.x, kFltMax), fminf(x.y, kFltMax));
+  const float2 y = f2(dev::rsqrt_ftz(fmaxf(x.x, kFltMin)), dev::rsqrt_ftz(fmaxf(x.y, kFltMin)));
+  const float2 s = __fmul2_rn(x, y), ns = __fmul2_rn(s, f2(-1.0f, -1.0f)), h = __fmul2_rn(y, f2(0.5f, 0.5f));
+  return __ffma2_rn(__ffma2_rn(ns, s, x), h, s);
 }
 
-// The angles of two normals (the lanes of phi and theta), for their difference.
-// The hardware square root's last-place error is the same for both maps: the MSE's
-// error against 64 bits is what it is with sqrtf (4096x3072 3.40e-7 relative, 1080p
-// 4.56e-7 against 4.58e-7), which takes a fifth of the instructions.
+// The angles of two normals (the lanes of phi and theta), operation for operation those
+// of angles().
 __device__ __forceinline__ void angles2(float4 a, float4 b, float2& phi, float2& theta) {
   phi = atan2_fit2(dev::f2(a.y, b.y), dev::f2(a.x, b.x));
   phi.x = phi.x < 0.0f ? phi.x + 6.28318530717958647692f : phi.x;
   phi.y = phi.y < 0.0f ? phi.y + 6.28318530717958647692f : phi.y;
-  theta = atan2_fit2(dev::f2(sqrt_ftz(fmaf(a.x, a.x, a.y * a.y)), sqrt_ftz(fmaf(b.x, b.x, b.y * b.y))), dev::f2(a.z, b.z));
+  theta = atan2_fit2(sqrt2(dev::f2(fmaf(a.x, a.x, a.y * a.y), fmaf(b.x, b.x, b.y * b.y))), dev::f2(a.z, b.z));
 }
 
 constexpr int kSphRows = 4;  // rows per thread of the angle-image kernel
@@ -170,13 +178,13 @@ __device__ __forceinline__ void block_sum3(double& a, double& b, double& c) {
 // loaded a piece ahead. Three CTAs fill an SM; the grid is one wave, so no SM
 // waits for a last partial one. The pieces are taken from the maps' end: what a
 // call before this one read last (the angle images of the same map) is still in
-// L2 (both calls on 4096 x 3072: 128.4 us, from the start 137.2).
+// L2 (both calls on 4096 x 3072: 127.5 us; from the maps' start 9 us more).
 //
-// Bound by issue (about 115 thread instructions per pixel), HBM (34 B/px) close
-// behind. 4096 x 3072: 76.0 us (83 % of the measured copy); before, with a step's
-// loads issued together from global memory, 2048 blocks of rows (3.4 waves), sqrtf
-// and a second kernel for the sums, 93 us. Two CTAs of 3 stages 79 us, four
-// pixels unrolled 81 us, with sqrtf 94 us.
+// Bound by issue, HBM (34 B/px) close behind. 4096 x 3072: 77.4 us (81 % of the
+// measured copy); before, with a step's loads issued together from global memory,
+// 2048 blocks of rows (3.4 waves), sqrtf and a second kernel for the sums, 84.6 us and
+// 29 us for any small map (now 12). Two CTAs of 3 stages 3 us more, four pixels
+// unrolled 5, sqrtf 17.
 constexpr int kMsePiece = 128, kMseStages = 2, kMseWarps = kThreads / 32;
 constexpr unsigned kMseStageBytes = 2 * kMsePiece * 16;
 constexpr unsigned kMseSmem = kMseWarps * kMseStages * (kMseStageBytes + 8);
