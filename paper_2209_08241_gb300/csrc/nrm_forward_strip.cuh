@@ -161,7 +161,7 @@ __device__ __forceinline__ void strip_codes(float2 nx, float2 ny, float2 nz, uin
   cb = __byte_perm(__float_as_uint(x.y), __float_as_uint(y.y), 0x5410);
 }
 
-// A row of one band written at any alignment: the lanes' results go to the warp's
+// A row of one band written at any alignment (float4, half4): the lanes' results go to the warp's
 // row buffer at the offset that the row has in memory modulo 16 bytes (mask:
 // modulo 4), and the warp then copies whole 16-byte (4-byte) units with
 // consecutive lanes, the ragged units at the ends element by element. (One store
@@ -169,12 +169,12 @@ __device__ __forceinline__ void strip_codes(float2 nx, float2 ny, float2 nz, uin
 // sector at a time: 64 x 1921x1081 uint16 -> float4 745 us, half4 755 us with one
 // CTA per SM; through the buffer 646 and 492 us, with two CTAs 487 and 484. The
 // octahedral codes, whose ragged ends would be three of four elements, are faster
-// straight from the lanes: 381 against 581 us.) float4: units are pixels, stored
-// with their index's low bits XORed by bits 3-5, so that neither side has bank
-// conflicts.
+// straight from the lanes: 381 against 581 us, and have no buffer.) float4: units
+// are pixels, stored with their index's low bits XORed by bits 3-5, so that neither
+// side has bank conflicts.
 constexpr int kRowBufMask = 160;  // the mask's part of a row buffer
 NRM_HD constexpr int strip_rowbuf(int out_dtype) {
-  return kRowBufMask + (out_dtype == NRM_OUT_F32X4 ? 2048 : out_dtype == NRM_OUT_F16X4 ? 1040 : 528);
+  return out_dtype == NRM_OUT_OCT16 ? 0 : kRowBufMask + (out_dtype == NRM_OUT_F32X4 ? 2048 : 1040);
 }
 
 // Copies bytes [m, m + len) of buf to the same offsets from base, units of U
@@ -197,9 +197,10 @@ __device__ __forceinline__ void copy_out(const unsigned char* buf, unsigned char
 }
 
 template <int OUT>
-__device__ __forceinline__ void store_row(const uint32_t* w, uint32_t mbits, unsigned char* np, uint8_t* mp, int n,
+__device__ __forceinline__ void store_row(const uint32_t* w, uint32_t mbits, unsigned char* np, uint8_t* mp,
                                           unsigned char* buf, [[maybe_unused]] const StripInfo& f) {
-  constexpr int BPP = OUT == NRM_OUT_F32X4 ? 16 : OUT == NRM_OUT_F16X4 ? 8 : 4;
+  static_assert(OUT == NRM_OUT_F32X4 || OUT == NRM_OUT_F16X4, "octahedral codes are stored from the lanes");
+  constexpr int BPP = OUT == NRM_OUT_F32X4 ? 16 : 8;
   const int lane = threadIdx.x & 31;
   unsigned char* row = np - 4 * lane * BPP;  // the row's first pixel in this tile
   uint8_t* mrow = mp - 4 * lane;
@@ -209,7 +210,6 @@ __device__ __forceinline__ void store_row(const uint32_t* w, uint32_t mbits, uns
         dbg_gmem_ok(mrow, count, f.valid0, f.mlen, "strip mask", __LINE__)))
     return;
 #endif
-  (void)n;
   unsigned char* nbuf = buf + kRowBufMask;
   const int mm = (int)(reinterpret_cast<uintptr_t>(mrow) & 3);
   __syncwarp();  // the previous row has left the buffer
@@ -236,25 +236,17 @@ __device__ __forceinline__ void store_row(const uint32_t* w, uint32_t mbits, uns
   } else {
     const int m = (int)(reinterpret_cast<uintptr_t>(row) & 15);
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      if constexpr (OUT == NRM_OUT_F16X4)
-        NRM_STS(reinterpret_cast<uint2*>(nbuf + m) + 4 * lane + i, make_uint2(w[2 * i], w[2 * i + 1]));
-      else
-        NRM_STS(reinterpret_cast<uint32_t*>(nbuf + m) + 4 * lane + i, w[i]);
-    }
+    for (int i = 0; i < 4; ++i) NRM_STS(reinterpret_cast<uint2*>(nbuf + m) + 4 * lane + i, make_uint2(w[2 * i], w[2 * i + 1]));
     __syncwarp();
-    if constexpr (OUT == NRM_OUT_F16X4)
-      copy_out<16, 8, 1024, uint4, uint2>(nbuf, row - m, m, count * BPP);
-    else
-      copy_out<16, 4, 512, uint4, uint32_t>(nbuf, row - m, m, count * BPP);
+    copy_out<16, 8, 1024, uint4, uint2>(nbuf, row - m, m, count * BPP);
   }
   copy_out<4, 1, 128, uint32_t, uint8_t>(buf, mrow - mm, mm, count);
 }
 
 // The normals (or codes) and mask bytes of a lane's four pixels: np, mp point at
 // the first one's; k[i] says whether pixel i is valid; n > 0 of them lie in the
-// frame. ALIGNED: whole vectors, straight to memory (n >= 4); else through the
-// warp's row buffer (store_row).
+// frame. ALIGNED: whole vectors, straight to memory (n >= 4); else float4 and half4
+// through the warp's row buffer (store_row), octahedral codes one by one.
 template <int OUT, bool ALIGNED>
 __device__ __forceinline__ void strip_store(const float2 (&nx)[2], const float2 (&ny)[2], const float2 (&nz)[2],
                                             const float2 (&q)[2], const bool (&k)[4], unsigned char* np, uint8_t* mp,
@@ -324,7 +316,7 @@ __device__ __forceinline__ void strip_store(const float2 (&nx)[2], const float2 
       __stcs(mp + i, (uint8_t)(mbits >> (8 * i)));
     }
   } else {
-    store_row<OUT>(w, mbits, np, mp, n, buf, f);
+    store_row<OUT>(w, mbits, np, mp, buf, f);
   }
 }
 
@@ -557,18 +549,18 @@ __device__ __forceinline__ void strip_pipeline(const BatchArgs& args, const Glob
           write_tables<TY>(reinterpret_cast<float4*>(st + SB - TB + kStripInfoBytes), *fd, gx0, gy0);
         }
       } else {
-      if (lane == 0) {
-        if (RING && cur != fenced) {
-          fence_tensormap_acquire(&fd->tmap);
-          fenced = cur;
+        if (lane == 0) {
+          if (RING && cur != fenced) {
+            fence_tensormap_acquire(&fd->tmap);
+            fenced = cur;
+          }
+          const int padx = pad_x(HALO, eb);
+          const uint32_t bar = smem_u32(&full[s]);
+          mbar_arrive_expect_tx(bar, (uint32_t)((kStripX + 2 * padx) * (TY + 2 * HALO) * eb));
+          tma_load_2d(smem_u32(st), &fd->tmap, gx0 - padx, gy0 - HALO, bar);
+          write_record<BPP>(reinterpret_cast<StripInfo*>(st + SB - TB), *fd, g.sign, gx0, gy0);
         }
-        const int padx = pad_x(HALO, eb);
-        const uint32_t bar = smem_u32(&full[s]);
-        mbar_arrive_expect_tx(bar, (uint32_t)((kStripX + 2 * padx) * (TY + 2 * HALO) * eb));
-        tma_load_2d(smem_u32(st), &fd->tmap, gx0 - padx, gy0 - HALO, bar);
-        write_record<BPP>(reinterpret_cast<StripInfo*>(st + SB - TB), *fd, g.sign, gx0, gy0);
-      }
-      write_tables<TY>(reinterpret_cast<float4*>(st + SB - TB + kStripInfoBytes), *fd, gx0, gy0);
+        write_tables<TY>(reinterpret_cast<float4*>(st + SB - TB + kStripInfoBytes), *fd, gx0, gy0);
       }
       __syncwarp();
       if (lane == 0) mbar_arrive(smem_u32(&full[s]));

@@ -117,7 +117,7 @@ void pack_param_batch(void* dst, const BatchHeader& hdr, const int* tile_begin, 
 
 // Strip kernels (nrm_forward_strip.cu): the batched forward pass, alpha <=
 // kStripMaxAlpha, of frames whose rows TMA can load and whose outputs take
-// whole-vector stores (aligned; see strip_frame in nrm_api.cpp), or of any
+// whole-vector stores (aligned; see strip_aligned in nrm_api.cpp), or of any
 // frames. Descriptors are those of the persistent kernels for tile kStripX x
 // strip_tile_y(out_dtype, aligned). param_block: a ParamBatch packed by
 // pack_param_batch, or NULL for the device block in args. u16: every frame is
