@@ -1087,14 +1087,22 @@ void fill_work_list(const BatchPart& p, FrameDesc* fd, nrm::BatchHeader* hdr, in
   tile_begin[p.n] = acc;
 }
 
-// The 128-byte aligned parameter block of one part's launch, in scratch memory.
-void* pack_part(std::vector<int>& tb, std::vector<unsigned char>& raw, const BatchPart& p, FrameDesc* fd) {
+// One part's parameter block into pb (128-byte aligned, param_batch_bytes()); tb: room
+// for its tile offsets.
+void pack_part(int* tb, void* pb, const BatchPart& p, FrameDesc* fd) {
+  nrm::BatchHeader hdr;
+  fill_work_list(p, fd, &hdr, tb);
+  nrm::pack_param_batch(pb, hdr, tb, fd + p.first, p.n);
+}
+
+// The same in the handle's scratch memory.
+void* pack_scratch(nrm_handle* h, const BatchPart& p, FrameDesc* fd) {
+  std::vector<int>& tb = h->scratch_tb;
+  std::vector<unsigned char>& raw = h->scratch_param;
   if (tb.size() < (size_t)p.n + 1) tb.resize((size_t)p.n + 1);
   if (raw.size() < nrm::param_batch_bytes() + 128) raw.resize(nrm::param_batch_bytes() + 128);
   void* pb = raw.data() + (128 - reinterpret_cast<uintptr_t>(raw.data()) % 128) % 128;
-  nrm::BatchHeader hdr;
-  fill_work_list(p, fd, &hdr, tb.data());
-  nrm::pack_param_batch(pb, hdr, tb.data(), fd + p.first, p.n);
+  pack_part(tb.data(), pb, p, fd);
   return pb;
 }
 
@@ -1130,8 +1138,8 @@ int launch_part(nrm_handle* h, bool aligned, const nrm::BatchArgs& args, const B
 }  // namespace
 
 // From this size on one frame takes the strip kernels, as a batch of one whose
-// descriptors travel in the parameter block (built in memory of the calling
-// thread, so that several threads may use one handle's single-frame call). Below it
+// descriptors travel in the parameter block (built on the stack: this call allocates
+// nothing, and several threads may use one handle's single-frame call). Below it
 // the plain launch stays: its host side is 3 us shorter, which a caller that makes
 // its tensors per call would see (1280x720: plain 5.8-6.6 us, strip 7.3; 1920x1080:
 // GPU time 12.4 against 10.4, but 13.3 with the views made per call). Plain / strip
@@ -1151,15 +1159,16 @@ static bool single_takes_strip(const nrm_handle* h, const nrm_frame& f, BatchPla
 }
 
 static int estimate_single_strip(nrm_handle* h, const nrm_frame& f, const BatchPlan& plan, void* cuda_stream) {
-  static thread_local std::vector<int> tb;
-  static thread_local std::vector<unsigned char> raw;
+  alignas(128) unsigned char pb[nrm::kParamBlockMaxBytes];
+  int tb[2];
+  if (nrm::param_batch_bytes() > sizeof(pb)) return fail(NRM_ERR_UNSUPPORTED, "parameter block too large");
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   FrameDesc d[1];
   BatchPart part[2];
   split_batch(h, &f, 1, plan, d, part);
   for (int k = 0; k < 2; ++k) {
     if (part[k].tiles == 0) continue;
-    void* pb = pack_part(tb, raw, part[k], d);
+    pack_part(tb, pb, part[k], d);
     const nrm::BatchArgs ring = {};
     NRM_CHECK(launch_part(h, k == 0, ring, part[k], pb, st));
   }
@@ -1246,7 +1255,7 @@ static int estimate_batched_param(nrm_handle* h, const nrm_frame* frames, int n,
   }
   for (int k = 0; k < 2; ++k) {
     if (part[k].tiles == 0) continue;
-    void* pb = pack_part(h->scratch_tb, h->scratch_param, part[k], fd.data());
+    void* pb = pack_scratch(h, part[k], fd.data());
     nrm::BatchArgs ring;
     std::memset(&ring, 0, sizeof(ring));
     NRM_CHECK(launch_part(h, k == 0, ring, part[k], pb, st));
@@ -1835,7 +1844,7 @@ int nrm_estimate_batched_multiscale(nrm_handle* h, const nrm_frame* frames, int 
     p.n = std::min(part[0].n - first, nrm::kParamMaxFrames);
     p.tiles = 0;
     for (int i = 0; i < p.n; ++i) p.tiles += fd[first + i].tiles_x * ((fd[first + i].H + p.tile_y - 1) / p.tile_y);
-    void* pb = pack_part(h->scratch_tb, h->scratch_param, p, fd);
+    void* pb = pack_scratch(h, p, fd);
     NRM_CUDA(nrm::launch_multiscale_strip(ms, g, h->p.out_dtype, scales->form, p.tiles, p.u16, st, pb),
              "launch fwd_ms_strip_kernel");
   }
@@ -1855,7 +1864,7 @@ int nrm_estimate_batched_multiscale(nrm_handle* h, const nrm_frame* frames, int 
       args.tile_begin = reinterpret_cast<const int*>(dbase + nrm::kTileBeginOffset);
       args.frames = reinterpret_cast<const FrameDesc*>(dbase + nrm::frames_offset(sp->capacity)) + rest.first;
     } else {
-      pb = pack_part(h->scratch_tb, h->scratch_param, rest, fd);
+      pb = pack_scratch(h, rest, fd);
     }
     const cudaError_t e = nrm::launch_multiscale_batched(args, ms, g, h->p.out_dtype, scales->form, rest.tiles,
                                                          rest.u16, st, pb);

@@ -85,6 +85,7 @@ struct Globals {
 // Frames per capture-safe batched launch, whose descriptor block travels as
 // one kernel parameter (under the 32,764-byte parameter limit).
 constexpr int kParamMaxFrames = 100;
+constexpr size_t kParamBlockMaxBytes = 32764;
 
 struct BatchArgs {
   const BatchHeader* hdr;

@@ -9,6 +9,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <new>
 #include <string>
 #include <vector>
 
@@ -22,6 +23,7 @@ int g_fail_at = -1;     // the launch that fails (0 = the next), or none
 int g_timing = 0;       // elapsed-time queries answered so far
 int g_fastest = -1;     // the query that gets the shortest time
 int g_event_syncs = 0;
+bool g_no_memory = false;  // allocations fail
 
 cudaError_t launched(const std::string& line) {
   if (g_fail_at == 0) {
@@ -29,7 +31,10 @@ cudaError_t launched(const std::string& line) {
     return cudaErrorLaunchFailure;
   }
   if (g_fail_at > 0) --g_fail_at;
+  const bool none = g_no_memory;  // (the log itself may grow)
+  g_no_memory = false;
   g_log += line + "\n";
+  g_no_memory = none;
   return cudaSuccess;
 }
 
@@ -59,6 +64,14 @@ const char* kernel_name(const void* fn) {
 
 }  // namespace
 
+void* operator new(size_t n) {
+  void* p = g_no_memory ? nullptr : malloc(n ? n : 1);
+  if (!p) throw std::bad_alloc();
+  return p;
+}
+void operator delete(void* p) noexcept { free(p); }
+void operator delete(void* p, size_t) noexcept { free(p); }
+
 #define FAKE extern "C" __attribute__((visibility("default")))
 
 FAKE const char* fake_log() { return g_log.c_str(); }
@@ -74,6 +87,7 @@ FAKE void fake_capture(int on) { g_capture = on; }
 FAKE void fake_fail_launch(int k) { g_fail_at = k; }
 FAKE void fake_fastest(int k) { g_fastest = k; }
 FAKE int fake_timings() { return g_timing; }
+FAKE void fake_no_memory(int on) { g_no_memory = on != 0; }
 FAKE int fake_event_syncs() { return g_event_syncs; }
 
 extern "C" {
