@@ -57,7 +57,8 @@ KERNEL_SOURCES = ("paper_2209_08241_gb300/csrc/nrm_forward.cu", "paper_2209_0824
                   "paper_2209_08241_gb300/csrc/nrm_forward_kernels.cuh", "paper_2209_08241_gb300/csrc/nrm_device.cuh",
                   "paper_2209_08241_gb300/csrc/nrm_forward_vec.cuh",
                   "paper_2209_08241_gb300/csrc/nrm_forward_strip.cuh",
-                  "paper_2209_08241_gb300/csrc/nrm_forward_strip.cu")
+                  "paper_2209_08241_gb300/csrc/nrm_forward_strip.cu",
+                  "paper_2209_08241_gb300/csrc/nrm_forward_strip_any.cu")
 
 # DRAM bytes per launch of the batched kernel from ncu (dram__bytes_read.sum +
 # dram__bytes_write.sum) on the 64 x 1080p uint16 workload, valid only while

@@ -145,7 +145,9 @@ NRM_API int nrm_create(const nrm_intrinsics* K, int H, int W, const nrm_params* 
 /* Releases the handle and its device state. Waits for its pending work. */
 NRM_API void nrm_destroy(nrm_handle* h);
 
-/* Single frame, one plain launch (one CTA per tile, TMA-staged halo tiles).
+/* Single frame, one launch: one CTA per tile, or from three million pixels on
+ * (half4 output of frames that TMA cannot load: five) the kernels of a batched
+ * call with this frame alone, where those are the faster ones; the same bits.
  * depth: H x W (dense, pitch W) of the handle's in_dtype; normals: H x W x 4
  * (dense) of the handle's out_dtype; valid: H x W bytes (dense).
  * Sizes: H and W up to 2^24 (NRM_ERR_UNSUPPORTED above). A frame with more
@@ -160,18 +162,20 @@ NRM_API int nrm_estimate(nrm_handle* h, const void* depth, void* normals, uint8_
 NRM_API int nrm_estimate_points(nrm_handle* h, const void* depth, void* normals, uint8_t* valid, float* points,
                                 void* cuda_stream);
 
-/* n frames of any sizes, intrinsics and input dtypes in ONE persistent launch
- * over a (frame, tile) work list. The handle's alpha, mask mode, tau,
+/* n frames of any sizes, intrinsics and input dtypes in one persistent launch
+ * over a (frame, tile) work list, or in two where frames that take different
+ * kernels are mixed and each part is worth a launch. The handle's alpha, mask mode, tau,
  * depth_scale, out_dtype and orientation apply to all frames. n = 0 is a
  * no-op. The frames' buffers must not overlap.
  * Up to 100 frames without point buffers: the frame records and their TMA
  * tensor maps travel as one kernel parameter (no descriptor upload, no
- * tensor-map fences). Larger batches, or batches with point buffers: a CUDA
- * graph per descriptor slot (upload node, then the kernel node), replayed
- * from a ring of slots. Either way the host may return before the GPU has
+ * tensor-map fences). Larger batches: one upload into a ring of descriptor
+ * slots, then the launches. Batches with point buffers, and larger batches of
+ * handles with an explicit geometry or alpha > 4: a CUDA graph per descriptor
+ * slot (upload node, then the kernel node). In every case the host may return before the GPU has
  * started; it blocks only when every slot of the ring is still in use.
  * Stream capture: while cuda_stream is being captured (any capture mode), the
- * call records a single kernel node with the parameter form and no events or
+ * call records one or two kernel nodes with the parameter form and no events or
  * host synchronisation, so the captured graph can be replayed freely while
  * the frames' buffers stay valid; then n is at most 100 and frames may not
  * carry point buffers (NRM_ERR_UNSUPPORTED). The handle must have been
@@ -185,7 +189,7 @@ NRM_API int nrm_estimate_batched(nrm_handle* h, const nrm_frame* frames, int n, 
  * g = grad_normals, H x W x 4 float32 (the 4th component is ignored).
  * valid: the mask nrm_estimate produced for this depth (a pixel it marks valid
  * must have a positive finite five-point stencil; other masks give undefined
- * gradients). Deterministic (gather, no atomics).
+ * gradients). Deterministic (no atomics).
  * Returns NRM_ERR_UNSUPPORTED for a uint16 handle. A frame with more than 65535
  * tile rows runs as a one-frame nrm_backward_batched call (same results). */
 NRM_API int nrm_backward(nrm_handle* h, const void* depth, const float* grad_normals,
@@ -253,8 +257,10 @@ NRM_API int nrm_spherical(const float* normals, const uint8_t* valid, int H, int
 /* Mean squared error of the angle images (Section 4, Tables 2-5) between an
  * estimate and a reference normal map, over the pixels valid in both, with
  * plain differences of the [0, 2 pi) values. out: 3 doubles in device memory,
- * {MSE of I_theta, MSE of I_phi, number of pixels}. Deterministic: a fixed
- * reduction order, no atomics. Uses scratch owned by the handle (allocated on
+ * {MSE of I_theta, MSE of I_phi, number of pixels}. Deterministic: every sum in a
+ * fixed order (an atomic counter only tells the last block that it is the last).
+ * A bounded wait that ran out is reported by nrm_sync_status (NRM_ERR_TIMEOUT).
+ * Uses scratch owned by the handle (allocated on
  * the first call); calls on one handle must not overlap on the GPU. */
 NRM_API int nrm_angle_mse(nrm_handle* h, const float* normals, const uint8_t* valid, const float* ref_normals,
                           const uint8_t* ref_valid, int H, int W, long long pitch, double* out, void* cuda_stream);
@@ -301,13 +307,15 @@ NRM_API int nrm_estimate_multiscale(nrm_handle* h, const void* depth, void* norm
 NRM_API int nrm_estimate_batched_host(nrm_handle* h, const nrm_frame* frames, int n, void* cuda_stream);
 
 /* nrm_estimate_multiscale for n frames of any sizes, dtypes and intrinsics in
- * one persistent launch (the batched pipeline of nrm_estimate_batched, tile
- * 128 x 16, 256 compute threads). Frames as for nrm_estimate_batched; their
+ * one persistent launch (the batched pipeline of nrm_estimate_batched). Distances
+ * 1..K (K = 2..6) have kernels of their own, for frames with widths and output
+ * pitches in fours and aligned buffers, in batches large enough for them (100
+ * frames a launch, other frames in one more). Frames as for nrm_estimate_batched; their
  * points must be NULL (NRM_ERR_UNSUPPORTED otherwise). The per-scale constants
  * are formed on the GPU from each frame's intrinsics, so results can differ
  * from nrm_estimate_multiscale's in the last bits. n = 0 is a no-op. Up to 100
  * frames the descriptors travel as one kernel parameter, and while the stream
- * is being captured the call records a single kernel node (then n <= 100). */
+ * is being captured the call records one or two kernel nodes (then n <= 100). */
 NRM_API int nrm_estimate_batched_multiscale(nrm_handle* h, const nrm_frame* frames, int n, const nrm_scales* scales,
                                             void* cuda_stream);
 
@@ -326,7 +334,7 @@ NRM_API int nrm_estimate_batched_multiscale(nrm_handle* h, const nrm_frame* fram
  * Device pointers, asynchronous on the stream. radius in 1..NRM_MAX_PLANE_RADIUS,
  * else NRM_ERR_UNSUPPORTED. FP32 arithmetic on coordinates taken relative to the
  * window's centre point; the eigenproblem by cyclic Jacobi rotations. One CTA
- * per 32 x 8 tile: H above 65535 x 8 rows is NRM_ERR_UNSUPPORTED. */
+ * per 32 x 8 or 64 x 8 tile: H above 65535 x 8 rows is NRM_ERR_UNSUPPORTED. */
 #define NRM_MAX_PLANE_RADIUS 4
 NRM_API int nrm_plane_fit(nrm_handle* h, const void* depth, float* normals, uint8_t* valid, int radius,
                           void* cuda_stream);
@@ -362,9 +370,10 @@ NRM_API int nrm_sync_status(nrm_handle* h);
  * (64,32,256), (64,64,256). threads counts the compute threads; the persistent
  * kernel adds one producer warp. stages in {2, 3, 4} (persistent kernel only);
  * ctas_per_sm 0 = as many as fit. With the default geometry (128, 16, 256, 3, 0)
- * batched calls without point buffers use, for alpha <= 4 and frames whose
- * width is a multiple of 4 and whose buffers are aligned (as a dense allocation
- * is), kernels with tile shapes of their own; results are the same bits. */
+ * calls without point buffers may use, for alpha <= 4, kernels with tile shapes of
+ * their own (one for frames whose widths and output pitches are multiples of 4 and
+ * whose buffers are aligned, as a dense allocation is, one for any frame); the
+ * results are the same bits. */
 typedef struct {
   int tile_x, tile_y, threads, stages, ctas_per_sm;
 } nrm_tile_config;

@@ -2,10 +2,10 @@
 //
 // Responsibilities: argument validation (nothing is launched on bad input),
 // per-frame descriptors with the Eq. 4-6 constants and TMA tensor maps, the
-// plain per-frame launch, the batched persistent launch replayed from a CUDA
-// graph (descriptor upload node -> [event] -> kernel node -> [event]) over a
-// ring of descriptor slots, the adjoint launch, kernel timing, the device
-// status word and the autotuner with its JSON cache.
+// plain per-frame launch, the batched launches (which kernels take which frames,
+// descriptors as a kernel parameter, uploaded into a ring of slots or by a CUDA
+// graph per slot), the adjoint launch, kernel timing, the device status word and
+// the autotuner with its JSON cache.
 #include <cuda.h>
 #include <cuda_runtime.h>
 #include <unistd.h>
@@ -1232,7 +1232,7 @@ int nrm_estimate_points(nrm_handle* h, const void* depth, void* normals, uint8_t
 // (frame records and tensor maps in parameter space): no descriptor upload and
 // no tensor-map fences. Used for batches of at most kParamMaxFrames frames
 // without point buffers, and always while cuda_stream is being captured, when
-// the launch is recorded as a single kernel node with no ring slot, events or
+// the launch is recorded as one or two kernel nodes with no ring slot, events or
 // synchronisation. Frames were validated by the caller.
 static int estimate_batched_param(nrm_handle* h, const nrm_frame* frames, int n, cudaStream_t st, bool capture) {
   if (n > nrm::kParamMaxFrames)

@@ -15,9 +15,10 @@
 //           (98 %)  [10 warps, 4 stages 222 / 292; 8 x 8, 3 stages 221 / 294]
 // The tiled kernel in its default geometry (128x16, 256 threads) takes 441,
 // 348 and 1283 us on the float4, half4 and mixed batches.
-// The octahedral output is bound by instruction issue (about 40 instructions a
-// pixel), so as many warps as fit run: 4 warps x 8 rows, 192 us (71 %; tiled
-// 341 us); float32 input with 2 stages, 4 CTAs, 198 us (3 stages, 3 CTAs: 205).
+// The octahedral output is bound by instruction issue (37.5 warp instructions per 32
+// pixels, issue slots 65 % busy), so as many warps as fit run: 4 warps x 8 rows, 192 us
+// (71 %; tiled 341 us); float32 input with 2 stages, 4 CTAs, 198 us (3 stages, 3 CTAs:
+// 205).
 // Batches of few tiles take all the CTAs that fit: there the ramp counts, not the
 // steady state (16 x 640x480 float32: 18.8 us with 3 CTAs per SM, 20.9 with one;
 // 2 x 1080p 15.2 against 16.0, 4 x 1080p 30.7 against 29.6 us).
@@ -25,10 +26,11 @@
 // Frames of any alignment (loader warps instead of TMA; nothing comes near
 // saturating HBM): as many CTAs as fit, 6 compute and 4 loader warps (octahedral
 // 4 and 2). 64 x 1921x1081: uint16 -> float4 487 us (76 %; the tiled kernel's plain
-// loads 1092), float32 -> float4 503 (1181), uint16 -> half4 484 (818), octahedral
-// 381 (789); two 3001x2001 uint16 frames 44 us (75). [6 loader warps 521 / 520 /
-// 539; 4 compute warps, 3 CTAs 488 / 504 / 515; 12 and 16 compute warps, 1 CTA 650 /
-// 685 / 566.]
+// loads 1080), float32 -> float4 503 (1160), uint16 -> half4 485 (812), octahedral
+// 439 (831); two 3001x2001 uint16 frames 44 us (75). [float4 from uint16 and float32,
+// half4: 6 loader warps 521 / 520 / 539; 4 compute warps, 3 CTAs 488 / 504 / 515; 12
+// and 16 compute warps, 1 CTA 650 / 685 / 566.] Which calls take which kernel:
+// forward_plan in nrm_api.cpp.
 #include <algorithm>
 #include <atomic>
 

@@ -13,8 +13,9 @@
 // turn from registers; only the left and right neighbours are read a second
 // time. No decoded copy of the tile is kept in shared memory and no barrier
 // joins the warps of a CTA: a warp waits for its stage's TMA copy and frees the
-// stage when it is done with it. Thread instructions per pixel (uint16 input,
-// alpha 2): half4 33 (the tiled kernel's vector loop: 51), octahedral 40 (50).
+// stage when it is done with it. Warp instructions per 32 pixels (uint16 input,
+// alpha 2): float4 37.7, half4 36.8, octahedral 37.5 (the tiled kernel's vector loops
+// about 50 a pixel).
 //
 // Invalid depths are found per pixel from the smallest of the five depths
 // (three-operand minimum, NaN propagating) instead of coding each of them as
@@ -168,8 +169,8 @@ __device__ __forceinline__ void strip_codes(float2 nx, float2 ny, float2 nz, uin
 // per pixel straight from the lanes, 4 pixels apart, writes part of a 32-byte
 // sector at a time: 64 x 1921x1081 uint16 -> float4 745 us, half4 755 us with one
 // CTA per SM; through the buffer 646 and 492 us, with two CTAs 487 and 484. The
-// octahedral codes, whose ragged ends would be three of four elements, are faster
-// straight from the lanes: 381 against 581 us, and have no buffer.) float4: units
+// octahedral codes, whose ragged ends would be three of four elements, go straight
+// from the lanes, 439 us; through a buffer they took half as long again.) float4: units
 // are pixels, stored with their index's low bits XORed by bits 3-5, so that neither
 // side has bank conflicts.
 constexpr int kRowBufMask = 160;  // the mask's part of a row buffer

@@ -277,7 +277,9 @@ cudaError_t launch_backward_batched_param(const FrameDesc* frames, const BwdMaps
                                           const float* scale = nullptr);
 
 // Evaluation kernels (nrm_eval.cu).
-constexpr int kMseBlocks = 456;  // fixed, so that the reduction order never changes; three per SM of the GB300
+// Fixed, so that the reduction order never changes; three per SM, one wave, on the GB300's
+// 152 SMs (more waves on fewer SMs).
+constexpr int kMseBlocks = 456;
 cudaError_t launch_spherical(const float* normals, const uint8_t* valid, int H, int W, long long pitch, float* phi,
                              float* theta, cudaStream_t stream);
 // partials: 3 kMseBlocks doubles of device scratch; ticket: a zeroed device word,

@@ -7,7 +7,8 @@
 // decoded rows the vertical neighbours come from stay in registers (fully
 // unrolled, so a row is converted once for all scales), and the horizontal ones
 // come from one decoded window of the row, 4 (K <= 4) or 8 columns to the left and
-// right. With the distances compiled in, a scale costs its 8 (pair) or 10
+// right. (Each K is twelve kernels, unrolled over rows and scales. 7 and 8 scales are
+// not compiled and not measured here; they take the run-time kernel.) With the distances compiled in, a scale costs its 8 (pair) or 10
 // (quad) paired FP32 instructions per two pixels and no loads or indexing.
 //
 // Every operation on valid pixels is that of ms_compute (nrm_multiscale.cu) in its
