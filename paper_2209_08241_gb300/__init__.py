@@ -10,7 +10,7 @@ machine without the built library or a GPU every call raises.
     normals, mask = est(depth)              # depth: (H, W) float32 or uint16 CUDA tensor
 
     batch = BatchedEstimator(alpha=2)
-    outs = batch([(depth0, K0), (depth1, K1), ...])    # one persistent launch
+    outs = batch([(depth0, K0), (depth1, K1), ...])    # one persistent launch (or two)
 
     n = estimate_normals(depth, K)          # differentiable (float32 depth)
 """
@@ -368,7 +368,7 @@ def _frame(depth: torch.Tensor, K, normals: torch.Tensor, valid: torch.Tensor,
 
 class BatchedEstimator(_Handle):
     """Any number of frames of any sizes, intrinsics and input dtypes per call,
-    processed by one persistent launch replayed from a CUDA graph."""
+    processed by one persistent launch (or two, where kinds of frames that take different kernels are mixed)."""
 
     def __init__(self, params: NormalParams | None = None, device=None, **kw):
         params = params or NormalParams(**kw)

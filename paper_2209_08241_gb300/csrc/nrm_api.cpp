@@ -905,8 +905,8 @@ bool tma_rows(const nrm_frame& f) {
 // and depth rows that TMA can address.
 bool strip_aligned(const nrm_handle* h, const nrm_frame& f, const BatchPlan& plan) {
   const uintptr_t na = h->p.out_dtype == NRM_OUT_OCT16 ? 16 : 32;
-  return strip_domain(h, f, plan) && f.W % 4 == 0 && f.out_pitch % 4 == 0 && (uintptr_t)f.normals % na == 0 &&
-         (uintptr_t)f.valid % 4 == 0 && tma_rows(f);
+  return f.W % 4 == 0 && f.out_pitch % 4 == 0 && (uintptr_t)f.normals % na == 0 && (uintptr_t)f.valid % 4 == 0 &&
+         tma_rows(f) && strip_domain(h, f, plan);
 }
 
 // Descriptors of the n frames into fd: the aligned ones from the front, the
@@ -1005,6 +1005,11 @@ BatchPlan forward_plan(const nrm_handle* h, const nrm_frame* frames, int n) {
                     h->cfg.tile_x,
                     h->cfg.tile_y};
   if (!strip_handle(h)) return plan;
+  plan.strip = true;
+  int i0 = 0;  // (most batches end here: with 256 frames of 64x48 the sums below cost 1 us of 28)
+  while (i0 < n && ((long long)frames[i0].H * frames[i0].W == 0 || strip_aligned(h, frames[i0], plan))) ++i0;
+  if (i0 == n) return plan;
+  plan.strip = false;
   bool any_ok = true;
   double strip = 0, any[2] = {0, 0}, tiled[2] = {0, 0};  // us beyond the ramps: aligned frames, the rest
   int count[2] = {0, 0};
@@ -1024,10 +1029,6 @@ BatchPlan forward_plan(const nrm_handle* h, const nrm_frame* frames, int n) {
     any[k] += mpx * (aligned ? c.any.aligned : tma ? c.any.ragged : c.any.plain);
     tiled[k] += mpx * (aligned ? c.tiled.aligned : tma ? c.tiled.ragged : c.tiled.plain);
     plain_loads = plain_loads || !tma;
-  }
-  if (count[1] == 0) {
-    plan.strip = true;
-    return plan;
   }
   const double tiled_ramp = c.tiled.ramp + (plain_loads ? 0.6 : 0.0);
   const double split = count[0] ? c.strip.ramp + strip + kSecondLaunch : INFINITY;  // the aligned part of two launches
