@@ -1056,8 +1056,9 @@ BatchPlan forward_plan(const nrm_handle* h, const nrm_frame* frames, int n) {
 // 6.6 / 7.3, 8.2 / 8.8; four 640x480, 160 tiles, 9.1 / 9.9, quad of 6 from float32
 // 11.8 / 10.7; sixteen 19.8 / 26.7, 27.9 / 35.5), and more in a batch with other
 // frames, where it is a second launch (7 of 640x480 and one of 641x481, 280 tiles, pair
-// of 2 scales 15.0 / 14.2; one of 1920x1080 and one of 1921x1081 19.2 / 18.1) or, past
-// the parameter block's frames, several.
+// of 2 scales 15.0 / 14.2; one of 1920x1080 and one of 1921x1081 19.2 / 18.1; four and
+// four, 1020 tiles, pair of 2 scales 87.1 / 83.8, of 4 75 / 86) or, past the parameter
+// block's frames, several.
 bool ms_strip_pays(const nrm_handle* h, const nrm_frame* frames, int n, const BatchPlan& plan) {
   long long tiles = 0;
   bool rest = false;
@@ -1069,8 +1070,9 @@ bool ms_strip_pays(const nrm_handle* h, const nrm_frame* frames, int n, const Ba
     else
       rest = true;
   }
-  const bool wide = plan.q == 4.0 && plan.scales >= 5;  // four directions, five scales and more
-  return 3 * tiles >= (long long)h->sm_count * (rest || n > nrm::kParamMaxFrames ? 8 : wide ? 6 : 2);
+  const bool quad = plan.q == 4.0;
+  const int several = !quad && plan.scales == 2 ? 30 : 8, alone = quad && plan.scales >= 5 ? 6 : 2;
+  return 3 * tiles >= (long long)h->sm_count * (rest || n > nrm::kParamMaxFrames ? several : alone);
 }
 
 // One part's header and tile offsets (tile_begin: n + 1 entries).

@@ -44,6 +44,9 @@ def test_mixed_batches(capture, other):
     for batch in ([aligned(), other()], [aligned()] * 7 + [other()], [aligned()] + [other()] * 7,
                   [aligned(1920, 1080), other()]):
         assert launches(batch, range(1, 5), "pair", capture=capture) == [("ms_tiled", len(batch))]
+    batch = [aligned(1920, 1080)] * 4 + [other(1921, 1081)] * 4
+    assert launches(batch, (1, 2), "pair", capture=capture) == [("ms_tiled", 8)]
+    assert launches(batch, (1, 2), "quad", capture=capture) == [("ms_strip", 4), ("ms_tiled", 4)]
     batch = [aligned(1920, 1080)] * 7 + [other()]
     assert launches(batch, range(1, 5), "quad", capture=capture) == [("ms_strip", 7), ("ms_tiled", 1)]
 
