@@ -115,14 +115,19 @@ __device__ __forceinline__ void persistent_pipeline(const BatchArgs& args, const
     if (threadIdx.x != NT) return;
     int cur = 0;      // frame cursor: this CTA's tiles increase monotonically
     int fenced = -1;  // last tensor map fenced
+    // Waits (bounded) for the copies of the last tiles before the j-th, the only ones
+    // that can be under way, so that none lands after the CTA has ended, also when the
+    // compute threads gave a late one up.
+    auto land = [&](int j) {
+      for (int k = j > S ? j - S : 0; k < j; ++k)
+        mbar_wait_bounded(smem_u32(&full[k % S]), (uint32_t)((k / S) & 1), g.timeout_ns);
+    };
     for (int j = 0; j < my; ++j) {
       const int s = j % S;
       if (j >= S &&
           !mbar_wait_bounded(smem_u32(&empty[s]), (uint32_t)(((j / S) - 1) & 1), g.timeout_ns)) {
         record_error(g.status, NRM_ERR_TIMEOUT);
-        // Let every copy this warp issued land before the CTA can exit.
-        for (int k = j - S; k < j; ++k)
-          mbar_wait_bounded(smem_u32(&full[k % S]), (uint32_t)((k / S) & 1), g.timeout_ns);
+        land(j);
         return;
       }
       const int t = (int)blockIdx.x + j * G;
@@ -155,6 +160,7 @@ __device__ __forceinline__ void persistent_pipeline(const BatchArgs& args, const
         mbar_arrive(bar);  // plain-load tile: the compute threads read global memory themselves
       }
     }
+    land(my);
     return;
   }
 

@@ -521,13 +521,18 @@ __device__ __forceinline__ void strip_pipeline(const BatchArgs& args, const Glob
     // ------------------------------------------------------------ producer
     int cur = 0, fenced = -1, s = 0;
     uint32_t parity = 1;
+    // Waits (bounded) for the copies of the last tiles before the j-th, the only ones
+    // that can be under way, so that none lands after the CTA has ended, also when a
+    // compute warp gave a late one up.
+    auto land = [&](int j) {
+      if (LOADERS == 0 && lane == 0)
+        for (int k = j > S ? j - S : 0; k < j; ++k)
+          mbar_wait_bounded(smem_u32(&full[k % S]), (uint32_t)((k / S) & 1), g.timeout_ns);
+    };
     for (int j = 0; j < my; ++j) {
       if (j >= S && !mbar_wait_warp(smem_u32(&empty[s]), parity, g.timeout_ns)) {
-        if (lane == 0) {
-          record_error(g.status, NRM_ERR_TIMEOUT);
-          for (int k = j - S; k < j; ++k)
-            mbar_wait_bounded(smem_u32(&full[k % S]), (uint32_t)((k / S) & 1), g.timeout_ns);
-        }
+        if (lane == 0) record_error(g.status, NRM_ERR_TIMEOUT);
+        land(j);
         return;
       }
       const int t = (int)blockIdx.x + j * G;
@@ -570,6 +575,7 @@ __device__ __forceinline__ void strip_pipeline(const BatchArgs& args, const Glob
         parity ^= 1;
       }
     }
+    land(my);
     return;
   }
 
